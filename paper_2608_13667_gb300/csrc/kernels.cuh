@@ -106,7 +106,8 @@ struct AttnParams {
   int32_t hold_loads;      // test hook (ST_FLAG_HOLD_LOADS): the loader issues nothing
   int32_t item_base;       // decode: CTA x reads item item_base + x
   int32_t keep_l2;         // decode: the launch's pages fit in L2; load them evict-normal so they stay
-  const MergeItem* mitems; // batched merge: CTA x takes mitems[x] (slot, L0, T above unused)
+  const MergeItem* mitems; // batched merge: cluster x takes mitems[x] (slot, L0, T above unused)
+  int32_t kv_split;        // merge: CTAs (a cluster) that share one row tile's keys
   // decode step (items flagged kItemAppend): the rows the step appends,
   // [L][n_br][Hkv][D], and the pools they go to
   const __nv_bfloat16* app_k;
@@ -178,6 +179,26 @@ cudaError_t launch_chained(void (*kernel)(KArgs...), dim3 grid, dim3 block, size
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<Args&&>(args)...);
 }
 
+// The same with clusters of `cluster` CTAs in x (1: none).
+template <typename... KArgs, typename... Args>
+cudaError_t launch_chained_cluster(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
+                                   int cluster, Args&&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = cluster;
+  attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = cluster > 1 ? 2 : 1;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<Args&&>(args)...);
+}
+
 cudaError_t launch_table_update(int32_t* table, const TableRun* runs, const int32_t* values,
                                 int n_runs, cudaStream_t s);
 cudaError_t launch_append(const AppendParams& p, const InlineAppendPlan* inl, int D, cudaStream_t s);
@@ -188,9 +209,10 @@ cudaError_t launch_decode_tc(const CUtensorMap& kmap, const CUtensorMap& vmap, c
                              const InlineDecodePlan* inl, int n_items, int D, bool wide, cudaStream_t s);
 // Causal merge prefill on tcgen05, two 128-row query tiles per CTA sharing
 // K/V (merge_tc.cu): one sequence (p.slot, p.L0, p.T; p.mitems null) or a
-// batch of n_items work items (p.mitems), p.q -> p.out_o, p.out_lse.
-cudaError_t launch_merge_tc(const CUtensorMap& kmap, const CUtensorMap& vmap, const AttnParams& p, int n_items,
-                            int D, cudaStream_t s);
+// batch of n_items work items (p.mitems, and the same items on the host),
+// p.q -> p.out_o, p.out_lse.
+cudaError_t launch_merge_tc(const CUtensorMap& kmap, const CUtensorMap& vmap, const AttnParams& p,
+                            const MergeItem* host_items, int n_items, int D, cudaStream_t s);
 // Decode partials of fork groups of 129 to 256 stacked rows on the same
 // paired tile (one CTA per item x KV head x layer, items from p.item_base on,
 // launched as a programmatic dependent like the other decode kernels).

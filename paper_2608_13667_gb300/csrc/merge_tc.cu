@@ -1,5 +1,6 @@
 // Merge prefill on the tcgen05 tensor cores: two 128-row query tiles per CTA
-// that share every K/V stage (one CTA per SM).
+// that share every K/V stage (one CTA per SM), the stages of a row tile split
+// over a cluster of CTAs where a launch has few row tiles.
 //
 // Section 3.5 of the paper: the harvested thoughts are appended after main's
 // context and read in order, so thought row i of a merge of T rows attends
@@ -11,6 +12,19 @@
 // new rows in one launch) gives each CTA its own (sequence, L0, T, row tile)
 // through a work list.
 //
+// Few rows.  A turn's thoughts are a few dozen rows onto a long context: in
+// one layer that is a row tile or three per KV head, 8 to 24 CTAs on 152 SMs,
+// each walking the whole context alone.  Two things split that walk:
+//   - a cluster of up to 16 CTAs shares a row tile, each taking a range of its
+//     stages; the partial results meet in distributed shared memory (no
+//     workspace, no second launch).  launch_merge_t picks the size.
+//   - a tile of at most 128 rows leaves tile B without rows: then both tiles
+//     hold the same rows, A takes the even stages and B the odd ones ("dual"),
+//     so the tensor cores do no work for padding and a stage costs half.
+// One layer, 32/8 heads, D 128, a context of 23040: 16 rows 350 -> 38 us, 44
+// rows 353 -> 50, 133 rows 363 -> 93, 512 rows 363 -> 197; 88 rows onto 8192
+// 140 -> 42 us.
+//
 // CTA layout (352 threads, one CTA per SM, all 512 TMEM columns):
 //   warps 0..3  softmax of tile A, warps 4..7 softmax of tile B: thread r of
 //               a tile owns its row r = TMEM lane r (warp w reads lanes
@@ -20,7 +34,9 @@
 //               only when a score exceeds it by more than 2^8 (O in TMEM is
 //               then rescaled in place), and writes P = 2^(s - m) as two bf16
 //               terms (P_hi + P_lo, exact to about 16 bits) into TMEM over its
-//               own scores.  At the end it normalises O.
+//               own scores.  At the end it writes O to shared memory, and the
+//               warps put rows together from there, from every CTA of the
+//               cluster and both tiles where those share the row.
 //   warp 8      K loader, warp 9 V loader: page ids from the block table (32
 //               per read, one batch ahead), one 2 KiB TMA copy per (page,
 //               64-wide half of D) into separate K and V rings.
@@ -58,6 +74,8 @@
 // stale shared or pool memory cannot turn 0 * x into NaN in a real row.
 #include <math.h>
 
+#include <algorithm>
+#include <mutex>
 #include <type_traits>
 
 #include "kernels.cuh"
@@ -83,6 +101,25 @@ __device__ __forceinline__ float fmax3(float a, float b, float c) {
   asm("max.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
   return d;
 }
+
+// CTAs of a cluster that share one row tile's keys in a merge, at most (16 is
+// the largest cluster of this part).
+constexpr int kMaxMergeSplit = 16;
+// Stages of 128 keys that a part of a split row tile has, at least.
+constexpr int kMinPartStages = 4;
+
+// Parts that a row tile of `all_tiles` stages is split into in a launch of
+// clusters of `cluster` CTAs.  It depends on the tile alone where the cluster
+// is large enough.
+__host__ __device__ constexpr int merge_parts(int all_tiles, int cluster) {
+  const int most = all_tiles / kMinPartStages;
+  return most < 1 ? 1 : most < cluster ? most : cluster;
+}
+
+struct MergeSplitCost {
+  int parts;
+  float total, longest;  // of its CTAs together, of one of them
+};
 
 template <int D>
 struct PairCfg {
@@ -127,19 +164,20 @@ __global__ void __launch_bounds__(kThreads, 1)
   const int layer = blockIdx.z;
   const int G = p.G;
 
-  // Decode: launched as a programmatic dependent of the kernel before it in
-  // the stream; the tensor-memory allocation touches no global memory, every
+  // Launched as a programmatic dependent of the kernel before it in the
+  // stream; the tensor-memory allocation touches no global memory, every
   // global access comes after the wait.
-  if constexpr (kDecode) {
-    if (warp == kMmaWarp) tmem_alloc(tmem_slot, kTmemCols);
-    griddep_wait();
-    griddep_launch_dependents();
-  }
+  if (warp == kMmaWarp) tmem_alloc(tmem_slot, kTmemCols);
+  griddep_wait();
+  griddep_launch_dependents();
   // one merge: its row tiles, the last ones (most keys) first; a batch: one
-  // work item per CTA (the host orders those longest first); a decode: one
+  // work item per cluster (the host orders those longest first); a decode: one
   // run of pages of a fork group (at most 256 stacked rows) per CTA, every
   // row over all of the run's keys
-  int slot = p.slot, L0 = p.L0, T = p.T, q_row0 = 0, row_base = (gridDim.x - 1 - blockIdx.x) * 2 * kTileRows;
+  const int cluster = kDecode ? 1 : p.kv_split;  // CTAs that share a row tile
+  const int rank = kDecode ? 0 : (int)blockIdx.x % cluster;
+  int slot = p.slot, L0 = p.L0, T = p.T, q_row0 = 0;
+  int row_base = ((int)gridDim.x / cluster - 1 - (int)blockIdx.x / cluster) * 2 * kTileRows;
   int page_begin = 0, n_rows, n_pages, n_valid_keys;
   AttnItem item{};
   const int32_t* members = nullptr;
@@ -154,7 +192,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     n_valid_keys = item.n_tokens;
   } else {
     if (p.mitems) {
-      const MergeItem mi = p.mitems[blockIdx.x];
+      const MergeItem mi = p.mitems[blockIdx.x / cluster];
       slot = mi.slot;
       L0 = mi.L0;
       T = mi.T;
@@ -166,7 +204,25 @@ __global__ void __launch_bounds__(kThreads, 1)
     n_pages = (L0 + t_last + 1 + kPageTokens - 1) / kPageTokens;
     n_valid_keys = L0 + T;
   }
-  const int n_tiles = (n_pages + kPagesPerStage - 1) / kPagesPerStage;
+  // this CTA's part of the row tile's stages (all of them without a split)
+  const int all_tiles = (n_pages + kPagesPerStage - 1) / kPagesPerStage;
+  const int n_parts = kDecode ? 1 : merge_parts(all_tiles, cluster);
+  if (rank >= n_parts) {  // a tile with fewer parts than the launch's clusters: nothing left for this CTA
+    __syncthreads();
+    if (warp == kMmaWarp) tmem_dealloc(*tmem_slot, kTmemCols);
+    if (n_parts > 1) {  // the barriers of the exchange below count every CTA of the cluster
+      cluster_sync();
+      cluster_sync();
+    }
+    return;
+  }
+  const int j0 = rank * all_tiles / n_parts, j1 = (rank + 1) * all_tiles / n_parts;
+  const int n_tiles = j1 - j0;
+  const int key_base = j0 * kKeys;
+  page_begin += j0 * kPagesPerStage;
+  n_pages = min(n_pages - j0 * kPagesPerStage, n_tiles * kPagesPerStage);
+  // at most 128 rows: both tiles hold them, tile A takes the even stages and tile B the odd ones
+  const bool dual = !kDecode && n_rows <= kTileRows;
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < kKS; ++s) {
@@ -186,15 +242,14 @@ __global__ void __launch_bounds__(kThreads, 1)
     mbar_init(q_ready, kSoftThreads);
     fence_mbar_init();
   }
-  if (!kDecode && warp == kMmaWarp) tmem_alloc(tmem_slot, kTmemCols);
   tc_fence_before_sync();
   __syncthreads();
   tc_fence_after_sync();
   const uint32_t tmem = *tmem_slot;
 
   // ---- loaders -------------------------------------------------------------------
-  if (warp == kKLoadWarp || warp == kVLoadWarp) {
-    if (p.hold_loads) return;  // test hook: nothing arrives, the other roles' waits run out
+  // (hold_loads, a test hook: nothing arrives, the other roles' waits run out)
+  if ((warp == kKLoadWarp || warp == kVLoadWarp) && !p.hold_loads) {
     const bool is_k = warp == kKLoadWarp;
     const CUtensorMap* map = is_k ? &kmap : &vmap;
     uint64_t* full = is_k ? k_full : v_full;
@@ -251,7 +306,6 @@ __global__ void __launch_bounds__(kThreads, 1)
       atomicCAS(p.status, 0, kDevTimeout);
       for (int t = max(0, j - n_st); t < j; ++t) mbar_wait(&full[t % n_st], (t / n_st) & 1);
     }
-    return;
   }
 
   // ---- MMA issuer ----------------------------------------------------------------
@@ -271,14 +325,11 @@ __global__ void __launch_bounds__(kThreads, 1)
       const uint64_t v_desc0 = tc_desc_sw128(smem_addr(base + C::kVOff), C::kKVHalfBytes, 1024);
       bool ok = __all_sync(0xffffffffu, mbar_wait(q_ready, 0));
       tc_fence_after_sync();
-      // O_t += P_t(i) V_i, P_t(i) read from TMEM over S_t(i); each half of P
+      // O_t += P_t(i) V, P_t(i) read from TMEM over S_t(i); each half of P
       // (64 keys) is published on its own, so the first half's MMAs run while
       // the softmax finishes the second
-      auto issue_pv = [&](auto tile, int i) -> bool {
+      auto issue_pv = [&](auto tile, int i, uint64_t vd) -> bool {
         constexpr int t = decltype(tile)::value;
-        const int s = i % kVS;
-        if (t == 0 && !__all_sync(0xffffffffu, mbar_wait(&v_full[s], (i / kVS) & 1))) return false;
-        const uint64_t vd = v_desc0 + (uint64_t)((s * C::kSlotBytes) >> 4);
         const uint32_t acc0 = i > 0 ? 1u : 0u;
 #pragma unroll
         for (int hf = 0; hf < 2; ++hf) {
@@ -294,44 +345,71 @@ __global__ void __launch_bounds__(kThreads, 1)
                                1u);                                                     // P_lo
           }
         }
-        if (t == 1) tc_commit_elect(&v_empty[s]);
         return true;
       };
-      // S_t(j) = Q_t K_j^T
-      auto issue_s = [&](auto tile, uint64_t kd) {
+      // S_t(i) = Q_t K^T
+      auto issue_s = [&](auto tile, uint64_t qd, uint64_t kd) {
         constexpr int t = decltype(tile)::value;
 #pragma unroll
         for (int h = 0; h < C::kHalves; ++h)
 #pragma unroll
           for (int kk = 0; kk < 4; ++kk)
-            tc_mma_bf16_elect(tmem + t * kTmemTile,
-                        q_desc + (uint64_t)((t * C::kQTileBytes + h * C::kQHalfBytes + kk * 32) >> 4),
-                        kd + (uint64_t)((h * C::kKVHalfBytes + kk * 32) >> 4), idesc_s, (h | kk) != 0);
+            tc_mma_bf16_elect(tmem + t * kTmemTile, qd + (uint64_t)((h * C::kQHalfBytes + kk * 32) >> 4),
+                              kd + (uint64_t)((h * C::kKVHalfBytes + kk * 32) >> 4), idesc_s, (h | kk) != 0);
         tc_commit_elect(&s_full[t]);
       };
       const std::integral_constant<int, 0> tile_a;
       const std::integral_constant<int, 1> tile_b;
-      for (int j = 0; ok && j < n_tiles; ++j) {
-        const int s = j % kKS;
-        const uint64_t kd = k_desc0 + (uint64_t)((s * C::kSlotBytes) >> 4);
-        if (j > 0 && !issue_pv(tile_a, j - 1)) {
-          ok = false;
-          break;
+      const uint64_t qd_b = q_desc + (uint64_t)(C::kQTileBytes >> 4);
+      if (!dual) {
+        // iteration i of both tiles is stage i
+        auto pv = [&](auto tile, int i) -> bool {
+          constexpr int t = decltype(tile)::value;
+          const int s = i % kVS;
+          if (t == 0 && !__all_sync(0xffffffffu, mbar_wait(&v_full[s], (i / kVS) & 1))) return false;
+          if (!issue_pv(tile, i, v_desc0 + (uint64_t)((s * C::kSlotBytes) >> 4))) return false;
+          if (t == 1) tc_commit_elect(&v_empty[s]);
+          return true;
+        };
+        for (int i = 0; ok && i < n_tiles; ++i) {
+          const int s = i % kKS;
+          const uint64_t kd = k_desc0 + (uint64_t)((s * C::kSlotBytes) >> 4);
+          ok = (i == 0 || pv(tile_a, i - 1)) && __all_sync(0xffffffffu, mbar_wait(&k_full[s], (i / kKS) & 1));
+          if (!ok) break;
+          tc_fence_after_sync();
+          issue_s(tile_a, q_desc, kd);
+          if (i > 0 && !pv(tile_b, i - 1)) {
+            ok = false;
+            break;
+          }
+          issue_s(tile_b, qd_b, kd);
+          tc_commit_elect(&k_empty[s]);
         }
-        if (!__all_sync(0xffffffffu, mbar_wait(&k_full[s], (j / kKS) & 1))) {
-          ok = false;
-          break;
-        }
-        tc_fence_after_sync();
-        issue_s(tile_a, kd);
-        if (j > 0 && !issue_pv(tile_b, j - 1)) {
-          ok = false;
-          break;
-        }
-        issue_s(tile_b, kd);
-        tc_commit_elect(&k_empty[s]);
+        if (ok && n_tiles > 0) ok = pv(tile_a, n_tiles - 1) && pv(tile_b, n_tiles - 1);
+      } else {
+        // iteration i of tile t is stage 2 i + t, its own K and V slot; of an
+        // odd number of stages B has one fewer
+        auto pv = [&](auto tile, int i) -> bool {
+          const int j = 2 * i + decltype(tile)::value, s = j % kVS;
+          if (!__all_sync(0xffffffffu, mbar_wait(&v_full[s], (j / kVS) & 1))) return false;
+          if (!issue_pv(tile, i, v_desc0 + (uint64_t)((s * C::kSlotBytes) >> 4))) return false;
+          tc_commit_elect(&v_empty[s]);
+          return true;
+        };
+        auto qk = [&](auto tile, int i) -> bool {
+          const int j = 2 * i + decltype(tile)::value, s = j % kKS;
+          if (!__all_sync(0xffffffffu, mbar_wait(&k_full[s], (j / kKS) & 1))) return false;
+          tc_fence_after_sync();
+          issue_s(tile, q_desc, k_desc0 + (uint64_t)((s * C::kSlotBytes) >> 4));
+          tc_commit_elect(&k_empty[s]);
+          return true;
+        };
+        const int n_a = (n_tiles + 1) / 2, n_b = n_tiles / 2;
+        for (int i = 0; ok && i < n_a; ++i)
+          ok = (i == 0 || pv(tile_a, i - 1)) && qk(tile_a, i) && (i == 0 || pv(tile_b, i - 1)) &&
+               (i >= n_b || qk(tile_b, i));
+        if (ok && n_a > 0) ok = pv(tile_a, n_a - 1) && (n_b < n_a || pv(tile_b, n_b - 1));
       }
-      if (ok && n_tiles > 0) ok = issue_pv(tile_a, n_tiles - 1) && issue_pv(tile_b, n_tiles - 1);
       tc_commit_elect(o_final);
       if (!ok && lane == 0) atomicCAS(p.status, 0, kDevTimeout);
     }
@@ -339,209 +417,411 @@ __global__ void __launch_bounds__(kThreads, 1)
     named_barrier_sync(1, kSoftThreads + 32);
     tc_fence_after_sync();
     tmem_dealloc(tmem, kTmemCols);
-    return;
   }
 
   // ---- softmax warps ---------------------------------------------------------------
-  const int t = warp >> 2;               // tile
+  const int t = warp >> 2;               // tile (of a softmax warp)
   const int r = (warp & 3) * 32 + lane;  // row within the tile = TMEM lane
-  const int tid = threadIdx.x & (kTileRows - 1);
-  const uint32_t t_lane = tmem + ((uint32_t)((warp & 3) * 32) << 16) + t * kTmemTile;
-  const int tile_row0 = row_base + t * kTileRows;
-  const bool valid = t * kTileRows + r < n_rows;
+  const int tile_row0 = row_base + (dual ? 0 : t * kTileRows);
+  const bool valid = warp < kKLoadWarp && tile_row0 - row_base + r < n_rows;
   int qrow = 0, head = 0;
   if (valid) {
     const int gr = tile_row0 + r;
     qrow = kDecode ? members[item.member_base + gr / G] : gr / G;
     head = kvh * G + gr % G;
   }
-  // causal limit of this row (a decode row sees the whole run)
-  const int limit = kDecode ? n_valid_keys : valid ? L0 + qrow + 1 : n_valid_keys;
-  const int min_limit = kDecode ? n_valid_keys : L0 + tile_row0 / G + 1;  // the tile's first row sees the fewest keys
   const int64_t io_row = (int64_t)layer * p.n_rows_q + q_row0 + qrow;  // this row in Q / O / LSE
-  {
-    const uint4* src = reinterpret_cast<const uint4*>(p.q + (io_row * p.Hq + head) * D);
-    uint8_t* q_s = base + C::kQOff + t * C::kQTileBytes;
-#pragma unroll
-    for (int c = 0; c < D / 8; ++c) {
-      const uint4 v = valid ? src[c] : make_uint4(0u, 0u, 0u, 0u);
-      *reinterpret_cast<uint4*>(q_s + (c >> 3) * C::kQHalfBytes + r * 128 + (((c & 7) ^ (r & 7)) << 4)) = v;
-    }
-    fence_proxy_async_smem();
-  }
-  mbar_arrive(q_ready);
+  // Results on their way out, over the K, V and Q buffers once every MMA has
+  // completed: xo [2 tiles][128 rows][D/4] float4 of the unnormalised O (xo_at:
+  // columns swizzled by the row, so that a warp reads or writes a column of 32
+  // rows and a row of 32 columns without bank conflicts); xml [2 tiles][128
+  // rows], a row's max and sum; and of the rows that this CTA puts together, at
+  // most 256 / parts of them from as many sources: xw and xwt, the sources'
+  // maxima, sums and weights, and xrow, their places in the output.
+  constexpr int kQuads = D / 4;
+  float4* xo = reinterpret_cast<float4*>(base + C::kKOff);
+  float2* xml = reinterpret_cast<float2*>(base + C::kQOff);
+  float2* xw = xml + 2 * kTileRows;
+  float* xwt = reinterpret_cast<float*>(xw + 4 * kTileRows);
+  int64_t* xrow = reinterpret_cast<int64_t*>(xw + 8 * kTileRows);
+  auto xo_at = [&](int tile, int row, int c) { return (tile * kTileRows + row) * kQuads + (c ^ (row & (kQuads - 1))); };
+  const int64_t in_row = io_row * p.Hq + head;
+  static_assert(2 * kTileRows * D * 4 <= C::kBarOff - C::kKOff, "the exchange fits the K and V rings");
 
-  const float sl2 = p.scale_log2;
-  float m_used = -1e30f, l = 0.f;
   bool ok = true;
-  for (int j = 0; j < n_tiles; ++j) {
-    if (!__all_sync(0xffffffffu, mbar_wait(&s_full[t], j & 1))) {
-      ok = false;
-      break;
-    }
-    tc_fence_after_sync();
-    const int key0 = j * kKeys;
-    const int loaded = min(kPagesPerStage, n_pages - j * kPagesPerStage) * kPageTokens;
-    const bool edge = key0 + kKeys > min_limit || loaded < kKeys;
-    // scores of keys [hf * 64, hf * 64 + 64), masked past the stage's pages and
-    // past this row's causal limit
-    auto load_half = [&](int hf, float* sc) {
-      tmem_ld64(t_lane + hf * 64, sc);
-      if (edge) {
+  if (warp < kKLoadWarp) {
+    const int tid = threadIdx.x & (kTileRows - 1);
+    const uint32_t t_lane = tmem + ((uint32_t)((warp & 3) * 32) << 16) + t * kTmemTile;
+    // causal limit of this row (a decode row sees the whole run)
+    const int limit = kDecode ? n_valid_keys : valid ? L0 + qrow + 1 : n_valid_keys;
+    const int min_limit = kDecode ? n_valid_keys : L0 + tile_row0 / G + 1;  // the tile's first row sees the fewest keys
+    if (!dual || t == 0) {
+      const uint4* src = reinterpret_cast<const uint4*>(p.q + in_row * D);
+      uint8_t* q_s = base + C::kQOff + t * C::kQTileBytes;
 #pragma unroll
-        for (int c = 0; c < 64; ++c)
-          if (hf * 64 + c >= loaded || key0 + hf * 64 + c >= limit) sc[c] = -INFINITY;
-      }
-    };
-    // row max over both halves: independent chains of three-input max
-    float mx;
-    {
-      float mx8[8];
-#pragma unroll
-      for (int i = 0; i < 8; ++i) mx8[i] = -INFINITY;
-#pragma unroll 1  // one half's scores live at a time
-      for (int hf = 0; hf < 2; ++hf) {
-        float sc[64];
-        load_half(hf, sc);
-#pragma unroll
-        for (int c = 0; c < 64; c += 16)
-#pragma unroll
-          for (int i = 0; i < 8; ++i) mx8[i] = fmax3(mx8[i], sc[c + i], sc[c + 8 + i]);
-      }
-      mx = fmax3(fmax3(mx8[0], mx8[1], mx8[2]), fmax3(mx8[3], mx8[4], mx8[5]), fmaxf(mx8[6], mx8[7]));
-    }
-    const float m_new = fmaxf(m_used, mx * sl2);  // sl2 > 0: max commutes with the scale
-    const bool need = valid && m_new > m_used + kRescaleThreshold;
-    if (__any_sync(0xffffffffu, need)) {
-      const float alpha = need ? ex2(m_used - m_new) : 1.f;
-      if (j > 0) {
-        // O_t += P_t(j-1) V_{j-1} has completed (covered by the commit of S_t(j))
-#pragma unroll 1
-        for (int k = 0; k < D / 32; ++k) {
-          float o[32];
-          tmem_ld32(t_lane + kTmemO + k * 32, o);
-#pragma unroll
-          for (int i = 0; i < 32; ++i) o[i] *= alpha;
-          tmem_st32(t_lane + kTmemO + k * 32, o);
-        }
-      }
-      l *= alpha;
-      if (need) m_used = m_new;
-    }
-    if (t == 0 && (key0 + kKeys > n_valid_keys || loaded < kKeys)) {
-      // zero the V rows of keys that are not valid once the stage's copies
-      // have landed; both tiles' P V are issued after this tile's first P half
-      const int s = j % kVS;
-      if (!__all_sync(0xffffffffu, mbar_wait(&v_full[s], (j / kVS) & 1))) {
-        ok = false;
-        break;
-      }
-      uint8_t* vslot = base + C::kVOff + s * C::kSlotBytes;
-      for (int x = tid; x < kKeys * C::kHalves; x += kTileRows) {
-        const int c = x % kKeys, h = x / kKeys;
-        if (c >= loaded || key0 + c >= n_valid_keys) {
-#pragma unroll
-          for (int y = 0; y < 8; ++y)
-            *reinterpret_cast<uint4*>(vslot + h * C::kKVHalfBytes + c * 128 + y * 16) = make_uint4(0u, 0u, 0u, 0u);
-        }
+      for (int c = 0; c < D / 8; ++c) {
+        const uint4 v = valid ? src[c] : make_uint4(0u, 0u, 0u, 0u);
+        *reinterpret_cast<uint4*>(q_s + (c >> 3) * C::kQHalfBytes + r * 128 + (((c & 7) ^ (r & 7)) << 4)) = v;
       }
       fence_proxy_async_smem();
     }
-    // P = 2^(s sl2 - m) (two keys per packed f32x2 FMA / add) as two bf16
-    // terms, P_hi = bf16(P) and P_lo = bf16(P - P_hi), so that P V is exact to
-    // about 16 bits whatever the spread of the scores.  The 16 score columns
-    // of keys [16 ks, 16 ks + 16) take P_hi of those keys (8 columns of bf16
-    // pairs) and then P_lo (8 columns): each store overwrites only scores
-    // already read.
-    {
-      const float2 scale2 = make_float2(sl2, sl2), neg_m2 = make_float2(-m_used, -m_used);
-      float2 rs[4] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
-#pragma unroll 1
-      for (int hf = 0; hf < 2; ++hf) {
-        float sc[64];
-        load_half(hf, sc);
+    mbar_arrive(q_ready);
+
+    const float sl2 = p.scale_log2;
+    float m_used = -1e30f, l = 0.f;
+    const int n_it = dual ? (n_tiles + 1 - t) / 2 : n_tiles;
+    for (int it = 0; it < n_it; ++it) {
+      const int j = dual ? 2 * it + t : it;  // the stage
+      if (!__all_sync(0xffffffffu, mbar_wait(&s_full[t], it & 1))) {
+        ok = false;
+        break;
+      }
+      tc_fence_after_sync();
+      const int key0 = key_base + j * kKeys;
+      const int loaded = min(kPagesPerStage, n_pages - j * kPagesPerStage) * kPageTokens;
+      const bool edge = key0 + kKeys > min_limit || loaded < kKeys;
+      const int n_seen = min(loaded, limit - key0);  // this row's keys of the stage
+      // scores of keys [hf * 64, hf * 64 + 64), masked past the stage's pages and
+      // past this row's causal limit
+      auto load_half = [&](int hf, float* sc) {
+        tmem_ld64(t_lane + hf * 64, sc);
+        if (edge) {
 #pragma unroll
-        for (int kq = 0; kq < 4; ++kq) {  // 16 keys per step
-          uint32_t pk[16];
-#pragma unroll
-          for (int c = 0; c < 16; c += 2) {
-            const float2 x = __ffma2_rn(make_float2(sc[kq * 16 + c], sc[kq * 16 + c + 1]), scale2, neg_m2);
-            const float a = ex2(x.x), b = ex2(x.y);
-            rs[(c >> 1) & 3] = __fadd2_rn(rs[(c >> 1) & 3], make_float2(a, b));
-            const uint32_t hi = pack_bf16(a, b);
-            pk[c / 2] = hi;
-            pk[8 + c / 2] = pack_bf16(a - __uint_as_float(hi << 16), b - __uint_as_float(hi & 0xffff0000u));
-          }
-          tmem_st16u_nowait(t_lane + (hf * 4 + kq) * 16, pk);
+          for (int c = 0; c < 64; ++c)
+            if (c >= n_seen - hf * 64) sc[c] = -INFINITY;
         }
-        tmem_wait_st();
-        tc_fence_before_sync();
-        mbar_arrive(&p_full[2 * t + hf]);
-      }
-      const float2 s = __fadd2_rn(__fadd2_rn(rs[0], rs[1]), __fadd2_rn(rs[2], rs[3]));
-      l += s.x + s.y;
-    }
-  }
-  if (ok) ok = __all_sync(0xffffffffu, mbar_wait(o_final, 0));
-  tc_fence_after_sync();
-  if (ok) {
-    const float inv = 1.f / l;
-    // merge: the row's O and LSE; decode: its split-KV partial
-    const int64_t out_idx = kDecode ? (io_row * p.Hq + head) * p.max_splits + item.split : io_row * p.Hq + head;
-    float* dst = valid ? p.out_o + out_idx * D : nullptr;
-#pragma unroll 1
-    for (int k = 0; k < D / 32; ++k) {
-      float o[32];
-      tmem_ld32(t_lane + kTmemO + k * 32, o);
-      if (dst) {
+      };
+      // row max over both halves: independent chains of three-input max
+      float mx;
+      {
+        float mx8[8];
 #pragma unroll
-        for (int i = 0; i < 32; i += 4)
-          *reinterpret_cast<float4*>(dst + k * 32 + i) =
-              make_float4(o[i] * inv, o[i + 1] * inv, o[i + 2] * inv, o[i + 3] * inv);
+        for (int i = 0; i < 8; ++i) mx8[i] = -INFINITY;
+#pragma unroll 1  // one half's scores live at a time
+        for (int hf = 0; hf < 2; ++hf) {
+          float sc[64];
+          load_half(hf, sc);
+#pragma unroll
+          for (int c = 0; c < 64; c += 16)
+#pragma unroll
+            for (int i = 0; i < 8; ++i) mx8[i] = fmax3(mx8[i], sc[c + i], sc[c + 8 + i]);
+        }
+        mx = fmax3(fmax3(mx8[0], mx8[1], mx8[2]), fmax3(mx8[3], mx8[4], mx8[5]), fmaxf(mx8[6], mx8[7]));
+      }
+      const float m_new = fmaxf(m_used, mx * sl2);  // sl2 > 0: max commutes with the scale
+      const bool need = valid && m_new > m_used + kRescaleThreshold;
+      if (__any_sync(0xffffffffu, need)) {
+        const float alpha = need ? ex2(m_used - m_new) : 1.f;
+        if (it > 0) {
+          // the O_t += P_t V before has completed (covered by the commit of this S_t)
+#pragma unroll 1
+          for (int k = 0; k < D / 32; ++k) {
+            float o[32];
+            tmem_ld32(t_lane + kTmemO + k * 32, o);
+#pragma unroll
+            for (int i = 0; i < 32; ++i) o[i] *= alpha;
+            tmem_st32(t_lane + kTmemO + k * 32, o);
+          }
+        }
+        l *= alpha;
+        if (need) m_used = m_new;
+      }
+      if ((t == 0 || dual) && (key0 + kKeys > n_valid_keys || loaded < kKeys)) {
+        // zero the V rows of keys that are not valid once the stage's copies
+        // have landed; the P V that read the stage are issued after this tile's
+        // first P half
+        const int s = j % kVS;
+        if (!__all_sync(0xffffffffu, mbar_wait(&v_full[s], (j / kVS) & 1))) {
+          ok = false;
+          break;
+        }
+        uint8_t* vslot = base + C::kVOff + s * C::kSlotBytes;
+        for (int x = tid; x < kKeys * C::kHalves; x += kTileRows) {
+          const int c = x % kKeys, h = x / kKeys;
+          if (c >= loaded || key0 + c >= n_valid_keys) {
+#pragma unroll
+            for (int y = 0; y < 8; ++y)
+              *reinterpret_cast<uint4*>(vslot + h * C::kKVHalfBytes + c * 128 + y * 16) = make_uint4(0u, 0u, 0u, 0u);
+          }
+        }
+        fence_proxy_async_smem();
+      }
+      // P = 2^(s sl2 - m) (two keys per packed f32x2 FMA / add) as two bf16
+      // terms, P_hi = bf16(P) and P_lo = bf16(P - P_hi), so that P V is exact to
+      // about 16 bits whatever the spread of the scores.  The 16 score columns
+      // of keys [16 ks, 16 ks + 16) take P_hi of those keys (8 columns of bf16
+      // pairs) and then P_lo (8 columns): each store overwrites only scores
+      // already read.
+      {
+        const float2 scale2 = make_float2(sl2, sl2), neg_m2 = make_float2(-m_used, -m_used);
+        float2 rs[4] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+#pragma unroll 1
+        for (int hf = 0; hf < 2; ++hf) {
+          float sc[64];
+          load_half(hf, sc);
+#pragma unroll
+          for (int kq = 0; kq < 4; ++kq) {  // 16 keys per step
+            uint32_t pk[16];
+#pragma unroll
+            for (int c = 0; c < 16; c += 2) {
+              const float2 x = __ffma2_rn(make_float2(sc[kq * 16 + c], sc[kq * 16 + c + 1]), scale2, neg_m2);
+              const float a = ex2(x.x), b = ex2(x.y);
+              rs[(c >> 1) & 3] = __fadd2_rn(rs[(c >> 1) & 3], make_float2(a, b));
+              const uint32_t hi = pack_bf16(a, b);
+              pk[c / 2] = hi;
+              pk[8 + c / 2] = pack_bf16(a - __uint_as_float(hi << 16), b - __uint_as_float(hi & 0xffff0000u));
+            }
+            tmem_st16u_nowait(t_lane + (hf * 4 + kq) * 16, pk);
+          }
+          tmem_wait_st();
+          tc_fence_before_sync();
+          mbar_arrive(&p_full[2 * t + hf]);
+        }
+        const float2 s = __fadd2_rn(__fadd2_rn(rs[0], rs[1]), __fadd2_rn(rs[2], rs[3]));
+        l += s.x + s.y;
       }
     }
-    if (valid) p.out_lse[out_idx] = (m_used + log2f(l)) * kLn2;
-  } else if (lane == 0) {
-    atomicCAS(p.status, 0, kDevTimeout);
+    if (ok) ok = __all_sync(0xffffffffu, mbar_wait(o_final, 0));
+    tc_fence_after_sync();
+    if (!ok && lane == 0) atomicCAS(p.status, 0, kDevTimeout);
+    const bool some = ok && n_it > 0;
+    if (some) {
+#pragma unroll 1
+      for (int k = 0; k < D / 32; ++k) {
+        float o[32];
+        tmem_ld32(t_lane + kTmemO + k * 32, o);
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+          xo[xo_at(t, r, k * 8 + i)] = make_float4(o[4 * i], o[4 * i + 1], o[4 * i + 2], o[4 * i + 3]);
+      }
+    }
+    xml[t * kTileRows + r] = make_float2(m_used, some ? l : 0.f);
+    tc_fence_before_sync();
+    named_barrier_sync(1, kSoftThreads + 32);
   }
-  tc_fence_before_sync();
-  named_barrier_sync(1, kSoftThreads + 32);
+
+  // ---- results ---------------------------------------------------------------------
+  // A row's sources are the CTAs of its cluster, and in each both tiles when
+  // they share their rows: O = sum 2^(m_s - m) O_s / sum 2^(m_s - m) l_s.  The
+  // rows are dealt out to the CTAs, and D/4 lanes put together a row: every
+  // read of a source's row, through distributed shared memory, and every write
+  // of O are D contiguous values (a thread writing its own row touches 32 rows
+  // per store: 5.6 us for a CTA's 256 rows, against 3 this way).  A source without a key
+  // for the row has l = 0, and its O was perhaps never written.
+  // This code runs once per CTA, so its time is mostly that of fetching its
+  // instructions: loops are kept rolled (a version with 16 loads in flight
+  // took 12 us where the same work rolled took 5).
+  if (n_parts > 1) cluster_sync();  // (one part: the barrier above has ordered the exchange)
+  if (warp < kKLoadWarp) {
+    const int per_cta = dual ? 2 : 1, n_src = n_parts * per_cta;
+    const int x0 = rank * n_rows / n_parts, n_own = (rank + 1) * n_rows / n_parts - x0;  // this CTA's rows: x0 + [0, n_own)
+    // source s of row x: CTA s (tile x / 128), or tile s & 1 of CTA s >> 1
+    auto src_cta = [&](int s) { return (uint32_t)(dual ? s >> 1 : s); };
+    auto src_tile = [&](int s, int x) { return dual ? s & 1 : x >> 7; };
+    const int n_pairs = n_own * n_src;
+#pragma unroll 1
+    for (int i = threadIdx.x; i < n_pairs; i += kSoftThreads) {
+      const int x = x0 + i / n_src, s = i % n_src;
+      xw[i] = ld_cluster_f2(smem_addr(xml + src_tile(s, x) * kTileRows + (x & (kTileRows - 1))), src_cta(s));
+    }
+    named_barrier_sync(2, kSoftThreads);
+    // each pair's weight, 2^(m_s - m) / sum 2^(m_s - m) l_s
+#pragma unroll 1
+    for (int i = threadIdx.x; i < n_pairs; i += kSoftThreads) {
+      const int k = i / n_src;
+      const float2* ml = xw + k * n_src;
+      float m = -1e30f, l = 0.f;
+#pragma unroll 1
+      for (int s = 0; s < n_src; ++s) {
+        const float2 x = ml[s];
+        if (x.y == 0.f) continue;
+        const float m_new = fmaxf(m, x.x);
+        l = l * ex2(m - m_new) + x.y * ex2(x.x - m_new);
+        m = m_new;
+      }
+      const float2 mine = xw[i];
+      xwt[i] = (mine.y != 0.f ? ex2(mine.x - m) : 0.f) / l;  // (NaN for a row without any weight)
+      if (i == k * n_src) {
+        const int gr = row_base + x0 + k;
+        const int row = kDecode ? members[item.member_base + gr / G] : q_row0 + gr / G;
+        int64_t out_row = ((int64_t)layer * p.n_rows_q + row) * p.Hq + kvh * G + gr % G;
+        if constexpr (kDecode) out_row = out_row * p.max_splits + item.split;  // a split-KV partial
+        xrow[k] = out_row;
+        if (ok) p.out_lse[out_row] = (m + log2f(l)) * kLn2;
+      }
+    }
+    named_barrier_sync(2, kSoftThreads);
+    // the pairs of a warp's rows one after another, a few loads in flight
+    constexpr int kRows = 32 / kQuads < 1 ? 1 : 32 / kQuads, kStep = kRows * (kSoftThreads / 32), kBatch = 4;
+    const int c = lane % kQuads;
+    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+    int k = warp * kRows + lane / kQuads, s = 0;  // the next pair to load: row x0 + k, source s
+#pragma unroll 1
+    while (k < n_own) {
+      float4 v[kBatch];
+      float w[kBatch];
+      int done[kBatch];  // the row that the pair completes, or -1
+#pragma unroll
+      for (int u = 0; u < kBatch; ++u) {
+        w[u] = 0.f;
+        v[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+        done[u] = -1;
+        if (k < n_own) {
+          w[u] = xwt[k * n_src + s];
+          if (w[u] != 0.f)
+            v[u] = ld_cluster_f4(smem_addr(xo + xo_at(src_tile(s, x0 + k), (x0 + k) & (kTileRows - 1), c)), src_cta(s));
+          if (++s == n_src) {
+            done[u] = k;
+            s = 0;
+            k += kStep;
+          }
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < kBatch; ++u) {
+        acc.x += w[u] * v[u].x;
+        acc.y += w[u] * v[u].y;
+        acc.z += w[u] * v[u].z;
+        acc.w += w[u] * v[u].w;
+        if (done[u] >= 0) {
+          if (ok) reinterpret_cast<float4*>(p.out_o + xrow[done[u]] * D)[c] = acc;
+          acc = make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+      }
+    }
+  }
+  if (n_parts > 1) cluster_sync();  // a CTA's buffers stay until its peers have read them
 }
 
+// Per device: the shared-memory opt-in, and how many CTAs of clusters of n are
+// resident at once (a cluster sits inside one GPC, so the SMs that a size
+// leaves over stay idle; 0: the size is not available).
+struct PairSetup {
+  bool done = false;
+  int resident[kMaxMergeSplit + 1] = {};
+};
+
 template <int D, bool kDecode>
-cudaError_t launch_pair_t(const CUtensorMap& km, const CUtensorMap& vm, const AttnParams& p,
-                          const InlineDecodePlan& inl, int n_ctas, cudaStream_t s) {
+cudaError_t pair_setup(const PairSetup** out) {
   using C = PairCfg<D>;
-  // the shared-memory opt-in is a per-device function attribute
-  static bool configured[64] = {};
+  static PairSetup setups[64];
+  static std::mutex mu;
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
-  if (!configured[dev]) {
-    e = cudaFuncSetAttribute(merge_pair_kernel<D, kDecode>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             C::kSmemBytes);
+  PairSetup& ps = setups[dev];
+  std::lock_guard<std::mutex> lock(mu);
+  if (!ps.done) {
+    auto* kernel = merge_pair_kernel<D, kDecode>;
+    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmemBytes);
     if (e != cudaSuccess) return e;
-    configured[dev] = true;
+    if constexpr (!kDecode) {
+      e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+      if (e != cudaSuccess) return e;
+      for (int n = 1; n <= kMaxMergeSplit; ++n) {
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(n);
+        cfg.blockDim = dim3(kThreads);
+        cfg.dynamicSmemBytes = C::kSmemBytes;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = n;
+        attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        int clusters = 0;
+        if (cudaOccupancyMaxActiveClusters(&clusters, kernel, &cfg) != cudaSuccess) {
+          cudaGetLastError();  // a size this part does not offer
+          clusters = 0;
+        }
+        ps.resident[n] = clusters * n;
+      }
+      if (ps.resident[1] < 1) return cudaErrorInvalidConfiguration;
+    }
+    ps.done = true;
   }
-  dim3 grid(n_ctas, p.Hkv, p.L);
-  if constexpr (kDecode)
-    return launch_chained(merge_pair_kernel<D, true>, grid, dim3(kThreads), C::kSmemBytes, s, km, vm, p, inl);
-  merge_pair_kernel<D, false><<<grid, kThreads, C::kSmemBytes, s>>>(km, vm, p, inl);
-  return cudaGetLastError();
+  *out = &ps;
+  return cudaSuccess;
 }
 
 const InlineDecodePlan kNoInline{};
 
+// Cost of a row tile's CTAs in a launch of clusters of `split`.
+MergeSplitCost merge_tile_cost(int all_tiles, int n_rows, int split) {
+  // microseconds, measured: a stage of 128 keys for 256 rows and for up to 128
+  // (the tiles taking the stages in turn), a CTA's start and end, the exchange
+  // (a merge of 183 stages took 352, 187, 105, 62 and 50 us in 1, 2, 4, 8 and
+  // 12 parts)
+  constexpr float kStage = 1.9f, kDualStage = 1.15f, kCta = 10.f, kExchange = 6.f;
+  const int parts = merge_parts(all_tiles, split);
+  const float stage = n_rows <= kTileRows ? kDualStage : kStage;
+  const float fixed = kCta + (parts > 1 ? kExchange : 0.f);
+  return {parts, parts * fixed + all_tiles * stage, fixed + (float)((all_tiles + parts - 1) / parts) * stage};
+}
+
+template <int D>
+cudaError_t launch_merge_t(const CUtensorMap& km, const CUtensorMap& vm, AttnParams p, const MergeItem* host_items,
+                           int n_items, cudaStream_t s) {
+  const PairSetup* ps = nullptr;
+  cudaError_t e = pair_setup<D, false>(&ps);
+  if (e != cudaSuccess) return e;
+  const int64_t copies = (int64_t)p.Hkv * p.L;  // of every row tile
+  // CTAs per row tile: the size with the least estimated time, which is waves
+  // of CTAs of average length, or the longest CTA if that is more.  Over 19
+  // shapes and 12 sizes the choice was within 6% of the best one measured (10
+  // parts for 24 row tiles, say, need two waves and take 114 us, where 5 take
+  // 93).  With 8 waves and more the last one's loss is small and a split only
+  // adds CTAs: 4 layers of 256 row tiles took 2.01 ms whole, 2.23 in two parts.
+  int split = 1;
+  if (n_items * copies < 8 * (int64_t)ps->resident[1]) {
+    float best = 0.f;
+    for (int n = 1; n <= kMaxMergeSplit; ++n) {
+      if (ps->resident[n] < 1) continue;
+      int64_t ctas = 0;
+      float total = 0.f, longest = 0.f;
+      for (int i = 0; i < n_items; ++i) {
+        const int T = host_items ? host_items[i].T : p.T, L0 = host_items ? host_items[i].L0 : p.L0;
+        const int row_base = host_items ? host_items[i].row_base : i * 2 * kTileRows;
+        const int rows = std::min(2 * kTileRows, T * p.G - row_base);
+        const int keys = L0 + (row_base + rows - 1) / p.G + 1;
+        const MergeSplitCost c = merge_tile_cost((keys + kKeys - 1) / kKeys, rows, n);
+        ctas += c.parts;
+        total += c.total;
+        longest = std::max(longest, c.longest);
+      }
+      const int64_t waves = (ctas * copies + ps->resident[n] - 1) / ps->resident[n];
+      const float time = std::max(longest, waves * total / ctas);
+      if (n == 1 || time < 0.97f * best) {
+        best = time;
+        split = n;
+      }
+    }
+  }
+  p.kv_split = split;
+  return launch_chained_cluster(merge_pair_kernel<D, false>, dim3(n_items * split, p.Hkv, p.L), dim3(kThreads),
+                                PairCfg<D>::kSmemBytes, s, split, km, vm, p, kNoInline);
+}
+
+template <int D>
+cudaError_t launch_decode_pair_t(const CUtensorMap& km, const CUtensorMap& vm, const AttnParams& p,
+                                 const InlineDecodePlan& inl, int n_items, cudaStream_t s) {
+  const PairSetup* ps = nullptr;
+  cudaError_t e = pair_setup<D, true>(&ps);
+  if (e != cudaSuccess) return e;
+  return launch_chained(merge_pair_kernel<D, true>, dim3(n_items, p.Hkv, p.L), dim3(kThreads), PairCfg<D>::kSmemBytes,
+                        s, km, vm, p, inl);
+}
+
 }  // namespace
 
-cudaError_t launch_merge_tc(const CUtensorMap& km, const CUtensorMap& vm, const AttnParams& p, int n_items,
-                            int D, cudaStream_t s) {
+cudaError_t launch_merge_tc(const CUtensorMap& km, const CUtensorMap& vm, const AttnParams& p,
+                            const MergeItem* host_items, int n_items, int D, cudaStream_t s) {
   // one merge: ceil(T G / 256) row tiles; a batch: its work items
-  const int n_ctas = p.mitems ? n_items : (p.T * p.G + 2 * kTileRows - 1) / (2 * kTileRows);
-  if (n_ctas <= 0) return cudaSuccess;
-  if (D == 128) return launch_pair_t<128, false>(km, vm, p, kNoInline, n_ctas, s);
-  if (D == 64) return launch_pair_t<64, false>(km, vm, p, kNoInline, n_ctas, s);
+  if (!p.mitems) n_items = (p.T * p.G + 2 * kTileRows - 1) / (2 * kTileRows);
+  if (n_items <= 0) return cudaSuccess;
+  if (D == 128) return launch_merge_t<128>(km, vm, p, host_items, n_items, s);
+  if (D == 64) return launch_merge_t<64>(km, vm, p, host_items, n_items, s);
   return cudaErrorInvalidValue;
 }
 
@@ -549,8 +829,8 @@ cudaError_t launch_decode_pair(const CUtensorMap& km, const CUtensorMap& vm, con
                                const InlineDecodePlan* inl, int n_items, int D, cudaStream_t s) {
   const InlineDecodePlan& ip = inl ? *inl : kNoInline;
   if (n_items <= 0) return cudaSuccess;
-  if (D == 128) return launch_pair_t<128, true>(km, vm, p, ip, n_items, s);
-  if (D == 64) return launch_pair_t<64, true>(km, vm, p, ip, n_items, s);
+  if (D == 128) return launch_decode_pair_t<128>(km, vm, p, ip, n_items, s);
+  if (D == 64) return launch_decode_pair_t<64>(km, vm, p, ip, n_items, s);
   return cudaErrorInvalidValue;
 }
 

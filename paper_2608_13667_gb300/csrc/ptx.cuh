@@ -358,4 +358,33 @@ __device__ __forceinline__ void named_barrier_sync(int id, int n_threads) {
   asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n_threads) : "memory");
 }
 
+// Barrier of every thread of the cluster; shared-memory writes before it are
+// visible to the cluster after it.
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+}
+
+// Loads from the shared memory of CTA `cta` of the cluster, at the place of
+// this CTA's shared address `saddr`.
+__device__ __forceinline__ uint32_t cluster_addr(uint32_t saddr, uint32_t cta) {
+  uint32_t a;
+  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(saddr), "r"(cta));
+  return a;
+}
+
+__device__ __forceinline__ float2 ld_cluster_f2(uint32_t saddr, uint32_t cta) {
+  float2 v;
+  asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(cluster_addr(saddr, cta)) : "memory");
+  return v;
+}
+
+__device__ __forceinline__ float4 ld_cluster_f4(uint32_t saddr, uint32_t cta) {
+  float4 v;
+  asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
+               : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+               : "r"(cluster_addr(saddr, cta))
+               : "memory");
+  return v;
+}
+
 }  // namespace st

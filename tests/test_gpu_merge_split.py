@@ -1,0 +1,69 @@
+"""Merges whose row tiles are split over a cluster of CTAs, and tiles of at
+most 128 rows, whose two halves of the tensor memory take the stages in turn:
+against the float64 oracle at the sizes where a part, a stage or a tile begins
+or ends.  A stage is 128 keys and a part at least 4 stages."""
+import pytest
+
+from fg_harness import Run, compare
+from oracle import attention as A
+from workloads import Workload
+
+pytestmark = pytest.mark.gpu
+
+
+def _merge(D, Hq, Hkv, ctx, T, L=1):
+    w = Workload(name=f"split_{D}_{Hq}_{Hkv}_{ctx}_{T}", n_layers=L, n_q_heads=Hq, n_kv_heads=Hkv, head_dim=D,
+                 n_blocks=(ctx + T) // 16 + 8, seed=51)
+    run = Run(w, max_seqs=2, max_decode_branches=1, max_splits=2)
+    m = run.create()
+    if ctx:
+        run.append([m], ctx, ("ctx",))
+    q, o, lse, L0 = run.merge(m, T, ("rows",))
+    run.pool.sync()
+    for layer in range(L):
+        k, v = run.context(m, layer)
+        o_ref, l_ref = A.merge_prefill(q[layer].cpu(), k, v, L0)
+        compare(o[layer], lse[layer], o_ref, l_ref, f"layer {layer}")
+
+
+@pytest.mark.parametrize("ctx,T", [
+    (0, 1),                  # one key: one stage, tile B without any
+    (127, 1), (128, 1),      # one stage full, a second one with one key
+    (300, 32),               # 128 rows: the largest tile that takes the stages in turn
+    (300, 33),               # 132 rows: the smallest of two tiles
+    (1022, 2),               # 8 stages, 2 parts, the last key the last of its part
+    (1023, 2),               # 9 stages: the last part's last stage holds one key
+    (510, 130),              # causal limits on both sides of a part's first key
+    (4096, 20), (6000, 45),  # parts of 4 and 5 stages
+])
+def test_merge_at_part_and_stage_edges(stlib, ctx, T):
+    _merge(128, 32, 8, ctx, T)
+
+
+@pytest.mark.parametrize("ctx,T", [(130, 3), (2050, 16), (9000, 40)])
+def test_merge_split_head_dim_64(stlib, ctx, T):
+    _merge(64, 8, 2, ctx, T)          # 2 row tiles or fewer: clusters of up to 16
+
+
+def test_merge_split_over_many_stages(stlib):
+    _merge(128, 8, 1, 20000, 5)       # one row tile: the largest cluster
+
+
+def test_batch_of_short_and_long_tiles_in_one_cluster_size(stlib):
+    # the launch's clusters suit the long context; the short ones have fewer
+    # parts than a cluster has CTAs, or one
+    w = Workload(name="split_batch", n_layers=2, n_q_heads=32, n_kv_heads=8, head_dim=128, n_blocks=1024, seed=52)
+    run = Run(w, max_seqs=4, max_decode_branches=1, max_splits=2)
+    lens, counts, rids = (9000, 5, 1500), (9, 70, 33), []
+    for i, n in enumerate(lens):
+        rids.append(run.create())
+        run.append([rids[-1]], n, ("ctx", i))
+    q, o, lse, L0 = run.prefill_batch(rids, counts, ("rows",))
+    run.pool.sync()
+    at = 0
+    for r, n, l0 in zip(rids, counts, L0):
+        for layer in range(2):
+            k, v = run.context(r, layer)
+            o_ref, l_ref = A.merge_prefill(q[layer, at:at + n].cpu(), k, v, l0)
+            compare(o[layer, at:at + n], lse[layer, at:at + n], o_ref, l_ref, f"seq {r} layer {layer}")
+        at += n
