@@ -12,14 +12,39 @@ namespace st {
 
 namespace {
 
-__global__ void table_update_kernel(int32_t* __restrict__ table, const TableRun* __restrict__ runs,
-                                    const int32_t* __restrict__ values, int n_runs) {
+// Entries of one run that a block of kTableThreads writes.
+constexpr int kTableThreads = 256;
+constexpr int kTableChunk = 4 * kTableThreads;
+
+// runs and values are in the pinned staging slot and read from there: a copy
+// to the device first is an operation of another engine, whose hand-overs
+// break the chain of dependent launches (with its 2 MiB slot copied whole it
+// took 12 us; the update itself takes 2).  A block's loads are in flight
+// together, since each is a round trip to the host's memory.
+__global__ void __launch_bounds__(kTableThreads)
+    table_update_kernel(int32_t* __restrict__ table, const TableRun* __restrict__ runs,
+                        const int32_t* __restrict__ values) {
   griddep_wait();
   griddep_launch_dependents();
-  for (int r = blockIdx.x; r < n_runs; r += gridDim.x) {
-    const TableRun run = runs[r];
-    for (int i = threadIdx.x; i < run.count; i += blockDim.x) table[run.dst + i] = values[run.src + i];
-  }
+  const TableRun run = runs[blockIdx.x];
+  const int i0 = blockIdx.y * kTableChunk + threadIdx.x;
+  int32_t v[kTableChunk / kTableThreads];
+#pragma unroll
+  for (int u = 0; u < kTableChunk / kTableThreads; ++u)
+    if (i0 + u * kTableThreads < run.count) v[u] = values[run.src + i0 + u * kTableThreads];
+#pragma unroll
+  for (int u = 0; u < kTableChunk / kTableThreads; ++u)
+    if (i0 + u * kTableThreads < run.count) table[run.dst + i0 + u * kTableThreads] = v[u];
+}
+
+// A plan from its pinned staging slot to the device, 16 bytes a thread.  A
+// kernel rather than a copy, so that it is one of the chain of dependent
+// launches.
+__global__ void __launch_bounds__(256) plan_copy_kernel(uint4* __restrict__ dst, const uint4* __restrict__ src, int n) {
+  griddep_wait();
+  griddep_launch_dependents();
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < n) dst[i] = src[i];
 }
 
 // One thread moves 16 bytes (8 bf16).  Index space: copy-on-write chunks
@@ -104,11 +129,17 @@ int grid_for(int64_t total, int threads) {
 
 }  // namespace
 
-cudaError_t launch_table_update(int32_t* table, const TableRun* runs, const int32_t* values,
-                                int n_runs, cudaStream_t s) {
-  if (n_runs <= 0) return cudaSuccess;
-  const int grid = n_runs < 1024 ? n_runs : 1024;
-  return launch_chained(table_update_kernel, dim3(grid), dim3(256), 0, s, table, runs, values, n_runs);
+cudaError_t launch_table_update(int32_t* table, const TableRun* runs, const int32_t* values, int n_runs,
+                                int max_count, cudaStream_t s) {
+  if (n_runs <= 0 || max_count <= 0) return cudaSuccess;
+  const dim3 grid(n_runs, (max_count + kTableChunk - 1) / kTableChunk);
+  return launch_chained(table_update_kernel, grid, dim3(kTableThreads), 0, s, table, runs, values);
+}
+
+cudaError_t launch_plan_copy(void* dst, const void* src, size_t bytes, cudaStream_t s) {
+  const int n = (int)((bytes + 15) / 16);
+  return launch_chained(plan_copy_kernel, dim3((n + 255) / 256), dim3(256), 0, s, static_cast<uint4*>(dst),
+                        static_cast<const uint4*>(src), n);
 }
 
 cudaError_t launch_append(const AppendParams& p, const InlineAppendPlan* inl, int D, cudaStream_t s) {

@@ -1,6 +1,7 @@
 // Parameter blocks and launchers of the device kernels.
 //
 //   table_update  -- refresh rows of the device block tables from the host's
+//   plan_copy     -- a call's plan to the device, where it is too large for the kernel parameters
 //   append_kv     -- copy-on-write page copies + scatter of new K/V rows
 //   attend_tc     -- paged decode partials (tcgen05, TMEM accumulators)
 //   merge_pair    -- causal merge prefill, two query tiles per CTA (tcgen05)
@@ -199,8 +200,11 @@ cudaError_t launch_chained_cluster(void (*kernel)(KArgs...), dim3 grid, dim3 blo
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<Args&&>(args)...);
 }
 
-cudaError_t launch_table_update(int32_t* table, const TableRun* runs, const int32_t* values,
-                                int n_runs, cudaStream_t s);
+// runs, values: readable by the device, here in pinned host memory; max_count: the longest run's.
+cudaError_t launch_table_update(int32_t* table, const TableRun* runs, const int32_t* values, int n_runs,
+                                int max_count, cudaStream_t s);
+// bytes rounded up to 16 from pinned host memory to the device; both 16-byte aligned.
+cudaError_t launch_plan_copy(void* dst, const void* src, size_t bytes, cudaStream_t s);
 cudaError_t launch_append(const AppendParams& p, const InlineAppendPlan* inl, int D, cudaStream_t s);
 cudaError_t launch_combine(const CombineParams& p, const InlineSplits* inl, int D, cudaStream_t s);
 // Decode partials on tcgen05 (one CTA per item x KV head x layer; items from

@@ -159,6 +159,7 @@ struct st_pool {
   int64_t l2_bytes = 0;
   // staging ring
   uint8_t* h_stage = nullptr;
+  uint8_t* h_stage_dev = nullptr;  // the device's address of h_stage
   cudaEvent_t stage_ev[kStageSlots] = {};
   bool stage_used[kStageSlots] = {};
   int stage_next = 0;
@@ -302,9 +303,16 @@ st_status acquire_plan(st_pool* P, Plan* plan, int* slot_out) {
   return ST_OK;
 }
 
+// The device's address of a place in the pinned staging ring.
+template <class T>
+const T* on_device(st_pool* P, const T* h) {
+  return reinterpret_cast<const T*>(P->h_stage_dev + (reinterpret_cast<const uint8_t*>(h) - P->h_stage));
+}
+
 st_status submit_plan(st_pool* P, const Plan& plan, cudaStream_t s) {
-  if (plan.off) CUDA_TRY(P, cudaMemcpyAsync(plan.d, plan.h, plan.off, cudaMemcpyHostToDevice, s));
-  return ST_OK;
+  if (!plan.off) return ST_OK;
+  return run_kernel(P, kKTable, (double)plan.off * 2, 0, s,
+                    [&] { return launch_plan_copy(plan.d, on_device(P, plan.h), plan.off, s); });
 }
 
 st_status retire_plan(st_pool* P, int slot, cudaStream_t s) {
@@ -334,24 +342,21 @@ st_status flush_tables(st_pool* P, cudaStream_t s) {
   while (slot < n) {
     Plan plan;
     int ps;
-    bool any = false;
+    int n_dirty = 0;
     for (int i = slot; i < n; ++i)
-      if (bp.slot(i).live && bp.slot(i).dirty_hi > bp.slot(i).dirty_lo) {
-        any = true;
-        break;
-      }
-    if (!any) return ST_OK;
+      if (bp.slot(i).live && bp.slot(i).dirty_hi > bp.slot(i).dirty_lo) ++n_dirty;
+    if (n_dirty == 0) return ST_OK;
     st_status st = acquire_plan(P, &plan, &ps);
     if (st != ST_OK) return st;
     // runs first (bounded count), then values
-    const int max_runs = 4096;
-    const TableRun* d_runs;
-    TableRun* runs = plan.alloc<TableRun>(max_runs, &d_runs);
+    const int max_runs = std::min(n_dirty, 4096);
+    const TableRun* unused_runs;
+    TableRun* runs = plan.alloc<TableRun>(max_runs, &unused_runs);
     const size_t vals_cap = (plan.cap - plan.off - 64) / sizeof(int32_t);
-    const int32_t* d_vals;
-    int32_t* vals = plan.alloc<int32_t>(vals_cap, &d_vals);
+    const int32_t* unused_vals;
+    int32_t* vals = plan.alloc<int32_t>(vals_cap, &unused_vals);
     int n_runs = 0;
-    size_t n_vals = 0;
+    size_t n_vals = 0, longest = 0;
     for (; slot < n && n_runs < max_runs; ++slot) {
       SeqSlot& ss = bp.slot_mut(slot);
       if (!ss.live || ss.dirty_hi <= ss.dirty_lo) continue;
@@ -362,16 +367,16 @@ st_status flush_tables(st_pool* P, cudaStream_t s) {
       runs[n_runs] = TableRun{(int64_t)slot * bp.max_pages() + ss.dirty_lo, (int32_t)take, (int32_t)n_vals};
       std::memcpy(vals + n_vals, ss.table.data() + ss.dirty_lo, take * sizeof(int32_t));
       n_vals += take;
+      longest = std::max(longest, take);
       ++n_runs;
       ss.dirty_lo += (int32_t)take;
       if (ss.dirty_lo < ss.dirty_hi) break;  // slot only partly uploaded: continue it next round
       ss.dirty_lo = ss.dirty_hi = 0;
     }
-    st = submit_plan(P, plan, s);
-    if (st != ST_OK) return st;
     int32_t* tbl = P->d_tables;
-    st = run_kernel(P, kKTable, (double)n_vals * 8 + n_runs * 16, 0, s,
-                    [&] { return launch_table_update(tbl, d_runs, d_vals, n_runs, s); });
+    st = run_kernel(P, kKTable, (double)n_vals * 8 + n_runs * 16, 0, s, [&] {
+      return launch_table_update(tbl, on_device(P, runs), on_device(P, vals), n_runs, (int)longest, s);
+    });
     if (st != ST_OK) return st;
     st = retire_plan(P, ps, s);
     if (st != ST_OK) return st;
@@ -605,7 +610,9 @@ ST_API st_status st_pool_create(const st_config* cfg, void* k_pool, void* v_pool
   P->decode_ctas_per_sm = decode_tc_ctas_per_sm(cfg->head_dim);
   if (P->decode_ctas_per_sm < 1) return bail(ST_ERR_CUDA);
   if (cudaHostAlloc(reinterpret_cast<void**>(&P->h_stage), (size_t)kStageSlots * kStageSlotBytes,
-                    cudaHostAllocDefault) != cudaSuccess)
+                    cudaHostAllocMapped) != cudaSuccess)
+    return bail(ST_ERR_CUDA);
+  if (cudaHostGetDevicePointer(reinterpret_cast<void**>(&P->h_stage_dev), P->h_stage, 0) != cudaSuccess)
     return bail(ST_ERR_CUDA);
   for (int i = 0; i < kStageSlots; ++i)
     if (cudaEventCreateWithFlags(&P->stage_ev[i], cudaEventDisableTiming) != cudaSuccess)
