@@ -7,92 +7,101 @@
 // softmaxes, lse = log sum_i exp(lse_i) and O = sum_i exp(lse_i - lse) O_i.
 #include <math.h>
 
+#include <type_traits>
+
 #include "kernels.cuh"
 
 namespace st {
 
 namespace {
 
-// One row (one layer, branch and query head) for one warp: lse = log sum_i
+// kWarps warps per row (one layer, branch and query head): lse = log sum_i
 // exp(lse_i), O = sum_i exp(lse_i - lse) O_i over the row's ns partials
-// (ns <= 32).
-template <int D>
-__device__ __forceinline__ void combine_row(const float* lse_i, const float* part_o, int ns, float* o_out,
-                                            float* lse_out, int lane) {
+// (ns <= 32).  Every warp has all the lse values (one per lane) and takes the
+// partials [8 w, 8 w + 8), [8 w + 8 kWarps, ...), eight loads in flight; with
+// more than one warp their sums meet in shared memory.  One warp moves the
+// least for many rows; a launch of few rows is a chain of round trips to L2,
+// which four warps make in one (a single agent's step, 28 partials on each of
+// 160 rows: from the wait for the decode to the last write 3.1 us with one warp
+// and 16 loads in flight, 1.3 with four).  All index arithmetic comes ahead of that wait, in 32 bits.
+constexpr int kBatch = 8;
+constexpr int kFewRows = 152 * 16;  // rows of a small launch
+
+template <int D, int kWarps>
+__global__ void __launch_bounds__(128) combine_kernel(const CombineParams p, const __grid_constant__ InlineSplits inl) {
   constexpr int kPer = D / 32;
-  constexpr int kBatch = 16;  // partials whose loads are in flight together
-  const float* po = part_o + lane * kPer;
-  // this lane's column slice of partial i (zero past the row's partials)
+  using Vec = std::conditional_t<kPer == 4, float4, float2>;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int row = kWarps == 1 ? blockIdx.x * 4 + warp : blockIdx.x;
+  const int part = kWarps == 1 ? 0 : warp;  // this warp's share of the partials
+  const bool live = row < p.n_rows;
+  const int b = (row / p.Hq) % p.n_br;
+  const float* lse_i = p.part_lse + (int64_t)row * p.max_splits;
+  const Vec* po = reinterpret_cast<const Vec*>(p.part_o + (int64_t)row * p.max_splits * D) + lane;
+  griddep_wait();
+  griddep_launch_dependents();
+  if (kWarps == 1 && !live) return;
+  const int ns = p.n_splits ? p.n_splits[b] : inl.n_splits[b];
+  // the first partials are loaded together with the lse values: the loads do
+  // not depend on the weights
   auto load = [&](int i, float* x) {
     if (i < ns) {
-      if constexpr (kPer == 4) {
-        const float4 v = __ldcg(reinterpret_cast<const float4*>(po + (int64_t)i * D));
-        x[0] = v.x;
-        x[1] = v.y;
-        x[2] = v.z;
-        x[3] = v.w;
-      } else {
-        const float2 v = __ldcg(reinterpret_cast<const float2*>(po + (int64_t)i * D));
-        x[0] = v.x;
-        x[1] = v.y;
-      }
+      const Vec v = __ldcg(po + i * 32);
+#pragma unroll
+      for (int e = 0; e < kPer; ++e) x[e] = reinterpret_cast<const float*>(&v)[e];
     } else {
 #pragma unroll
       for (int e = 0; e < kPer; ++e) x[e] = 0.f;
     }
   };
-  // the first batch of partials is loaded together with the lse values: the
-  // loads do not depend on the weights
   const float li = lane < ns ? __ldcg(lse_i + lane) : -INFINITY;
   float x[kBatch][kPer];
 #pragma unroll
-  for (int u = 0; u < kBatch; ++u) load(u, x[u]);
+  for (int u = 0; u < kBatch; ++u) load(part * kBatch + u, x[u]);
   float mx = li;
 #pragma unroll
   for (int off = 16; off; off >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, off));
-  const float w = lane < ns ? expf(li - mx) : 0.f;
+  float w = lane < ns ? expf(li - mx) : 0.f;
   float sum = w;
 #pragma unroll
   for (int off = 16; off; off >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, off);
-  const float lse = mx + logf(sum);
-  const float inv_sum = 1.f / sum;
+  w *= 1.f / sum;
   float out[kPer];
 #pragma unroll
   for (int e = 0; e < kPer; ++e) out[e] = 0.f;
-  for (int i0 = 0; i0 < ns; i0 += kBatch) {
-    if (i0 > 0) {
+#pragma unroll 1
+  for (int i0 = part * kBatch; i0 < ns; i0 += kWarps * kBatch) {
+    if (i0 != part * kBatch) {
 #pragma unroll
       for (int u = 0; u < kBatch; ++u) load(i0 + u, x[u]);
     }
 #pragma unroll
     for (int u = 0; u < kBatch; ++u) {
-      const float wv = i0 + u < ns ? __shfl_sync(0xffffffffu, w, (i0 + u) & 31) * inv_sum : 0.f;
+      const float wv = __shfl_sync(0xffffffffu, w, (i0 + u) & 31);  // 0 past the row's partials
 #pragma unroll
       for (int e = 0; e < kPer; ++e) out[e] += wv * x[u][e];
     }
   }
-  float* dst = o_out + lane * kPer;
-  if constexpr (kPer == 4)
-    *reinterpret_cast<float4*>(dst) = make_float4(out[0], out[1], out[2], out[3]);
-  else
-    *reinterpret_cast<float2*>(dst) = make_float2(out[0], out[1]);
-  if (lane == 0) *lse_out = lse;
-}
-
-
-// One warp per (layer, branch, query head).
-template <int D>
-__global__ void __launch_bounds__(128) combine_kernel(const CombineParams p, const __grid_constant__ InlineSplits inl) {
-  griddep_wait();
-  griddep_launch_dependents();
-  const int32_t* n_splits = p.n_splits ? p.n_splits : inl.n_splits;
-  const int lane = threadIdx.x & 31;
-  const int64_t idx = (int64_t)blockIdx.x * 4 + (threadIdx.x >> 5);
-  const int64_t total = (int64_t)p.L * p.n_br * p.Hq;
-  if (idx >= total) return;
-  const int b = (int)((idx / p.Hq) % p.n_br);
-  combine_row<D>(p.part_lse + idx * p.max_splits, p.part_o + idx * p.max_splits * D, n_splits[b], p.o + idx * D,
-                 p.lse + idx, lane);
+  if constexpr (kWarps > 1) {
+    __shared__ Vec sums[kWarps][32];
+    Vec v;
+#pragma unroll
+    for (int e = 0; e < kPer; ++e) reinterpret_cast<float*>(&v)[e] = out[e];
+    sums[warp][lane] = v;
+    __syncthreads();
+    if (warp != 0) return;
+#pragma unroll
+    for (int k = 1; k < kWarps; ++k) {
+      const Vec o = sums[k][lane];
+#pragma unroll
+      for (int e = 0; e < kPer; ++e) out[e] += reinterpret_cast<const float*>(&o)[e];
+    }
+  }
+  Vec v;
+#pragma unroll
+  for (int e = 0; e < kPer; ++e) reinterpret_cast<float*>(&v)[e] = out[e];
+  reinterpret_cast<Vec*>(p.o + (int64_t)row * D)[lane] = v;
+  if (lane == 0) p.lse[row] = mx + logf(sum);
 }
 
 }  // namespace
@@ -100,11 +109,18 @@ __global__ void __launch_bounds__(128) combine_kernel(const CombineParams p, con
 cudaError_t launch_combine(const CombineParams& p, const InlineSplits* inl, int D, cudaStream_t s) {
   static const InlineSplits kNone{};
   const InlineSplits& ip = inl ? *inl : kNone;
-  const int64_t total = (int64_t)p.L * p.n_br * p.Hq;
-  if (total == 0) return cudaSuccess;
-  const int grid = (int)((total + 3) / 4);
-  if (D == 128) return launch_chained(combine_kernel<128>, dim3(grid), dim3(128), 0, s, p, ip);
-  if (D == 64) return launch_chained(combine_kernel<64>, dim3(grid), dim3(128), 0, s, p, ip);
+  if (p.n_rows == 0) return cudaSuccess;
+  // four warps per row while every row's block is resident at once (a block is
+  // 128 threads, of which an SM holds 16): fewer round trips; beyond, one warp
+  // per row
+  const bool wide = p.n_rows <= kFewRows;
+  const dim3 grid(wide ? p.n_rows : (p.n_rows + 3) / 4);
+  if (D == 128)
+    return wide ? launch_chained(combine_kernel<128, 4>, grid, dim3(128), 0, s, p, ip)
+                : launch_chained(combine_kernel<128, 1>, grid, dim3(128), 0, s, p, ip);
+  if (D == 64)
+    return wide ? launch_chained(combine_kernel<64, 4>, grid, dim3(128), 0, s, p, ip)
+                : launch_chained(combine_kernel<64, 1>, grid, dim3(128), 0, s, p, ip);
   return cudaErrorInvalidValue;
 }
 

@@ -123,7 +123,7 @@ struct CombineParams {
   float* o;                 // [L][n_br][Hq][D]
   float* lse;               // [L][n_br][Hq]
   const int32_t* n_splits;  // [n_br]
-  int32_t n_br, Hq, L, max_splits;
+  int32_t n_br, Hq, n_rows, max_splits;  // n_rows: layers x n_br x Hq
 };
 
 // Small per-call plans travel inside the kernel parameters (no staging copy,

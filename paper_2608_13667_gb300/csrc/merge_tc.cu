@@ -96,12 +96,6 @@ constexpr uint32_t kTmemTile = 256, kTmemO = 128;  // per-tile column base, O of
 constexpr float kRescaleThreshold = 8.f;           // log2 units
 constexpr float kLn2 = 0.69314718055994530942f;
 
-__device__ __forceinline__ float fmax3(float a, float b, float c) {
-  float d;
-  asm("max.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
-  return d;
-}
-
 // CTAs of a cluster that share one row tile's keys in a merge, at most (16 is
 // the largest cluster of this part).
 constexpr int kMaxMergeSplit = 16;

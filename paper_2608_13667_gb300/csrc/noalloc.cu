@@ -268,7 +268,7 @@ extern "C" ST_API st_status st_decode_attn_noalloc(const st_config* geom, const 
   cp.n_splits = dplan->n_splits;
   cp.n_br = n_br;
   cp.Hq = c.n_q_heads;
-  cp.L = c.n_layers;
+  cp.n_rows = c.n_layers * n_br * c.n_q_heads;
   cp.max_splits = kSplitStride;
   if (launch_combine(cp, nullptr, c.head_dim, s) != cudaSuccess) return ST_ERR_CUDA;
   return ST_OK;

@@ -104,9 +104,31 @@ __device__ __forceinline__ float ex2(float x) {
   return y;
 }
 
+__device__ __forceinline__ float fmax3(float a, float b, float c) {
+  float d;
+  asm("max.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
+  return d;
+}
+
 __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
   __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
   return *reinterpret_cast<uint32_t*>(&v);
+}
+
+// Two probabilities 2^(s sl2 - m) of raw scores s as two bf16 terms each,
+// P_hi = bf16(P) and P_lo = bf16(P - P_hi) (P - P_hi is exact in fp32), packed
+// in pairs, and added to a running pair of sums: nine instructions for the two,
+// with the packed f32x2 forms, where separate ones take twelve.
+__device__ __forceinline__ void prob_pair(float s0, float s1, float2 scale2, float2 neg_m2, float2* sum,
+                                          uint32_t* hi, uint32_t* lo) {
+  const float2 x = __ffma2_rn(make_float2(s0, s1), scale2, neg_m2);
+  const float2 p = make_float2(ex2(x.x), ex2(x.y));
+  *sum = __fadd2_rn(*sum, p);
+  const uint32_t h = pack_bf16(p.x, p.y);
+  const float2 r = __ffma2_rn(make_float2(__uint_as_float(h << 16), __uint_as_float(h & 0xffff0000u)),
+                              make_float2(-1.f, -1.f), p);
+  *hi = h;
+  *lo = pack_bf16(r.x, r.y);
 }
 
 }  // namespace st

@@ -1094,7 +1094,7 @@ st_status decode_impl(st_pool* P, const std::vector<int>& slots, const void* q, 
   cp.n_splits = d_nsplit;
   cp.n_br = n_br;
   cp.Hq = c.n_q_heads;
-  cp.L = c.n_layers;
+  cp.n_rows = c.n_layers * n_br * c.n_q_heads;
   cp.max_splits = c.max_splits;
   // algorithmic: O and LSE written once; the partials it reads are the split's own traffic
   const double cbytes = (double)c.n_layers * n_br * c.n_q_heads * (c.head_dim + 1) * 4;
