@@ -64,6 +64,16 @@
 // after it (a single agent's step, 5 stages per CTA: the first scores 1.8 us
 // after the wait, 2.3 with the set-up behind it).
 //
+// A call with large groups launches their tiles first and the narrow items,
+// most of them the branches' own pages, right behind as their programmatic
+// dependents (beside_prev).  Those do not depend on the large tiles' results,
+// and by the time they start, every CTA of the large tiles has passed its own
+// wait: whatever was before both is complete.  So they skip the wait and run on
+// the SMs that the large tiles' last wave leaves idle; only the grid's last CTA
+// waits, at its end, so that what follows (the combine) sees both complete.
+// 12 branches per group, 2 groups, 4 layers: 449 -> 420 us for the two launches;
+// 24 branches, 2 layers: 340 -> 315; one layer, 4 groups of 20: 118 -> 94.
+//
 // Shared-memory operands use the 128-byte swizzle (8-row x 128-byte atoms):
 //   Q  [D/64][rows][64]       K-major A (SBO 1024)
 //   K  [D/64][keys][64]       K-major B (SBO 1024)
@@ -182,7 +192,7 @@ __global__ void __launch_bounds__(kThreads, 2)
   // kernel in the stream (the one that wrote the pages): the tensor-memory
   // allocation, and all of the set-up when the item is in the parameters.
   if (warp == kMmaWarp) tmem_alloc(tmem_slot, kTmemCols);
-  if (p.items) griddep_wait();
+  if (p.items && !p.beside_prev) griddep_wait();
 
   // ---- what this CTA reads and for whom ------------------------------------------
   const int32_t* members = p.members ? p.members : inl.members;
@@ -221,7 +231,7 @@ __global__ void __launch_bounds__(kThreads, 2)
   __syncthreads();
   tc_fence_after_sync();
   const uint32_t tmem = *tmem_slot;
-  if (!p.items) griddep_wait();
+  if (!p.items && !p.beside_prev) griddep_wait();
   griddep_launch_dependents();
 
   // ---- loader --------------------------------------------------------------------
@@ -478,6 +488,9 @@ __global__ void __launch_bounds__(kThreads, 2)
     named_barrier_sync(1, n_swt + 32);
     tc_fence_after_sync();
     tmem_dealloc(tmem, kTmemCols);
+    // beside_prev: this grid is complete only once the one before it is
+    if (p.beside_prev && blockIdx.x == gridDim.x - 1 && blockIdx.y == gridDim.y - 1 && blockIdx.z == gridDim.z - 1)
+      griddep_wait();
     return;
   }
   if (warp >= n_sw) return;

@@ -1071,14 +1071,17 @@ st_status decode_impl(st_pool* P, const std::vector<int>& slots, const void* q, 
   const int n_pair = n_items - n_narrow - n_wide;
   st = run_kernel(P, kKDecode, bytes, flops, s, [&] {
     const InlineDecodePlan* ip = inline_plan ? &inl : nullptr;
-    cudaError_t e = launch_decode_tc(P->kmap, P->vmap, ap, ip, n_narrow, c.head_dim, false, s);
-    if (e != cudaSuccess) return e;
+    // the large tiles first, the narrow items beside their last wave
     AttnParams aw = ap;
     aw.item_base = n_narrow;
-    e = launch_decode_tc(P->kmap, P->vmap, aw, ip, n_wide, c.head_dim, true, s);
+    cudaError_t e = launch_decode_tc(P->kmap, P->vmap, aw, ip, n_wide, c.head_dim, true, s);
     if (e != cudaSuccess) return e;
     aw.item_base = n_narrow + n_wide;
-    return launch_decode_pair(P->kmap, P->vmap, aw, ip, n_pair, c.head_dim, s);
+    e = launch_decode_pair(P->kmap, P->vmap, aw, ip, n_pair, c.head_dim, s);
+    if (e != cudaSuccess) return e;
+    aw.item_base = 0;
+    aw.beside_prev = n_wide > 0 || n_pair > 0 ? 1 : 0;
+    return launch_decode_tc(P->kmap, P->vmap, aw, ip, n_narrow, c.head_dim, false, s);
   }, (n_narrow > 0 ? 1 : 0) + (n_wide > 0 ? 1 : 0) + (n_pair > 0 ? 1 : 0),
                   dp.reread_bytes + part_bytes);
   if (st != ST_OK) {
