@@ -64,6 +64,21 @@
 // after it (a single agent's step, 5 stages per CTA: the first scores 1.8 us
 // after the wait, 2.3 with the set-up behind it).
 //
+// More than one wave (kPersist).  A run of pages is some 20 us of streaming,
+// and a CTA of its own for each spends about 7 more on its start and its end,
+// in which its half of the SM's shared memory has nothing in flight.  So a CTA
+// that has issued its run's last loads but one asks for a CTA of the grid that
+// has not started (cluster launch control: no queue, no counter to reset) and
+// goes on with its item: the loads of the next run follow at once, its Q goes in
+// and its first S is computed while the results of this one come out.  Stage,
+// S-buffer and barrier counts run on over a CTA's items.  The loader passes the
+// items on through two slots; every role reads them in order.  The request is
+// made late, because an item taken over early waits behind its CTA while
+// another SM may have run dry (batched serving: 214 us early, 211 late; 221
+// with a CTA for every run).  32 layers over 23k tokens 481 -> 461 us, 64
+// unforked sequences 376 -> 356, 12 branches per group 417 -> 403, D = 64 142
+// -> 129, long trajectories 1339 -> 1335.
+//
 // A call with large groups launches their tiles first and the narrow items,
 // most of them the branches' own pages, right behind as their programmatic
 // dependents (beside_prev).  Those do not depend on the large tiles' results,
@@ -151,10 +166,17 @@ struct TcCfg {
   // memory, so the kernel requires the dynamic shared memory to start on a
   // 1024-byte boundary (it does when a kernel has no static shared memory;
   // the kernel checks and reports ST_ERR_CUDA otherwise)
-  static constexpr int kSmemBytes = kBarOffset + 256;
+  static constexpr int kSmemBytes = kBarOffset + 512;
 };
 
-template <int D, bool kWide, bool kElect>
+// An item of a launch for one KV head of one layer.
+struct Work {
+  AttnItem item;
+  int kvh, layer;
+  int valid;  // 0: there is none
+};
+
+template <int D, bool kWide, bool kElect, bool kPersist>
 __global__ void __launch_bounds__(kThreads, 2)
     attend_tc_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant__ CUtensorMap vmap,
                      const AttnParams p, const __grid_constant__ InlineDecodePlan inl) {
@@ -177,35 +199,39 @@ __global__ void __launch_bounds__(kThreads, 2)
   uint64_t* s_full = bars + 2 * C::kStages;   // [2] per S buffer
   uint64_t* p_full = s_full + 2;              // [2] per S buffer
   uint64_t* o_ready = s_full + 4;             // one phase per P V
-  uint64_t* o_final = s_full + 5;
-  uint64_t* q_ready = s_full + 6;
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(s_full + 7);
-  uint64_t* v_full = s_full + 8;               // [kVStages] wide: V landed
+  uint64_t* q_ready = s_full + 5;
+  uint64_t* v_full = s_full + 6;               // [kVStages] wide: V landed
   uint64_t* v_empty = v_full + C::kVStages;    // [kVStages] wide: V slot free
+  uint64_t* work_full = v_empty + C::kVStages; // [2] an item taken over is in its slot
+  uint64_t* work_empty = work_full + 2;        // [2] every role has read it
+  uint64_t* clc_bar = work_full + 4;           // the answer to a request for one has landed
+  uint64_t* o_final = work_full + 5;           // one phase per item: its last P V
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(work_full + 6);
+  uint8_t* clc_resp = reinterpret_cast<uint8_t*>(base + C::kBarOffset + 384);  // 16 bytes
+  Work* work_slots = reinterpret_cast<Work*>(base + C::kBarOffset + 400);      // [2]
+  static_assert(8 * (2 * C::kStages + 6 + 2 * C::kVStages + 7) <= 384 && 400 + 2 * sizeof(Work) <= 512, "barrier area");
 
   const int warp = threadIdx.x >> 5;
   const int lane = threadIdx.x & 31;
-  const int kvh = blockIdx.y;
-  const int layer = blockIdx.z;
   const int G = p.G;
   // What touches no global memory comes ahead of the wait for the previous
   // kernel in the stream (the one that wrote the pages): the tensor-memory
   // allocation, and all of the set-up when the item is in the parameters.
   if (warp == kMmaWarp) tmem_alloc(tmem_slot, kTmemCols);
-  if (p.items && !p.beside_prev) griddep_wait();
+  const bool beside = !kPersist && p.beside_prev;
+  if (p.items && !beside) griddep_wait();
 
   // ---- what this CTA reads and for whom ------------------------------------------
   const int32_t* members = p.members ? p.members : inl.members;
-  const int item_idx = p.item_base + blockIdx.x;
-  const AttnItem item = p.items ? p.items[item_idx] : inl.items[item_idx];
-  const int slot = item.slot;
-  const int page_begin = item.page_begin;
-  const int n_pages = item.n_pages;
-  const int n_valid_keys = item.n_tokens;
-  const int n_rows = item.n_members * G;
-  const int n_tiles = (n_pages + C::kPagesPerStage - 1) / C::kPagesPerStage;
-  const int n_sw = (n_rows + C::kRowsPerWarp - 1) / C::kRowsPerWarp;  // softmax warps with rows
-  const int n_swt = n_sw * 32;
+  auto item_at = [&](int x) -> const AttnItem& {
+    return p.items ? p.items[p.item_base + x] : inl.items[p.item_base + x];
+  };
+  Work work{item_at(blockIdx.x), (int)blockIdx.y, (int)blockIdx.z, 1};
+  auto stages_of = [&](const Work& w) { return (w.item.n_pages + C::kPagesPerStage - 1) / C::kPagesPerStage; };
+  // softmax warps with rows of an item
+  auto warps_of = [&](const Work& w) { return (w.item.n_members * G + C::kRowsPerWarp - 1) / C::kRowsPerWarp; };
+  // warps that take part in the hand-overs: with items of different rows to come, all of them
+  const int n_part = kPersist ? 4 : warps_of(work);
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < C::kStages; ++s) {
@@ -220,30 +246,47 @@ __global__ void __launch_bounds__(kThreads, 2)
     }
     for (int b = 0; b < 2; ++b) {
       mbar_init(&s_full[b], 1);
-      mbar_init(&p_full[b], n_swt);
+      mbar_init(&p_full[b], n_part);
+      mbar_init(&work_full[b], 1);
+      mbar_init(&work_empty[b], 5);  // the softmax warps and the MMA warp
     }
     mbar_init(o_ready, 1);
     mbar_init(o_final, 1);
-    mbar_init(q_ready, n_swt);
+    mbar_init(q_ready, n_part);
+    mbar_init(clc_bar, 1);
     fence_mbar_init();
   }
   tc_fence_before_sync();
   __syncthreads();
   tc_fence_after_sync();
   const uint32_t tmem = *tmem_slot;
-  if (!p.items && !p.beside_prev) griddep_wait();
+  if (!p.items && !beside) griddep_wait();
   griddep_launch_dependents();
+
+  // The item after a role's n-th: written to slot n % 2 by the loader.  False
+  // when there is none (or the wait ran out: *ok).
+  auto next_work = [&](int n, Work* w, bool* ok, bool one_lane) -> bool {
+    const int b = n & 1;
+    *ok = one_lane ? mbar_wait(&work_full[b], (n >> 1) & 1)
+                   : __all_sync(0xffffffffu, mbar_wait(&work_full[b], (n >> 1) & 1));
+    if (!*ok) return false;
+    *w = work_slots[b];
+    if (!one_lane) __syncwarp();
+    if (one_lane || lane == 0) mbar_arrive(&work_empty[b]);
+    return w->valid != 0;
+  };
 
   // ---- loader --------------------------------------------------------------------
   if (warp == kLoadWarp) {
-    if (!kWide && (item.flags & kItemAppend)) {
-      // a decode step: this run's last key is the row the step appends.  The
-      // warp writes this (layer, KV head)'s K and V of it into the pool (16
-      // bytes per lane) before anything else, so the row is stored even if a
-      // wait of this CTA runs out later, and makes the writes visible to the
-      // TMA copy that loads the page.
-      const int last = n_valid_keys - 1;  // key within the run
-      const int blk = p.table[(int64_t)slot * p.max_pages + page_begin + last / kPageTokens];
+    // A decode step: the last key of a flagged item is the row the step appends.
+    // The warp writes this (layer, KV head)'s K and V of it into the pool (16
+    // bytes per lane) before anything else, so the row is stored even if a
+    // wait of this CTA runs out later, and makes the writes visible to the
+    // TMA copy that loads the page.
+    auto append_row = [&](const Work& w) {
+      if (kWide || !(w.item.flags & kItemAppend)) return;
+      const int last = w.item.n_tokens - 1;  // key within the run
+      const int blk = p.table[(int64_t)w.item.slot * p.max_pages + w.item.page_begin + last / kPageTokens];
       constexpr int kChunks = D / 8;
       if (lane < 2 * kChunks) {
         if ((uint64_t)blk >= (uint64_t)p.n_blocks) {
@@ -251,129 +294,134 @@ __global__ void __launch_bounds__(kThreads, 2)
         } else {
           const bool is_v = lane >= kChunks;
           const int c = lane % kChunks;
-          const int64_t src = (((int64_t)layer * p.n_rows_q + members[item.member_base]) * p.Hkv + kvh) * D + c * 8;
+          const int64_t src =
+              (((int64_t)w.layer * p.n_rows_q + members[w.item.member_base]) * p.Hkv + w.kvh) * D + c * 8;
           const int64_t dst =
-              ((((int64_t)layer * p.n_blocks + blk) * p.Hkv + kvh) * kPageTokens + last % kPageTokens) * D + c * 8;
+              ((((int64_t)w.layer * p.n_blocks + blk) * p.Hkv + w.kvh) * kPageTokens + last % kPageTokens) * D + c * 8;
           *reinterpret_cast<uint4*>((is_v ? p.v_pool : p.k_pool) + dst) =
               *reinterpret_cast<const uint4*>((is_v ? p.app_v : p.app_k) + src);
           fence_proxy_async_global();
         }
       }
       __syncwarp();
+    };
+    if (p.hold_loads) {  // test hook: nothing arrives, the other roles' waits run out
+      append_row(work);
+      return;
     }
-    if (p.hold_loads) return;  // test hook: nothing arrives, the other roles' waits run out
     if (lane == 0) {
       prefetch_tensormap(&kmap);
       prefetch_tensormap(&vmap);
     }
-    // a page is streamed once, unless a sibling item (the group's other
-    // subgroup, scheduled next to this one) reads it too, or the whole launch
-    // fits in L2 (one agent's step, read again by the next step): then keep it
-    const uint64_t policy =
-        (p.keep_l2 || (item.flags & kItemReread)) ? l2_policy_evict_normal() : l2_policy_evict_first();
-    const int32_t* ids = p.table + (int64_t)slot * p.max_pages + page_begin;
-    int base_id = 0;
-    int cur = lane < n_pages ? ids[lane] : 0;
-    int nxt = 32 + lane < n_pages ? ids[32 + lane] : 0;
-    // waits for the slot of stage j in a ring of `depth` slots to be
-    // released (lane 0 waits)
-    auto slot_free = [&](uint64_t* ring_empty, int depth, int j) -> bool {
+    // lane 0 waits, for the warp
+    auto wait0 = [&](uint64_t* bar, uint32_t parity) -> bool {
       int w = 1;
-      if (j >= depth && lane == 0) w = mbar_wait(&ring_empty[j % depth], ((j / depth) - 1) & 1) ? 1 : 0;
+      if (lane == 0) w = mbar_wait(bar, parity) ? 1 : 0;
       return __shfl_sync(0xffffffffu, w, 0) != 0;
     };
-    // pages of stage j (j increasing): the count and the TMA page coordinates
-    auto stage_pages = [&](int j, int* c3) -> int {
-      const int page0 = j * C::kPagesPerStage;
-      if (page0 >= base_id + 32) {
-        base_id += 32;
-        cur = nxt;
-        nxt = base_id + 32 + lane < n_pages ? ids[base_id + 32 + lane] : 0;
-      }
-      const int np = min(C::kPagesPerStage, n_pages - page0);
-#pragma unroll
-      for (int q = 0; q < C::kPagesPerStage; ++q) {
-        int b = __shfl_sync(0xffffffffu, cur, (page0 - base_id + q) & 31);
-        if (q < np && (uint64_t)b >= (uint64_t)p.n_blocks) {
-          if (lane == 0) atomicCAS(p.status, 0, kDevBadIndex);
-          b = 0;
-        }
-        c3[q] = layer * (int)p.n_blocks + b;
-      }
-      return np;
+    // waits for the slot of the CTA's g-th stage in a ring of `depth` slots to be released
+    auto slot_free = [&](uint64_t* ring_empty, int depth, int g) -> bool {
+      return g < depth || wait0(&ring_empty[g % depth], ((g / depth) - 1) & 1);
     };
-    // wide: np pages of one operand into a slot, completing on bar, one copy
-    // per lane (lane = D/64 q + h), after lane 0's expect-tx
     const uint32_t page_bytes = (uint32_t)(C::kHalves * kPageTokens * 128);
-    auto issue = [&](const CUtensorMap* map, uint8_t* dst, uint64_t* bar, const int* c3, int np) {
-      __syncwarp();
-      const int q = lane / C::kHalves, h = lane % C::kHalves;
-      int cq = c3[0];
-#pragma unroll
-      for (int i = 1; i < C::kPagesPerStage; ++i)
-        if (q == i) cq = c3[i];
-      if (lane < C::kHalves * np)
-        tma_load_4d(dst + h * C::kKVHalfBytes + q * kPageTokens * 128, map, bar, 0, h, kvh * kPageTokens, cq,
-                    policy);
-    };
-    int jk = 0, jv = 0;  // stages whose K and V copies have been issued
+    int gk = 0, gv = 0;  // stages whose K and V copies have been issued, over all items
     bool ok = true;
-    for (; jk < n_tiles; ++jk) {
-      const int s = jk % C::kStages;
-      if (!slot_free(empty, C::kStages, jk)) {
-        ok = false;
-        break;
-      }
-      uint8_t* kst = k_slot(s);
-      if constexpr (C::kSplitKV) {
-        int c3[C::kPagesPerStage];
-        const int np = stage_pages(jk, c3);
-        if (lane == 0) mbar_arrive_expect_tx(&full[s], np * page_bytes);
-        issue(&kmap, kst, &full[s], c3, np);
-        // the K slot was released by S_j-kStages, the V slot waits for P_j-kVStages V_j-kVStages
-        const int sv = jk % C::kVStages;
-        if (!slot_free(v_empty, C::kVStages, jk)) {
+    for (int n = 0;; ++n) {  // the CTA's items
+      append_row(work);
+      const int n_pages = work.item.n_pages, n_tiles = stages_of(work);
+      // a page is streamed once, unless a sibling item (the group's other
+      // subgroup, scheduled next to this one) reads it too, or the whole launch
+      // fits in L2 (one agent's step, read again by the next step): then keep it
+      const uint64_t policy =
+          (p.keep_l2 || (work.item.flags & kItemReread)) ? l2_policy_evict_normal() : l2_policy_evict_first();
+      const int32_t* ids = p.table + (int64_t)work.item.slot * p.max_pages + work.item.page_begin;
+      int base_id = 0;
+      int cur = lane < n_pages ? ids[lane] : 0;
+      int nxt = 32 + lane < n_pages ? ids[32 + lane] : 0;
+      bool asked = false;
+      for (int j = 0; j < n_tiles; ++j) {
+        // ask for the next item just early enough: one taken over sooner waits
+        // here while another SM may have run dry
+        if (kPersist && j == max(0, n_tiles - 2)) {
+          asked = true;
+          if (lane == 0) {
+            mbar_arrive_expect_tx(clc_bar, 16);
+            clc_try_cancel(clc_resp, clc_bar);
+          }
+        }
+        if (!slot_free(empty, C::kStages, gk)) {
           ok = false;
-          ++jk;  // K_j is in flight
           break;
         }
-        if (lane == 0) mbar_arrive_expect_tx(&v_full[sv], np * page_bytes);
-        issue(&vmap, v_slot(sv), &v_full[sv], c3, np);
-        jv = jk + 1;
-      } else {
-        uint8_t* vst = v_slot(s);
-        const int page0 = jk * C::kPagesPerStage;
+        const int page0 = j * C::kPagesPerStage;
         if (page0 >= base_id + 32) {
           base_id += 32;
           cur = nxt;
           nxt = base_id + 32 + lane < n_pages ? ids[base_id + 32 + lane] : 0;
         }
         const int np = min(C::kPagesPerStage, n_pages - page0);
-        if (lane == 0) mbar_arrive_expect_tx(&full[s], 2 * np * page_bytes);
-        __syncwarp();
-        // one copy per lane (lane = 2 D/64 q + (V ? D/64 : 0) + h): a single
-        // thread issuing them one after another is what limits the stage rate
-        constexpr int kPerPage = 2 * C::kHalves;
-        const int q = lane / kPerPage, r = lane % kPerPage;
-        const int h = r % C::kHalves;
-        const bool is_v = r >= C::kHalves;
+        // one copy per lane (a single thread issuing them one after another is
+        // what limits the stage rate): lane = D/64 q + h for an operand of its
+        // own, 2 D/64 q + (V ? D/64 : 0) + h for K and V together
+        constexpr int kPerPage = (C::kSplitKV ? 1 : 2) * C::kHalves;
+        const int q = lane / kPerPage, r = lane % kPerPage, h = r % C::kHalves;
         int b = __shfl_sync(0xffffffffu, cur, (page0 - base_id + (q < C::kPagesPerStage ? q : 0)) & 31);
-        if (lane < kPerPage * np) {
-          if ((uint64_t)b >= (uint64_t)p.n_blocks) {
-            atomicCAS(p.status, 0, kDevBadIndex);
-            b = 0;
+        const bool mine = lane < kPerPage * np;
+        if (mine && (uint64_t)b >= (uint64_t)p.n_blocks) {
+          atomicCAS(p.status, 0, kDevBadIndex);
+          b = 0;
+        }
+        const uint32_t at = h * C::kKVHalfBytes + q * kPageTokens * 128;
+        const int c2 = work.kvh * kPageTokens, c3 = work.layer * (int)p.n_blocks + b;
+        uint64_t* bar = &full[gk % C::kStages];
+        uint8_t* kst = k_slot(gk % C::kStages);
+        if (lane == 0) mbar_arrive_expect_tx(bar, (C::kSplitKV ? 1 : 2) * np * page_bytes);
+        __syncwarp();
+        if constexpr (C::kSplitKV) {
+          if (mine) tma_load_4d(kst + at, &kmap, bar, 0, h, c2, c3, policy);
+          ++gk;
+          // the K slot was released by an S, the V slot waits for its P V
+          if (!slot_free(v_empty, C::kVStages, gv)) {
+            ok = false;
+            break;
           }
-          tma_load_4d((is_v ? vst : kst) + h * C::kKVHalfBytes + q * kPageTokens * 128, is_v ? &vmap : &kmap,
-                      &full[s], 0, h, kvh * kPageTokens, layer * (int)p.n_blocks + b, policy);
+          uint64_t* vbar = &v_full[gv % C::kVStages];
+          if (lane == 0) mbar_arrive_expect_tx(vbar, np * page_bytes);
+          __syncwarp();
+          if (mine) tma_load_4d(v_slot(gv % C::kVStages) + at, &vmap, vbar, 0, h, c2, c3, policy);
+          ++gv;
+        } else {
+          const bool is_v = r >= C::kHalves;
+          if (mine)
+            tma_load_4d((is_v ? v_slot(gk % C::kStages) : kst) + at, is_v ? &vmap : &kmap, bar, 0, h, c2, c3, policy);
+          ++gk;
         }
       }
+      if (!kPersist) break;
+      uint32_t x = 0, y = 0, z = 0;
+      const bool answered = asked && __all_sync(0xffffffffu, mbar_wait(clc_bar, n & 1));
+      const bool more = answered && clc_answer(clc_resp, &x, &y, &z);
+      fence_proxy_async_smem();  // every lane has read the answer before the next one lands
+      __syncwarp();
+      if (more) work = Work{item_at(x), (int)y, (int)z, 1};
+      else work.valid = 0;
+      ok = ok && answered && (n < 2 || wait0(&work_empty[n & 1], ((n >> 1) - 1) & 1));
+      if (!ok) {  // the item taken over is lost with this CTA, but not the row it appends
+        if (more) append_row(work);
+        break;
+      }
+      if (lane == 0) {
+        work_slots[n & 1] = work;
+        mbar_arrive(&work_full[n & 1]);
+      }
+      if (!work.valid) break;
     }
     if (!ok && lane == 0) {
       atomicCAS(p.status, 0, kDevTimeout);
       // wait (bounded) for this CTA's copies still in flight before it exits
-      for (int t = max(0, jk - C::kStages); t < jk; ++t) mbar_wait(&full[t % C::kStages], (t / C::kStages) & 1);
+      for (int t = max(0, gk - C::kStages); t < gk; ++t) mbar_wait(&full[t % C::kStages], (t / C::kStages) & 1);
       if constexpr (C::kSplitKV)
-        for (int t = max(0, jv - C::kVStages); t < jv; ++t)
+        for (int t = max(0, gv - C::kVStages); t < gv; ++t)
           mbar_wait(&v_full[t % C::kVStages], (t / C::kVStages) & 1);
     }
     return;
@@ -412,88 +460,96 @@ __global__ void __launch_bounds__(kThreads, 2)
       const uint64_t q_desc = tc_desc_sw128(smem_addr(q_s), 16, 1024);
       const uint64_t k_desc0 = tc_desc_sw128(smem_addr(ring), 16, 1024);
       const uint64_t v_desc0 = tc_desc_sw128(smem_addr(ring + C::kKRingBytes), C::kKVHalfBytes, 1024);
-      bool ok = wait(q_ready, 0);
-      tc_fence_after_sync();
-      // S_j = Q K_j^T into S buffer j & 1
-      auto issue_s = [&](int j) -> bool {
-        const int s = j % C::kStages;
-        if (!wait(&full[s], (j / C::kStages) & 1)) return false;
+      // S of the CTA's g-th stage = Q K^T into S buffer g & 1
+      auto issue_s = [&](int g) -> bool {
+        const int s = g % C::kStages;
+        if (!wait(&full[s], (g / C::kStages) & 1)) return false;
         tc_fence_after_sync();
         const uint64_t kd = k_desc0 + (uint64_t)((s * C::kKSlotBytes) >> 4);
 #pragma unroll
         for (int h = 0; h < C::kHalves; ++h)
 #pragma unroll
           for (int kk = 0; kk < 4; ++kk)
-            mma_ss(tmem + kTmemS + (j & 1) * C::kKeys, q_desc + (uint64_t)((h * C::kQHalfBytes + kk * 32) >> 4),
+            mma_ss(tmem + kTmemS + (g & 1) * C::kKeys, q_desc + (uint64_t)((h * C::kQHalfBytes + kk * 32) >> 4),
                    kd + (uint64_t)((h * C::kKVHalfBytes + kk * 32) >> 4), idesc_s, (h | kk) != 0);
-        commit(&s_full[j & 1]);
-        if constexpr (C::kSplitKV) commit(&empty[s]);  // K_j has been read
+        commit(&s_full[g & 1]);
+        if constexpr (C::kSplitKV) commit(&empty[s]);  // K has been read
         return true;
       };
-      if (ok) ok = issue_s(0);
-      for (int j = 0; ok && j < n_tiles; ++j) {
-        // S buffer (j+1)&1 was last read by the softmax of stage j-1, whose P
-        // this thread has already waited for.  Issue S_{j+1} ahead of P_j V_j
-        // only when its data has already landed, so that a slow load never
-        // delays P_j V_j.
-        const int jn = j + 1;
-        bool early = false;
-        if (jn < n_tiles && landed(&full[jn % C::kStages], (jn / C::kStages) & 1)) {
-          if (!issue_s(jn)) {
-            ok = false;
-            break;
-          }
-          early = true;
-        }
-        if (!wait(&p_full[j & 1], (j >> 1) & 1)) {
-          ok = false;
-          break;
-        }
+      bool ok = true;
+      int g0 = 0;  // the item's first stage among the CTA's
+      for (int n = 0;; ++n) {
+        const int g1 = g0 + stages_of(work);
+        ok = wait(q_ready, n & 1);
         tc_fence_after_sync();
-        const int s = j % C::kStages, sv = j % C::kVStages;
-        const uint64_t kd = k_desc0 + (uint64_t)((s * C::kKSlotBytes) >> 4);
-        const uint64_t vd0 = v_desc0 + (uint64_t)((sv * C::kVSlotBytes) >> 4);
-        if constexpr (kWide) {
-          if (!wait(&v_full[sv], (j / C::kVStages) & 1)) {
+        if (ok) ok = issue_s(g0);
+        for (int g = g0; ok && g < g1; ++g) {
+          // S buffer (g + 1) & 1 was last read by the softmax of stage g - 1,
+          // whose P this thread has already waited for.  Issue S of the next
+          // stage ahead of this one's P V only when its data has already
+          // landed, so that a slow load never delays P V.
+          const int gn = g + 1;
+          bool early = false;
+          if (gn < g1 && landed(&full[gn % C::kStages], (gn / C::kStages) & 1)) {
+            if (!issue_s(gn)) {
+              ok = false;
+              break;
+            }
+            early = true;
+          }
+          if (!wait(&p_full[g & 1], (g >> 1) & 1)) {
             ok = false;
             break;
           }
           tc_fence_after_sync();
-          // P_hi, P_lo of keys [16 ks, 16 ks + 16) in the 16 TMEM columns of their scores
-          const uint32_t p_tm = tmem + kTmemS + (j & 1) * C::kKeys;
+          const int s = g % C::kStages, sv = g % C::kVStages;
+          const uint64_t kd = k_desc0 + (uint64_t)((s * C::kKSlotBytes) >> 4);
+          const uint64_t vd0 = v_desc0 + (uint64_t)((sv * C::kVSlotBytes) >> 4);
+          if constexpr (kWide) {
+            if (!wait(&v_full[sv], (g / C::kVStages) & 1)) {
+              ok = false;
+              break;
+            }
+            tc_fence_after_sync();
+            // P_hi, P_lo of keys [16 ks, 16 ks + 16) in the 16 TMEM columns of their scores
+            const uint32_t p_tm = tmem + kTmemS + (g & 1) * C::kKeys;
 #pragma unroll
-          for (int ks = 0; ks < C::kKeys / 16; ++ks) {
-            const uint64_t vd = vd0 + (uint64_t)((ks * 16 * 128) >> 4);
-            mma_ts(tmem + kTmemO, p_tm + ks * 16, vd, idesc_o, (j > 0 || ks > 0) ? 1u : 0u);
-            mma_ts(tmem + kTmemO, p_tm + ks * 16 + 8, vd, idesc_o, 1u);
+            for (int ks = 0; ks < C::kKeys / 16; ++ks) {
+              const uint64_t vd = vd0 + (uint64_t)((ks * 16 * 128) >> 4);
+              mma_ts(tmem + kTmemO, p_tm + ks * 16, vd, idesc_o, (g > g0 || ks > 0) ? 1u : 0u);
+              mma_ts(tmem + kTmemO, p_tm + ks * 16 + 8, vd, idesc_o, 1u);
+            }
+          } else {
+            // [P_hi; P_lo] V: one M = 128 product per 16 keys for both terms
+#pragma unroll
+            for (int ks = 0; ks < C::kKeys / 16; ++ks)
+              mma_ss(tmem + kTmemO, kd + (uint64_t)((ks * 32) >> 4), vd0 + (uint64_t)((ks * 16 * 128) >> 4), idesc_o,
+                     (g > g0 || ks > 0) ? 1u : 0u);
           }
-        } else {
-          // [P_hi; P_lo] V: one M = 128 product per 16 keys for both terms
-#pragma unroll
-          for (int ks = 0; ks < C::kKeys / 16; ++ks)
-            mma_ss(tmem + kTmemO, kd + (uint64_t)((ks * 32) >> 4), vd0 + (uint64_t)((ks * 16 * 128) >> 4), idesc_o,
-                   (j > 0 || ks > 0) ? 1u : 0u);
+          commit(C::kSplitKV ? &v_empty[sv] : &empty[s]);
+          commit(o_ready);
+          if (gn < g1 && !early && !issue_s(gn)) {
+            ok = false;
+            break;
+          }
         }
-        commit(C::kSplitKV ? &v_empty[sv] : &empty[s]);
-        commit(o_ready);
-        if (jn < n_tiles && !early && !issue_s(jn)) {
-          ok = false;
-          break;
-        }
+        commit(o_final);
+        g0 = g1;
+        if (!kPersist || !ok || !next_work(n, &work, &ok, !kElect)) break;
       }
-      commit(o_final);
       if (!ok && lane == 0) atomicCAS(p.status, 0, kDevTimeout);
     }
     __syncwarp();
-    named_barrier_sync(1, n_swt + 32);
+    named_barrier_sync(1, n_part * 32 + 32);
     tc_fence_after_sync();
     tmem_dealloc(tmem, kTmemCols);
-    // beside_prev: this grid is complete only once the one before it is
-    if (p.beside_prev && blockIdx.x == gridDim.x - 1 && blockIdx.y == gridDim.y - 1 && blockIdx.z == gridDim.z - 1)
+    // beside_prev: this grid is complete only once the one before it is (not
+    // with kPersist, where this CTA may be taken over before it starts)
+    if (beside && blockIdx.x == gridDim.x - 1 && blockIdx.y == gridDim.y - 1 && blockIdx.z == gridDim.z - 1)
       griddep_wait();
     return;
   }
-  if (warp >= n_sw) return;
+  if (warp >= n_part) return;
 
   // ---- softmax warps ---------------------------------------------------------------
   // Narrow: threads t and t + 16 of a warp share row t and half of the
@@ -502,240 +558,304 @@ __global__ void __launch_bounds__(kThreads, 2)
   // of O_lo (P_lo V).  Wide: one thread per row.
   constexpr bool kPair = !kWide;
   constexpr int kKpt = C::kKeys / (kPair ? 2 : 1);  // keys per thread per stage
-  const int tid = threadIdx.x;                      // 0 .. n_swt-1, for cooperative loops
   const int half = kPair ? (lane >> 4) : 0;
   const int r = kPair ? warp * 16 + (lane & 15) : threadIdx.x;  // this thread's row
   const uint32_t t_lane = tmem + ((uint32_t)(warp * 32) << 16);
-  const bool valid = r < n_rows;
-  int qrow = 0, head = 0;
-  if (valid) {
-    qrow = members[item.member_base + r / G];
-    head = kvh * G + r % G;
-  }
-  if (r < C::kQRows) {
-    const uint4* src = reinterpret_cast<const uint4*>(p.q + (((int64_t)layer * p.n_rows_q + qrow) * p.Hq + head) * D);
-    constexpr int kChunks = D / 8 / (kPair ? 2 : 1);  // 16-byte chunks of the row this thread writes
+
+  // this thread's row of an item among the rows of Q, or -1
+  auto q_row = [&](const Work& w) -> int64_t {
+    if (r >= w.item.n_members * G) return -1;
+    const int64_t row = (int64_t)w.layer * p.n_rows_q + members[w.item.member_base + r / G];
+    return row * p.Hq + w.kvh * G + r % G;
+  };
+  // an item's Q to shared memory, where the S of the item before has been computed
+  auto load_q = [&](const Work& w, int64_t row) {
+    if (warp < warps_of(w) && r < C::kQRows) {
+      const uint4* src = reinterpret_cast<const uint4*>(p.q + row * D);
+      constexpr int kChunks = D / 8 / (kPair ? 2 : 1);  // 16-byte chunks of the row this thread writes
 #pragma unroll
-    for (int cc = 0; cc < kChunks; ++cc) {
-      const int c = half * kChunks + cc;
-      const uint4 v = valid ? src[c] : make_uint4(0u, 0u, 0u, 0u);
-      *reinterpret_cast<uint4*>(q_s + (c >> 3) * C::kQHalfBytes + r * 128 + (((c & 7) ^ (r & 7)) << 4)) = v;
+      for (int cc = 0; cc < kChunks; ++cc) {
+        const int c = half * kChunks + cc;
+        const uint4 v = row >= 0 ? src[c] : make_uint4(0u, 0u, 0u, 0u);
+        *reinterpret_cast<uint4*>(q_s + (c >> 3) * C::kQHalfBytes + r * 128 + (((c & 7) ^ (r & 7)) << 4)) = v;
+      }
+      fence_proxy_async_smem();
     }
-    fence_proxy_async_smem();
-  }
-  mbar_arrive(q_ready);
+    __syncwarp();
+    if (lane == 0) mbar_arrive(q_ready);
+  };
 
   // columns [32 k, 32 k + 32) of this thread's O lane
   auto o_load = [&](int k, float* o) { tmem_ld32(t_lane + kTmemO + k * 32, o); };
   auto o_store = [&](int k, const float* o) { tmem_st32(t_lane + kTmemO + k * 32, o); };
 
   const float sl2 = p.scale_log2;
-  float m_used = -1e30f, l = 0.f;  // l: this thread's share of the row sum
   bool ok = true;
-  for (int j = 0; j < n_tiles; ++j) {
-    const int s = j % C::kStages;
-    if (!__all_sync(0xffffffffu, mbar_wait(&s_full[j & 1], (j >> 1) & 1))) {
-      ok = false;
-      break;
-    }
-    tc_fence_after_sync();
-    // raw scores q.k of this thread's keys; the softmax works in the log2
-    // domain, x = s * sl2
-    float sc[kKpt];
-    static_assert(C::kKeys == 64, "64 keys per stage");
-    if constexpr (kPair) tmem_ld16x2_32<32>(t_lane + kTmemS + (j & 1) * C::kKeys, sc);
-    else tmem_ld64(t_lane + kTmemS + (j & 1) * C::kKeys, sc);
-    const int key0 = j * C::kKeys;
-    const int kbase = half * kKpt;  // this thread's first key within the stage
-    const int np = min(C::kPagesPerStage, n_pages - j * C::kPagesPerStage);
-    const int loaded = np * kPageTokens;
-    if (key0 + C::kKeys > n_valid_keys || loaded < C::kKeys) {
+  int64_t row = q_row(work);
+  load_q(work, row);
+  int g0 = 0;  // the item's first stage among the CTA's
+  for (int n = 0;; ++n) {
+    const bool valid = row >= 0;
+    const int n_sw = warps_of(work), n_swt = n_sw * 32, n_tiles = stages_of(work);
+    const int n_pages = work.item.n_pages, n_valid_keys = work.item.n_tokens;
+    float m_used = -1e30f, l = 0.f;  // l: this thread's share of the row sum
+    for (int j = 0; j < n_tiles; ++j) {
+      const int g = g0 + j, s = g % C::kStages;
+      if (!__all_sync(0xffffffffu, mbar_wait(&s_full[g & 1], (g >> 1) & 1))) {
+        ok = false;
+        break;
+      }
+      tc_fence_after_sync();
+      if (warp < n_sw) {
+        // raw scores q.k of this thread's keys; the softmax works in the log2
+        // domain, x = s * sl2
+        float sc[kKpt];
+        static_assert(C::kKeys == 64, "64 keys per stage");
+        if constexpr (kPair) tmem_ld16x2_32<32>(t_lane + kTmemS + (g & 1) * C::kKeys, sc);
+        else tmem_ld64(t_lane + kTmemS + (g & 1) * C::kKeys, sc);
+        const int key0 = j * C::kKeys;
+        const int kbase = half * kKpt;  // this thread's first key within the stage
+        const int np = min(C::kPagesPerStage, n_pages - j * C::kPagesPerStage);
+        const int loaded = np * kPageTokens;
+        if (key0 + C::kKeys > n_valid_keys || loaded < C::kKeys) {
 #pragma unroll
-      for (int c = 0; c < kKpt; ++c)
-        if (c >= min(loaded, n_valid_keys - key0) - kbase) sc[c] = -INFINITY;
-    }
-    // 8 independent chains of three-input max, then a tree (short dependency chains)
-    float mx8[8];
-#pragma unroll
-    for (int i = 0; i < 8; ++i) mx8[i] = fmaxf(sc[i], sc[8 + i]);
-#pragma unroll
-    for (int c = 16; c < kKpt; c += 16)
-#pragma unroll
-      for (int i = 0; i < 8; ++i) mx8[i] = fmax3(mx8[i], sc[c + i], sc[c + 8 + i]);
-    float mx = fmax3(fmax3(mx8[0], mx8[1], mx8[2]), fmax3(mx8[3], mx8[4], mx8[5]), fmaxf(mx8[6], mx8[7]));
-    if constexpr (kPair) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 16));
-    const float m_new = fmaxf(m_used, mx * sl2);  // sl2 > 0: max commutes with the scale
-    const bool need = valid && m_new > m_used + kRescaleThreshold;
-    if (__any_sync(0xffffffffu, need)) {
-      const float alpha = need ? ex2(m_used - m_new) : 1.f;
-      if (j > 0) {
-        // P_{j-1} V_{j-1} must have landed in O (P_j V_j cannot start before
-        // this thread's P_j, so the parity below is unambiguous)
-        if (!__all_sync(0xffffffffu, mbar_wait(o_ready, (j - 1) & 1))) {
-          ok = false;
-          break;
+          for (int c = 0; c < kKpt; ++c)
+            if (c >= min(loaded, n_valid_keys - key0) - kbase) sc[c] = -INFINITY;
         }
-        tc_fence_after_sync();
+        // 8 independent chains of three-input max, then a tree (short dependency chains)
+        float mx8[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) mx8[i] = fmaxf(sc[i], sc[8 + i]);
+#pragma unroll
+        for (int c = 16; c < kKpt; c += 16)
+#pragma unroll
+          for (int i = 0; i < 8; ++i) mx8[i] = fmax3(mx8[i], sc[c + i], sc[c + 8 + i]);
+        float mx = fmax3(fmax3(mx8[0], mx8[1], mx8[2]), fmax3(mx8[3], mx8[4], mx8[5]), fmaxf(mx8[6], mx8[7]));
+        if constexpr (kPair) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 16));
+        const float m_new = fmaxf(m_used, mx * sl2);  // sl2 > 0: max commutes with the scale
+        const bool need = valid && m_new > m_used + kRescaleThreshold;
+        if (__any_sync(0xffffffffu, need)) {
+          const float alpha = need ? ex2(m_used - m_new) : 1.f;
+          if (j > 0) {
+            // the P V before must have landed in O (this stage's cannot start
+            // before this thread's P, so the parity below is unambiguous)
+            if (!__all_sync(0xffffffffu, mbar_wait(o_ready, (g - 1) & 1))) {
+              ok = false;
+              break;
+            }
+            tc_fence_after_sync();
+#pragma unroll 1
+            for (int k = 0; k < D / 32; ++k) {
+              float o[32];
+              o_load(k, o);
+#pragma unroll
+              for (int i = 0; i < 32; ++i) o[i] *= alpha;
+              o_store(k, o);
+            }
+          }
+          l *= alpha;
+          if (need) m_used = m_new;
+        }
+        uint8_t* kslot = k_slot(s);  // narrow: S_j has been consumed, P_j goes over K_j
+        if constexpr (kWide) {
+          // P_hi, P_lo of keys [16 k, 16 k + 16) over the 16 TMEM columns of their
+          // scores (all read above).  The store is warp-wide: rows past the
+          // item's take 2^-inf = 0.
+          const uint32_t p_tm = t_lane + kTmemS + (g & 1) * C::kKeys;
+          const float mo = valid ? m_used : INFINITY;
+          const float2 scale2 = make_float2(sl2, sl2), neg_m2 = make_float2(-mo, -mo);
+          float2 rs[4] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+#pragma unroll
+          for (int kq = 0; kq < C::kKeys / 16; ++kq) {
+            uint32_t pk[16];
+#pragma unroll
+            for (int c = 0; c < 16; c += 2)
+              prob_pair(sc[kq * 16 + c], sc[kq * 16 + c + 1], scale2, neg_m2, &rs[(c >> 1) & 3], &pk[c / 2],
+                        &pk[8 + c / 2]);
+            tmem_st16u_nowait(p_tm + kq * 16, pk);
+          }
+          tmem_wait_st();
+          const float2 sum = __fadd2_rn(__fadd2_rn(rs[0], rs[1]), __fadd2_rn(rs[2], rs[3]));
+          l += sum.x + sum.y;
+        } else if (valid) {
+          uint32_t pk[kKpt / 2];
+          uint32_t pl[kKpt / 2];
+          const float2 scale2 = make_float2(sl2, sl2), neg_m2 = make_float2(-m_used, -m_used);
+          float2 rs[4] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+#pragma unroll
+          for (int c = 0; c < kKpt; c += 2)
+            prob_pair(sc[c], sc[c + 1], scale2, neg_m2, &rs[(c >> 1) & 3], &pk[c / 2], &pl[c / 2]);
+          const float2 sum = __fadd2_rn(__fadd2_rn(rs[0], rs[1]), __fadd2_rn(rs[2], rs[3]));
+          l += sum.x + sum.y;
+          // A rows of P_hi and P_lo: 32 w + t and 32 w + 16 + t (both = t mod 8)
+          const int a_hi = warp * 32 + (lane & 15);
+#pragma unroll
+          for (int cc = 0; cc < kKpt / 8; ++cc) {
+            const int c = half * (kKpt / 8) + cc;  // 16-byte chunk of the P row (8 keys)
+            const uint32_t off = a_hi * 128 + ((c ^ (a_hi & 7)) << 4);
+            *reinterpret_cast<uint4*>(kslot + off) = make_uint4(pk[4 * cc], pk[4 * cc + 1], pk[4 * cc + 2], pk[4 * cc + 3]);
+            *reinterpret_cast<uint4*>(kslot + 16 * 128 + off) =
+                make_uint4(pl[4 * cc], pl[4 * cc + 1], pl[4 * cc + 2], pl[4 * cc + 3]);
+          }
+        }
+        if (key0 + C::kKeys > n_valid_keys || loaded < C::kKeys) {
+          // zero the V rows of keys that are not valid, once V_j has landed
+          // (narrow: with K_j, from which S_j was computed)
+          const int sv = g % C::kVStages;
+          if (!__all_sync(0xffffffffu, C::kSplitKV ? mbar_wait(&v_full[sv], (g / C::kVStages) & 1)
+                                                   : mbar_wait(&full[s], (g / C::kStages) & 1))) {
+            ok = false;
+            break;
+          }
+          uint8_t* vslot = v_slot(sv);
+          for (int t = threadIdx.x; t < C::kKeys * C::kHalves; t += n_swt) {
+            const int c = t % C::kKeys, h = t / C::kKeys;
+            if (c >= loaded || key0 + c >= n_valid_keys) {
+#pragma unroll
+              for (int x = 0; x < 8; ++x)
+                *reinterpret_cast<uint4*>(vslot + h * C::kKVHalfBytes + c * 128 + x * 16) = make_uint4(0u, 0u, 0u, 0u);
+            }
+          }
+        }
+        fence_proxy_async_smem();
+      }
+      tc_fence_before_sync();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&p_full[g & 1]);
+    }
+    if (!ok) break;
+    g0 += n_tiles;
+    // the next item's Q goes in before this one's results come out: its S
+    // (every S of this item has been computed) runs meanwhile.  Its first P V
+    // waits for this thread's P, behind the results.
+    Work next;
+    int64_t next_row = -1;
+    const bool more = kPersist && next_work(n, &next, &ok, false);
+    if (!ok) break;
+    if (more) {
+      next_row = q_row(next);
+      load_q(next, next_row);
+    }
+    if (warp < n_sw) {
+      // the last P V (not o_ready, whose phases this thread may be two behind)
+      if (!__all_sync(0xffffffffu, mbar_wait(o_final, n & 1))) {
+        ok = false;
+        break;
+      }
+      tc_fence_after_sync();
+      if constexpr (kPair) l += __shfl_xor_sync(0xffffffffu, l, 16);  // the row's full sum
+      const float inv = 1.f / l;
+      float* dst = nullptr;
+      float* dst_lse = nullptr;
+      if (valid) {
+        const int64_t idx = row * p.max_splits + work.item.split;
+        dst = p.out_o + idx * D;
+        if (half == 0) dst_lse = p.out_lse + idx;
+      }
+      if constexpr (kPair) {
+        // O = O_hi + O_lo: thread t writes columns [0, D/2) of the row, thread
+        // t + 16 columns [D/2, D); one shuffle per column pair swaps the halves
+        // each needs from the other's lane
+#pragma unroll 1
+        for (int k = 0; k < D / 64; ++k) {
+          float a[32], b[32];
+          o_load(k, a);           // columns [32 k, 32 k + 32)
+          o_load(k + D / 64, b);  // columns [D/2 + 32 k, D/2 + 32 k + 32)
+#pragma unroll
+          for (int i = 0; i < 32; ++i) {
+            const float other = __shfl_xor_sync(0xffffffffu, half ? a[i] : b[i], 16);
+            a[i] = (half ? b[i] : a[i]) + other;
+          }
+          if (dst) {
+            float* d = dst + half * (D / 2) + k * 32;
+#pragma unroll
+            for (int i = 0; i < 32; i += 4)
+              *reinterpret_cast<float4*>(d + i) = make_float4(a[i] * inv, a[i + 1] * inv, a[i + 2] * inv, a[i + 3] * inv);
+          }
+        }
+      } else {
 #pragma unroll 1
         for (int k = 0; k < D / 32; ++k) {
           float o[32];
           o_load(k, o);
+          if (dst) {
 #pragma unroll
-          for (int i = 0; i < 32; ++i) o[i] *= alpha;
-          o_store(k, o);
+            for (int i = 0; i < 32; i += 4)
+              *reinterpret_cast<float4*>(dst + k * 32 + i) =
+                  make_float4(o[i] * inv, o[i + 1] * inv, o[i + 2] * inv, o[i + 3] * inv);
+          }
         }
       }
-      l *= alpha;
-      if (need) m_used = m_new;
+      if (dst_lse) *dst_lse = (m_used + log2f(l)) * kLn2;
     }
-    uint8_t* kslot = k_slot(s);  // narrow: S_j has been consumed, P_j goes over K_j
-    if constexpr (kWide) {
-      // P_hi, P_lo of keys [16 k, 16 k + 16) over the 16 TMEM columns of their
-      // scores (all read above).  The store is warp-wide: rows past the
-      // item's take 2^-inf = 0.
-      const uint32_t p_tm = t_lane + kTmemS + (j & 1) * C::kKeys;
-      const float mo = valid ? m_used : INFINITY;
-      const float2 scale2 = make_float2(sl2, sl2), neg_m2 = make_float2(-mo, -mo);
-      float2 rs[4] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
-#pragma unroll
-      for (int kq = 0; kq < C::kKeys / 16; ++kq) {
-        uint32_t pk[16];
-#pragma unroll
-        for (int c = 0; c < 16; c += 2)
-          prob_pair(sc[kq * 16 + c], sc[kq * 16 + c + 1], scale2, neg_m2, &rs[(c >> 1) & 3], &pk[c / 2],
-                    &pk[8 + c / 2]);
-        tmem_st16u_nowait(p_tm + kq * 16, pk);
-      }
-      tmem_wait_st();
-      const float2 sum = __fadd2_rn(__fadd2_rn(rs[0], rs[1]), __fadd2_rn(rs[2], rs[3]));
-      l += sum.x + sum.y;
-    } else if (valid) {
-      uint32_t pk[kKpt / 2];
-      uint32_t pl[kKpt / 2];
-      const float2 scale2 = make_float2(sl2, sl2), neg_m2 = make_float2(-m_used, -m_used);
-      float2 rs[4] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
-#pragma unroll
-      for (int c = 0; c < kKpt; c += 2)
-        prob_pair(sc[c], sc[c + 1], scale2, neg_m2, &rs[(c >> 1) & 3], &pk[c / 2], &pl[c / 2]);
-      const float2 sum = __fadd2_rn(__fadd2_rn(rs[0], rs[1]), __fadd2_rn(rs[2], rs[3]));
-      l += sum.x + sum.y;
-      // A rows of P_hi and P_lo: 32 w + t and 32 w + 16 + t (both = t mod 8)
-      const int a_hi = warp * 32 + (lane & 15);
-#pragma unroll
-      for (int cc = 0; cc < kKpt / 8; ++cc) {
-        const int c = half * (kKpt / 8) + cc;  // 16-byte chunk of the P row (8 keys)
-        const uint32_t off = a_hi * 128 + ((c ^ (a_hi & 7)) << 4);
-        *reinterpret_cast<uint4*>(kslot + off) = make_uint4(pk[4 * cc], pk[4 * cc + 1], pk[4 * cc + 2], pk[4 * cc + 3]);
-        *reinterpret_cast<uint4*>(kslot + 16 * 128 + off) =
-            make_uint4(pl[4 * cc], pl[4 * cc + 1], pl[4 * cc + 2], pl[4 * cc + 3]);
-      }
-    }
-    if (key0 + C::kKeys > n_valid_keys || loaded < C::kKeys) {
-      // zero the V rows of keys that are not valid, once V_j has landed
-      // (narrow: with K_j, from which S_j was computed)
-      const int sv = j % C::kVStages;
-      if (!__all_sync(0xffffffffu, C::kSplitKV ? mbar_wait(&v_full[sv], (j / C::kVStages) & 1)
-                                               : mbar_wait(&full[s], (j / C::kStages) & 1))) {
-        ok = false;
-        break;
-      }
-      uint8_t* vslot = v_slot(sv);
-      for (int t = tid; t < C::kKeys * C::kHalves; t += n_swt) {
-        const int c = t % C::kKeys, h = t / C::kKeys;
-        if (c >= loaded || key0 + c >= n_valid_keys) {
-#pragma unroll
-          for (int x = 0; x < 8; ++x)
-            *reinterpret_cast<uint4*>(vslot + h * C::kKVHalfBytes + c * 128 + x * 16) = make_uint4(0u, 0u, 0u, 0u);
-        }
-      }
-    }
-    fence_proxy_async_smem();
-    tc_fence_before_sync();
-    mbar_arrive(&p_full[j & 1]);
+    if (!more) break;
+    work = next;
+    row = next_row;
   }
-  if (ok) ok = __all_sync(0xffffffffu, mbar_wait(o_final, 0));
-  tc_fence_after_sync();
-  if (ok) {
-    if constexpr (kPair) l += __shfl_xor_sync(0xffffffffu, l, 16);  // the row's full sum
-    const float inv = 1.f / l;
-    float* dst = nullptr;
-    float* dst_lse = nullptr;
-    if (valid) {
-      const int64_t idx = (((int64_t)layer * p.n_rows_q + qrow) * p.Hq + head) * p.max_splits + item.split;
-      dst = p.out_o + idx * D;
-      if (half == 0) dst_lse = p.out_lse + idx;
-    }
-    if constexpr (kPair) {
-      // O = O_hi + O_lo: thread t writes columns [0, D/2) of the row, thread
-      // t + 16 columns [D/2, D); one shuffle per column pair swaps the halves
-      // each needs from the other's lane
-#pragma unroll 1
-      for (int k = 0; k < D / 64; ++k) {
-        float a[32], b[32];
-        o_load(k, a);           // columns [32 k, 32 k + 32)
-        o_load(k + D / 64, b);  // columns [D/2 + 32 k, D/2 + 32 k + 32)
-#pragma unroll
-        for (int i = 0; i < 32; ++i) {
-          const float other = __shfl_xor_sync(0xffffffffu, half ? a[i] : b[i], 16);
-          a[i] = (half ? b[i] : a[i]) + other;
-        }
-        if (dst) {
-          float* d = dst + half * (D / 2) + k * 32;
-#pragma unroll
-          for (int i = 0; i < 32; i += 4)
-            *reinterpret_cast<float4*>(d + i) = make_float4(a[i] * inv, a[i + 1] * inv, a[i + 2] * inv, a[i + 3] * inv);
-        }
-      }
-    } else {
-#pragma unroll 1
-      for (int k = 0; k < D / 32; ++k) {
-        float o[32];
-        o_load(k, o);
-        if (dst) {
-#pragma unroll
-          for (int i = 0; i < 32; i += 4)
-            *reinterpret_cast<float4*>(dst + k * 32 + i) =
-                make_float4(o[i] * inv, o[i + 1] * inv, o[i + 2] * inv, o[i + 3] * inv);
-        }
-      }
-    }
-    if (dst_lse) *dst_lse = (m_used + log2f(l)) * kLn2;
-  } else if (lane == 0) {
-    atomicCAS(p.status, 0, kDevTimeout);
-  }
+  if (!ok && lane == 0) atomicCAS(p.status, 0, kDevTimeout);
   tc_fence_before_sync();
-  named_barrier_sync(1, n_swt + 32);
+  named_barrier_sync(1, n_part * 32 + 32);
 }
 
-template <int D, bool kWide, bool kElect>
+template <int D, bool kWide, bool kElect, bool kPersist>
 cudaError_t launch_tc_t(const CUtensorMap& km, const CUtensorMap& vm, const AttnParams& p,
-                        const InlineDecodePlan& inl, int n_ctas, cudaStream_t s) {
+                        const InlineDecodePlan& inl, int n_ctas, int dev, cudaStream_t s) {
   using C = TcCfg<D, kWide>;
   // the shared-memory opt-in is a per-device function attribute
   static bool configured[kMaxDevices] = {};
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return e;
-  if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
   if (!configured[dev]) {
-    e = cudaFuncSetAttribute(attend_tc_kernel<D, kWide, kElect>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             C::kSmemBytes);
+    const cudaError_t e = cudaFuncSetAttribute(attend_tc_kernel<D, kWide, kElect, kPersist>,
+                                               cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmemBytes);
     if (e != cudaSuccess) return e;
     configured[dev] = true;
   }
   dim3 grid(n_ctas, p.Hkv, p.L);
-  return launch_chained(attend_tc_kernel<D, kWide, kElect>, grid, dim3(kThreads), C::kSmemBytes, s, km, vm, p,
-                        inl);
+  return launch_chained(attend_tc_kernel<D, kWide, kElect, kPersist>, grid, dim3(kThreads), C::kSmemBytes, s, km, vm,
+                        p, inl);
+}
+
+// SMs of the current device, kept per device.
+cudaError_t current_device(int* dev, int* sms) {
+  static int sms_of[kMaxDevices] = {};
+  cudaError_t e = cudaGetDevice(dev);
+  if (e != cudaSuccess) return e;
+  if (*dev < 0 || *dev >= kMaxDevices) return cudaErrorInvalidDevice;
+  if (!sms_of[*dev]) {
+    e = cudaDeviceGetAttribute(&sms_of[*dev], cudaDevAttrMultiProcessorCount, *dev);
+    if (e != cudaSuccess) return e;
+  }
+  *sms = sms_of[*dev];
+  return cudaSuccess;
+}
+
+// The kernel's form for a launch: CTAs that take over further items where there
+// is more than one wave of them (two CTAs per SM), the elected MMA issue for a
+// narrow launch of one wave or so whose pages stay in L2.  A single wave gains
+// nothing from taking over (9 branches, one layer: 25.7 us without, 26.6 with),
+// nor do narrow items beside large tiles (24 branches: 313 and 319).
+template <int D>
+cudaError_t launch_decode_t(const CUtensorMap& km, const CUtensorMap& vm, const AttnParams& p,
+                            const InlineDecodePlan& ip, int n_items, bool wide, cudaStream_t s) {
+  int dev = 0, sms = 0;
+  const cudaError_t e = current_device(&dev, &sms);
+  if (e != cudaSuccess) return e;
+  const bool waves = (int64_t)n_items * p.Hkv * p.L > 2 * (int64_t)sms;
+  if (wide)
+    return waves ? launch_tc_t<D, true, false, true>(km, vm, p, ip, n_items, dev, s)
+                 : launch_tc_t<D, true, false, false>(km, vm, p, ip, n_items, dev, s);
+  if (p.keep_l2) return launch_tc_t<D, false, true, false>(km, vm, p, ip, n_items, dev, s);
+  return waves && !p.beside_prev ? launch_tc_t<D, false, false, true>(km, vm, p, ip, n_items, dev, s)
+                                 : launch_tc_t<D, false, false, false>(km, vm, p, ip, n_items, dev, s);
 }
 
 template <int D>
 int decode_ctas_per_sm_t() {
   using C = TcCfg<D, false>;
-  if (cudaFuncSetAttribute(attend_tc_kernel<D, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  if (cudaFuncSetAttribute(attend_tc_kernel<D, false, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            C::kSmemBytes) != cudaSuccess)
     return 0;
   int n = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, attend_tc_kernel<D, false, false>, kThreads, C::kSmemBytes) !=
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, attend_tc_kernel<D, false, false, false>, kThreads, C::kSmemBytes) !=
       cudaSuccess)
     return 0;
   return n < 2 ? n : 2;  // two CTAs' TMEM (2 x 256 columns) fill an SM
@@ -748,18 +868,8 @@ cudaError_t launch_decode_tc(const CUtensorMap& km, const CUtensorMap& vm, const
   static const InlineDecodePlan kNone{};
   const InlineDecodePlan& ip = inl ? *inl : kNone;
   if (n_items <= 0) return cudaSuccess;
-  // the narrow tile of a launch whose pages stay in L2 takes the elected issue
-  const bool elect = !wide && p.keep_l2;
-  if (D == 128) {
-    if (wide) return launch_tc_t<128, true, false>(km, vm, p, ip, n_items, s);
-    return elect ? launch_tc_t<128, false, true>(km, vm, p, ip, n_items, s)
-                 : launch_tc_t<128, false, false>(km, vm, p, ip, n_items, s);
-  }
-  if (D == 64) {
-    if (wide) return launch_tc_t<64, true, false>(km, vm, p, ip, n_items, s);
-    return elect ? launch_tc_t<64, false, true>(km, vm, p, ip, n_items, s)
-                 : launch_tc_t<64, false, false>(km, vm, p, ip, n_items, s);
-  }
+  if (D == 128) return launch_decode_t<128>(km, vm, p, ip, n_items, wide, s);
+  if (D == 64) return launch_decode_t<64>(km, vm, p, ip, n_items, wide, s);
   return cudaErrorInvalidValue;
 }
 

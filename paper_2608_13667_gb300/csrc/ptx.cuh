@@ -409,4 +409,30 @@ __device__ __forceinline__ float4 ld_cluster_f4(uint32_t saddr, uint32_t cta) {
   return v;
 }
 
+// Cluster launch control: ask for a CTA of this grid that has not started.  The
+// 16-byte answer lands in `resp` (16-byte aligned) and completes on `bar` (tx
+// bytes).  Not to be asked again after an answer without a CTA.
+__device__ __forceinline__ void clc_try_cancel(void* resp, uint64_t* bar) {
+  asm volatile("clusterlaunchcontrol.try_cancel.async.shared::cta.mbarrier::complete_tx::bytes.b128 [%0], [%1];" ::"r"(
+                   smem_addr(resp)),
+               "r"(smem_addr(bar))
+               : "memory");
+}
+
+// The answer: whether a CTA was taken over, and its coordinates.
+__device__ __forceinline__ bool clc_answer(const void* resp, uint32_t* x, uint32_t* y, uint32_t* z) {
+  uint32_t ok;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t.reg .b128 r;\n\t"
+      "ld.shared.b128 r, [%4];\n\t"
+      "clusterlaunchcontrol.query_cancel.is_canceled.pred.b128 p, r;\n\t"
+      "selp.u32 %3, 1, 0, p;\n\t"
+      "mov.u32 %0, 0;\n\tmov.u32 %1, 0;\n\tmov.u32 %2, 0;\n\t"
+      "@p clusterlaunchcontrol.query_cancel.get_first_ctaid.v4.b32.b128 {%0, %1, %2, _}, r;\n\t}"
+      : "=&r"(*x), "=&r"(*y), "=&r"(*z), "=&r"(ok)
+      : "r"(smem_addr(resp))
+      : "memory");
+  return ok != 0;
+}
+
 }  // namespace st

@@ -37,3 +37,45 @@ def test_stage_counts_around_the_ring(stlib, D, stages, n_aux):
 @pytest.mark.parametrize("L", [19, 20])      # 2432 and 2560 rows: four warps a row, one warp a row
 def test_combine_forms(stlib, D, L):
     _decode(D, 32, 8, L, 16 * 16 * 9, 3, 20, max_splits=32, layers=(0, L - 1))
+
+
+@pytest.mark.parametrize("D,Hq,Hkv", [(128, 32, 8), (64, 32, 8), (128, 64, 4)])
+def test_items_of_many_shapes_taken_over(stlib, D, Hq, Hkv):
+    """More than one wave of CTAs, so that each takes over further items: runs
+    of one page to many, of one branch to a whole group (one to four softmax
+    warps), short last pages, and groups on the wide tile."""
+    L = 24 if D == 64 else 12
+    w = Workload(name=f"taken_{D}_{Hq}_{Hkv}", n_layers=L, n_q_heads=Hq, n_kv_heads=Hkv, head_dim=D, n_blocks=2048,
+                 seed=62)
+    run = Run(w, max_seqs=64, max_decode_branches=48, max_splits=16)
+    rids = []
+    for g, (prefix, n_aux) in enumerate(((2000, 4), (640, 15), (5000, 1), (330, 12))):
+        m = run.create()
+        run.append([m], prefix, ("prefix", g))
+        family = [m] + run.fork(m, n_aux)
+        for i, r in enumerate(family):
+            if (i + g) % 3:
+                run.append([r], 1 + 13 * i, ("suffix", g, i))
+        rids += family
+    for i, n in enumerate((1, 15, 64, 65, 300, 1100)):
+        rids.append(run.create())
+        run.append([rids[-1]], n, ("single", i))
+    assert len(run.pool.decode_plan([run.handle[r] for r in rids])[0]) * Hkv * L > 2 * 304
+    for step in range(2):     # the rings and the slots start anew with every launch
+        q, o, lse = run.decode(rids, ("q", step))
+        run.pool.sync()
+        for layer in (0, L - 1):
+            o_ref, l_ref = run.oracle_decode(rids, q, layer)
+            compare(o[layer], lse[layer], o_ref, l_ref, f"step {step} layer {layer}")
+    # the rows of a step are stored by the items that are taken over
+    from workloads import kv_rows, queries
+    k, v = kv_rows(w, ("new",), len(rids), device="cuda")
+    q = queries(w, ("newq",), len(rids), device="cuda")
+    o, lse = run.pool.decode_step([run.handle[r] for r in rids], k, v, q)
+    run.pool.sync()
+    run.ref.append(rids, 1)
+    run.sizes[("new",)] = len(rids)
+    for i, r in enumerate(rids):
+        run.hist[r].append((("new",), i, 1))
+    o_ref, l_ref = run.oracle_decode(rids, q, L - 1)
+    compare(o[L - 1], lse[L - 1], o_ref, l_ref, "step with new rows")
