@@ -159,9 +159,31 @@ __global__ void __launch_bounds__(kThreads, 1)
   const int G = p.G;
 
   // Launched as a programmatic dependent of the kernel before it in the
-  // stream; the tensor-memory allocation touches no global memory, every
-  // global access comes after the wait.
+  // stream; the tensor-memory allocation and the barriers touch no global
+  // memory, every global access comes after the wait.
   if (warp == kMmaWarp) tmem_alloc(tmem_slot, kTmemCols);
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < kKS; ++s) {
+      mbar_init(&k_full[s], 1);
+      mbar_init(&k_empty[s], 1);
+    }
+    for (int s = 0; s < kVS; ++s) {
+      mbar_init(&v_full[s], 1);
+      mbar_init(&v_empty[s], 1);
+    }
+    for (int t = 0; t < 2; ++t) {
+      mbar_init(&s_full[t], 1);
+      mbar_init(&p_full[2 * t], kTileRows);
+      mbar_init(&p_full[2 * t + 1], kTileRows);
+    }
+    mbar_init(o_final, 1);
+    mbar_init(q_ready, kSoftThreads);
+    fence_mbar_init();
+  }
+  tc_fence_before_sync();
+  __syncthreads();
+  tc_fence_after_sync();
+  const uint32_t tmem = *tmem_slot;
   griddep_wait();
   griddep_launch_dependents();
   // one merge: its row tiles, the last ones (most keys) first; a batch: one
@@ -202,15 +224,16 @@ __global__ void __launch_bounds__(kThreads, 1)
   const int all_tiles = (n_pages + kPagesPerStage - 1) / kPagesPerStage;
   const int n_parts = kDecode ? 1 : merge_parts(all_tiles, cluster);
   if (rank >= n_parts) {  // a tile with fewer parts than the launch's clusters: nothing left for this CTA
-    __syncthreads();
-    if (warp == kMmaWarp) tmem_dealloc(*tmem_slot, kTmemCols);
+    if (warp == kMmaWarp) tmem_dealloc(tmem, kTmemCols);
     if (n_parts > 1) {  // the barriers of the exchange below count every CTA of the cluster
       cluster_sync();
       cluster_sync();
     }
     return;
   }
-  const int j0 = rank * all_tiles / n_parts, j1 = (rank + 1) * all_tiles / n_parts;
+  // (the longer parts first: the last one has the stages at the causal limit,
+  // whose masks cost it another microsecond or two)
+  const int j0 = (rank * all_tiles + n_parts - 1) / n_parts, j1 = ((rank + 1) * all_tiles + n_parts - 1) / n_parts;
   const int n_tiles = j1 - j0;
   const int key_base = j0 * kKeys;
   page_begin += j0 * kPagesPerStage;
@@ -218,28 +241,6 @@ __global__ void __launch_bounds__(kThreads, 1)
   // at most 128 rows: both tiles hold them, tile A takes the even stages and tile B the odd ones
   const bool dual = !kDecode && n_rows <= kTileRows;
 
-  if (threadIdx.x == 0) {
-    for (int s = 0; s < kKS; ++s) {
-      mbar_init(&k_full[s], 1);
-      mbar_init(&k_empty[s], 1);
-    }
-    for (int s = 0; s < kVS; ++s) {
-      mbar_init(&v_full[s], 1);
-      mbar_init(&v_empty[s], 1);
-    }
-    for (int t = 0; t < 2; ++t) {
-      mbar_init(&s_full[t], 1);
-      mbar_init(&p_full[2 * t], kTileRows);
-      mbar_init(&p_full[2 * t + 1], kTileRows);
-    }
-    mbar_init(o_final, 1);
-    mbar_init(q_ready, kSoftThreads);
-    fence_mbar_init();
-  }
-  tc_fence_before_sync();
-  __syncthreads();
-  tc_fence_after_sync();
-  const uint32_t tmem = *tmem_slot;
 
   // ---- loaders -------------------------------------------------------------------
   // (hold_loads, a test hook: nothing arrives, the other roles' waits run out)
