@@ -218,7 +218,7 @@ __global__ void __launch_bounds__(kThreads, 2)
   // kernel in the stream (the one that wrote the pages): the tensor-memory
   // allocation, and all of the set-up when the item is in the parameters.
   if (warp == kMmaWarp) tmem_alloc(tmem_slot, kTmemCols);
-  const bool beside = !kPersist && p.beside_prev;
+  const bool beside = !kWide && p.beside_prev;
   if (p.items && !beside) griddep_wait();
 
   // ---- what this CTA reads and for whom ------------------------------------------
@@ -543,9 +543,11 @@ __global__ void __launch_bounds__(kThreads, 2)
     named_barrier_sync(1, n_part * 32 + 32);
     tc_fence_after_sync();
     tmem_dealloc(tmem, kTmemCols);
-    // beside_prev: this grid is complete only once the one before it is (not
-    // with kPersist, where this CTA may be taken over before it starts)
-    if (beside && blockIdx.x == gridDim.x - 1 && blockIdx.y == gridDim.y - 1 && blockIdx.z == gridDim.z - 1)
+    // beside_prev: this grid is complete only once the one before it is (with
+    // kPersist the last CTA may be taken over before it starts: all wait, when
+    // there is nothing left to run)
+    if (beside && (kPersist || (blockIdx.x == gridDim.x - 1 && blockIdx.y == gridDim.y - 1 &&
+                                blockIdx.z == gridDim.z - 1)))
       griddep_wait();
     return;
   }
@@ -832,7 +834,10 @@ cudaError_t current_device(int* dev, int* sms) {
 // is more than one wave of them (two CTAs per SM), the elected MMA issue for a
 // narrow launch of one wave or so whose pages stay in L2.  A single wave gains
 // nothing from taking over (9 branches, one layer: 25.7 us without, 26.6 with),
-// nor do narrow items beside large tiles (24 branches: 313 and 319).
+// nor do a few waves of narrow items beside large tiles (24 branches: 313 and
+// 319), but many do: beyond four waves they are mostly runs of a page or two
+// (13 groups of 27 branches, D 64: 149 us without, 119 with; 14 groups of 9,
+// 4 layers: 342 and 321).
 template <int D>
 cudaError_t launch_decode_t(const CUtensorMap& km, const CUtensorMap& vm, const AttnParams& p,
                             const InlineDecodePlan& ip, int n_items, bool wide, cudaStream_t s) {
@@ -844,8 +849,9 @@ cudaError_t launch_decode_t(const CUtensorMap& km, const CUtensorMap& vm, const 
     return waves ? launch_tc_t<D, true, false, true>(km, vm, p, ip, n_items, dev, s)
                  : launch_tc_t<D, true, false, false>(km, vm, p, ip, n_items, dev, s);
   if (p.keep_l2) return launch_tc_t<D, false, true, false>(km, vm, p, ip, n_items, dev, s);
-  return waves && !p.beside_prev ? launch_tc_t<D, false, false, true>(km, vm, p, ip, n_items, dev, s)
-                                 : launch_tc_t<D, false, false, false>(km, vm, p, ip, n_items, dev, s);
+  const bool many = (int64_t)n_items * p.Hkv * p.L > 8 * (int64_t)sms;
+  return (p.beside_prev ? many : waves) ? launch_tc_t<D, false, false, true>(km, vm, p, ip, n_items, dev, s)
+                                        : launch_tc_t<D, false, false, false>(km, vm, p, ip, n_items, dev, s);
 }
 
 template <int D>

@@ -79,3 +79,26 @@ def test_items_of_many_shapes_taken_over(stlib, D, Hq, Hkv):
         run.hist[r].append((("new",), i, 1))
     o_ref, l_ref = run.oracle_decode(rids, q, L - 1)
     compare(o[L - 1], lse[L - 1], o_ref, l_ref, "step with new rows")
+
+
+def test_many_short_items_beside_a_wide_tile(stlib):
+    """Groups on the wide tile with more than four waves of one-page items
+    beside them: those take over from one another and all wait for the tiles."""
+    L = 16
+    w = Workload(name="beside_many", n_layers=L, n_q_heads=32, n_kv_heads=8, head_dim=64, n_blocks=1024, seed=63)
+    run = Run(w, max_seqs=64, max_decode_branches=40, max_splits=16)
+    rids = []
+    for g, n_aux in enumerate((19, 16)):      # 80 and 68 stacked rows
+        m = run.create()
+        run.append([m], 2600 + 16 * g, ("prefix", g))
+        family = [m] + run.fork(m, n_aux)
+        run.append(family, 3 + g, ("suffix", g))
+        rids += family
+    items, _, _ = run.pool.decode_plan([run.handle[r] for r in rids])
+    assert sum(1 for it in items if not it["flags"]) * 8 * L > 4 * 304
+    for step in range(2):
+        q, o, lse = run.decode(rids, ("q", step))
+        run.pool.sync()
+        for layer in (0, L - 1):
+            o_ref, l_ref = run.oracle_decode(rids, q, layer)
+            compare(o[layer], lse[layer], o_ref, l_ref, f"step {step} layer {layer}")
