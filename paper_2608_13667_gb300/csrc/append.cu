@@ -12,22 +12,15 @@ namespace st {
 
 namespace {
 
-// Entries of one run that a block of kTableThreads writes.
-constexpr int kTableThreads = 256;
-constexpr int kTableChunk = 4 * kTableThreads;
-
 // runs and values are in the pinned staging slot and read from there: a copy
 // to the device first is an operation of another engine, whose hand-overs
 // break the chain of dependent launches (with its 2 MiB slot copied whole it
 // took 12 us; the update itself takes 2).  A block's loads are in flight
 // together, since each is a round trip to the host's memory.
-__global__ void __launch_bounds__(kTableThreads)
-    table_update_kernel(int32_t* __restrict__ table, const TableRun* __restrict__ runs,
-                        const int32_t* __restrict__ values) {
-  griddep_wait();
-  griddep_launch_dependents();
-  const TableRun run = runs[blockIdx.x];
-  const int i0 = blockIdx.y * kTableChunk + threadIdx.x;
+__device__ __forceinline__ void table_chunk(int32_t* __restrict__ table, const TableRun* __restrict__ runs,
+                                            const int32_t* __restrict__ values, int r, int chunk) {
+  const TableRun run = runs[r];
+  const int i0 = chunk * kTableChunk + threadIdx.x;
   int32_t v[kTableChunk / kTableThreads];
 #pragma unroll
   for (int u = 0; u < kTableChunk / kTableThreads; ++u)
@@ -35,6 +28,14 @@ __global__ void __launch_bounds__(kTableThreads)
 #pragma unroll
   for (int u = 0; u < kTableChunk / kTableThreads; ++u)
     if (i0 + u * kTableThreads < run.count) table[run.dst + i0 + u * kTableThreads] = v[u];
+}
+
+__global__ void __launch_bounds__(kTableThreads)
+    table_update_kernel(int32_t* __restrict__ table, const TableRun* __restrict__ runs,
+                        const int32_t* __restrict__ values) {
+  griddep_wait();
+  griddep_launch_dependents();
+  table_chunk(table, runs, values, blockIdx.x, blockIdx.y);
 }
 
 // A plan from its pinned staging slot to the device, 16 bytes a thread.  A
@@ -50,20 +51,29 @@ __global__ void __launch_bounds__(256) plan_copy_kernel(uint4* __restrict__ dst,
 // One thread moves 16 bytes (8 bf16).  Index space: copy-on-write chunks
 // first (n_cow x L x Hkv x 16 rows x D/8, rows past the copy length idle),
 // then the appended rows in the input's own order [L][n_rows][Hkv][D/8];
-// row r belongs to the branch whose [row0, row0 + n) holds it.
+// row r belongs to the branch whose [row0, row0 + n) holds it.  A small append
+// that also changes the tables (new pages, or a fork's whole table) refreshes
+// them in its first blocks and takes its rows' pages from the parameters, one
+// launch and one hand-over less in the chain to the attention kernel (a merge
+// of 44 rows onto 23040, fork, merge and release: 49.3 us with the refresh in a
+// launch of its own, 47.5 without; a prompt of 17 rows 22.2 and 19.4).
 template <int D>
-__global__ void __launch_bounds__(256) append_kernel(const AppendParams p,
+__global__ void __launch_bounds__(kTableThreads) append_kernel(const AppendParams p,
                                                      const __grid_constant__ InlineAppendPlan inl) {
   griddep_wait();
   griddep_launch_dependents();
+  if ((int)blockIdx.x < p.n_table_blocks) {
+    table_chunk(p.table_out, p.runs, p.values, blockIdx.x / p.chunks_per_run, blockIdx.x % p.chunks_per_run);
+    return;
+  }
   const AppendBranch* branches = p.branches ? p.branches : inl.branches;
   const CowCopy* cows = p.cows ? p.cows : inl.cows;
   constexpr int kChunks = D / 8;
   const int64_t cow_total = (int64_t)p.n_cow * p.L * p.Hkv * kPageTokens * kChunks;
   const int64_t app_total = (int64_t)p.L * p.n_rows * p.Hkv * kChunks;
   const int64_t total = cow_total + app_total;
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += stride) {
+  const int64_t stride = (int64_t)(gridDim.x - p.n_table_blocks) * blockDim.x;
+  for (int64_t i = (int64_t)(blockIdx.x - p.n_table_blocks) * blockDim.x + threadIdx.x; i < total; i += stride) {
     if (i < cow_total) {
       int64_t x = i;
       const int c = (int)(x % kChunks); x /= kChunks;
@@ -102,7 +112,8 @@ __global__ void __launch_bounds__(256) append_kernel(const AppendParams p,
       }
       const AppendBranch br = branches[b];
       const int pos = br.start + (row - br.row0);
-      const int32_t blk = p.table[(int64_t)br.slot * p.max_pages + pos / kPageTokens];
+      const int32_t blk = p.n_table_blocks ? inl.pages[br.page0 + pos / kPageTokens - br.start / kPageTokens]
+                                           : p.table[(int64_t)br.slot * p.max_pages + pos / kPageTokens];
       if ((uint64_t)blk >= (uint64_t)p.n_blocks) {
         atomicCAS(p.status, 0, kDevBadIndex);
         continue;
@@ -148,9 +159,9 @@ cudaError_t launch_append(const AppendParams& p, const InlineAppendPlan* inl, in
   const int64_t total = (int64_t)p.n_cow * p.L * p.Hkv * kPageTokens * (D / 8) +
                         (int64_t)p.L * p.n_rows * p.Hkv * (D / 8);
   if (total == 0) return cudaSuccess;
-  const int grid = grid_for(total, 256);
-  if (D == 128) return launch_chained(append_kernel<128>, dim3(grid), dim3(256), 0, s, p, ip);
-  if (D == 64) return launch_chained(append_kernel<64>, dim3(grid), dim3(256), 0, s, p, ip);
+  const int grid = grid_for(total, kTableThreads) + p.n_table_blocks;
+  if (D == 128) return launch_chained(append_kernel<128>, dim3(grid), dim3(kTableThreads), 0, s, p, ip);
+  if (D == 64) return launch_chained(append_kernel<64>, dim3(grid), dim3(kTableThreads), 0, s, p, ip);
   return cudaErrorInvalidValue;
 }
 

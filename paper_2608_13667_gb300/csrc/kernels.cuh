@@ -40,6 +40,7 @@ struct AppendBranch {
   int32_t start;  // sequence length before this call
   int32_t row0;   // first of this branch's rows in the call's input
   int32_t n;      // rows appended to this branch
+  int32_t page0;  // with an inline page list: where the page of row `start` is in it
 };
 
 struct AppendParams {
@@ -55,6 +56,12 @@ struct AppendParams {
   int32_t n_cow, n_br, n_tok, L, Hkv, max_pages;
   int32_t n_rows;          // n_br * n_tok, or the sum of the branches' n
   int32_t ragged;          // 0: every branch takes n_tok rows (branch of row r is r / n_tok)
+  // a table refresh in the same launch (n_table_blocks > 0; the rows' pages
+  // then come from the inline list): runs and values in pinned host memory
+  const TableRun* runs;
+  const int32_t* values;
+  int32_t* table_out;
+  int32_t n_table_blocks, chunks_per_run;
 };
 
 // One unit of decode work: a run of pages of one block table, read for a set
@@ -144,10 +151,15 @@ struct InlineSplits {
 };
 constexpr int kInlineAppendBranches = 32;
 constexpr int kInlineCows = 32;
+constexpr int kInlinePages = 192;
 struct InlineAppendPlan {
   AppendBranch branches[kInlineAppendBranches];
   CowCopy cows[kInlineCows];
+  int32_t pages[kInlinePages];  // the pages of each branch's new rows
 };
+// Entries of one run that a block of a table refresh writes.
+constexpr int kTableThreads = 256;
+constexpr int kTableChunk = 4 * kTableThreads;
 
 // Programmatic dependent launch.  The small kernels of a decode step (table
 // update, append, decode partials, combine) are launched so that each may be

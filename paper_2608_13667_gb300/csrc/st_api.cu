@@ -291,7 +291,7 @@ st_status run_kernel(st_pool* P, int kid, double bytes, double flops, cudaStream
 // drop_plan.
 st_status acquire_plan(st_pool* P, Plan* plan, int* slot_out) {
   int i = P->stage_next;
-  while (P->stage_held & (1u << i)) i = (i + 1) % kStageSlots;  // at most two are ever held
+  while (P->stage_held & (1u << i)) i = (i + 1) % kStageSlots;  // at most three are ever held
   P->stage_next = (i + 1) % kStageSlots;
   if (P->stage_used[i]) CUDA_TRY(P, cudaEventSynchronize(P->stage_ev[i]));
   P->stage_held |= 1u << i;
@@ -334,48 +334,75 @@ size_t plan_bytes(std::initializer_list<size_t> parts) {
   return off;
 }
 
+// Block-table ranges the host has changed and the device has not seen.
+struct DirtyTables {
+  int runs = 0;
+  size_t values = 0;
+};
+
+DirtyTables dirty_tables(const BlockPool& bp, int first_slot = 0) {
+  DirtyTables d;
+  for (int i = first_slot; i < bp.max_seqs(); ++i) {
+    const SeqSlot& ss = bp.slot(i);
+    if (!ss.live || ss.dirty_hi <= ss.dirty_lo) continue;
+    ++d.runs;
+    d.values += (size_t)(ss.dirty_hi - ss.dirty_lo);
+  }
+  return d;
+}
+
+// Changed ranges written into a staging slot, from slot *slot on and as many as fit.
+struct TableRefresh {
+  const TableRun* runs = nullptr;  // device addresses
+  const int32_t* values = nullptr;
+  int n_runs = 0;
+  size_t n_values = 0, longest = 0;
+};
+
+TableRefresh stage_tables(st_pool* P, Plan* plan, int n_dirty, int* slot) {
+  BlockPool& bp = *P->pool;
+  // runs first (bounded count), then values
+  const int max_runs = std::min(n_dirty, 4096);
+  const TableRun* unused_runs;
+  TableRun* runs = plan->alloc<TableRun>(max_runs, &unused_runs);
+  const size_t vals_cap = (plan->cap - plan->off - 64) / sizeof(int32_t);
+  const int32_t* unused_vals;
+  int32_t* vals = plan->alloc<int32_t>(vals_cap, &unused_vals);
+  TableRefresh t;
+  t.runs = on_device(P, runs);
+  t.values = on_device(P, vals);
+  for (; *slot < bp.max_seqs() && t.n_runs < max_runs; ++*slot) {
+    SeqSlot& ss = bp.slot_mut(*slot);
+    if (!ss.live || ss.dirty_hi <= ss.dirty_lo) continue;
+    const size_t cnt = (size_t)(ss.dirty_hi - ss.dirty_lo);
+    const size_t room = vals_cap - t.n_values;
+    if (room == 0) break;
+    const size_t take = std::min(cnt, room);
+    runs[t.n_runs] = TableRun{(int64_t)*slot * bp.max_pages() + ss.dirty_lo, (int32_t)take, (int32_t)t.n_values};
+    std::memcpy(vals + t.n_values, ss.table.data() + ss.dirty_lo, take * sizeof(int32_t));
+    t.n_values += take;
+    t.longest = std::max(t.longest, take);
+    ++t.n_runs;
+    ss.dirty_lo += (int32_t)take;
+    if (ss.dirty_lo < ss.dirty_hi) break;  // slot only partly uploaded: continue it next round
+    ss.dirty_lo = ss.dirty_hi = 0;
+  }
+  return t;
+}
+
 // Refresh the device copy of every block-table range the host changed.
 st_status flush_tables(st_pool* P, cudaStream_t s) {
-  BlockPool& bp = *P->pool;
   int slot = 0;
-  const int n = bp.max_seqs();
-  while (slot < n) {
+  while (slot < P->pool->max_seqs()) {
+    const DirtyTables d = dirty_tables(*P->pool, slot);
+    if (d.runs == 0) return ST_OK;
     Plan plan;
     int ps;
-    int n_dirty = 0;
-    for (int i = slot; i < n; ++i)
-      if (bp.slot(i).live && bp.slot(i).dirty_hi > bp.slot(i).dirty_lo) ++n_dirty;
-    if (n_dirty == 0) return ST_OK;
     st_status st = acquire_plan(P, &plan, &ps);
     if (st != ST_OK) return st;
-    // runs first (bounded count), then values
-    const int max_runs = std::min(n_dirty, 4096);
-    const TableRun* unused_runs;
-    TableRun* runs = plan.alloc<TableRun>(max_runs, &unused_runs);
-    const size_t vals_cap = (plan.cap - plan.off - 64) / sizeof(int32_t);
-    const int32_t* unused_vals;
-    int32_t* vals = plan.alloc<int32_t>(vals_cap, &unused_vals);
-    int n_runs = 0;
-    size_t n_vals = 0, longest = 0;
-    for (; slot < n && n_runs < max_runs; ++slot) {
-      SeqSlot& ss = bp.slot_mut(slot);
-      if (!ss.live || ss.dirty_hi <= ss.dirty_lo) continue;
-      const size_t cnt = (size_t)(ss.dirty_hi - ss.dirty_lo);
-      const size_t room = vals_cap - n_vals;
-      if (room == 0) break;
-      const size_t take = std::min(cnt, room);
-      runs[n_runs] = TableRun{(int64_t)slot * bp.max_pages() + ss.dirty_lo, (int32_t)take, (int32_t)n_vals};
-      std::memcpy(vals + n_vals, ss.table.data() + ss.dirty_lo, take * sizeof(int32_t));
-      n_vals += take;
-      longest = std::max(longest, take);
-      ++n_runs;
-      ss.dirty_lo += (int32_t)take;
-      if (ss.dirty_lo < ss.dirty_hi) break;  // slot only partly uploaded: continue it next round
-      ss.dirty_lo = ss.dirty_hi = 0;
-    }
-    int32_t* tbl = P->d_tables;
-    st = run_kernel(P, kKTable, (double)n_vals * 8 + n_runs * 16, 0, s, [&] {
-      return launch_table_update(tbl, on_device(P, runs), on_device(P, vals), n_runs, (int)longest, s);
+    const TableRefresh t = stage_tables(P, &plan, d.runs, &slot);
+    st = run_kernel(P, kKTable, (double)t.n_values * 8 + t.n_runs * 16, 0, s, [&] {
+      return launch_table_update(P->d_tables, t.runs, t.values, t.n_runs, (int)t.longest, s);
     });
     if (st != ST_OK) return st;
     st = retire_plan(P, ps, s);
@@ -385,6 +412,11 @@ st_status flush_tables(st_pool* P, cudaStream_t s) {
 }
 
 bool aligned(const void* p, size_t a) { return ((uintptr_t)p % a) == 0; }
+
+// Pages that a branch's new rows are in.
+int32_t pages_of_rows(const AppendBranch& b) {
+  return b.n > 0 ? (b.start + b.n - 1) / kPageTokens - b.start / kPageTokens + 1 : 0;
+}
 
 // Validates and performs an append (shared by st_append_kv, st_merge and
 // st_prefill_batch).  Appends counts[i] rows to slots[i], in order (the same
@@ -434,7 +466,7 @@ st_status do_append_rows(st_pool* P, const int* slots, const int32_t* counts, in
   brs.resize(n_br);
   int32_t row0 = 0;
   for (int i = 0; i < n_br; ++i) {
-    brs[i] = AppendBranch{slots[i], (int32_t)bp.slot(slots[i]).len, row0, counts[i]};
+    brs[i] = AppendBranch{slots[i], (int32_t)bp.slot(slots[i]).len, row0, counts[i], 0};
     row0 += counts[i];
   }
   std::vector<CowEvent>& cows = P->app_cows;
@@ -446,15 +478,41 @@ st_status do_append_rows(st_pool* P, const int* slots, const int32_t* counts, in
   }
   if (P->meta_only || n_rows == 0) return ST_OK;
 
-  st_status st = flush_tables(P, s);
-  if (st != ST_OK) return poison(P, st);
-  if (deferred && cows.empty()) {
+  const bool defers = deferred && cows.empty();  // no append launch
+  const bool inline_plan = n_br <= kInlineAppendBranches && cows.size() <= (size_t)kInlineCows;
+  InlineAppendPlan inl;
+  // a small append refreshes the tables itself, its rows' pages in its parameters
+  size_t n_pages = 0;
+  for (int i = 0; i < n_br; ++i) n_pages += pages_of_rows(brs[i]);
+  const DirtyTables dirty = dirty_tables(bp);
+  const bool refreshes = !defers && inline_plan && dirty.runs > 0 && n_pages <= (size_t)kInlinePages &&
+                         plan_bytes({dirty.runs * sizeof(TableRun), dirty.values * sizeof(int32_t) + 64}) +
+                                 64 <= kStageSlotBytes && dirty.runs <= 4096;
+  st_status st = ST_OK;
+  int table_slot = -1;
+  TableRefresh refresh;
+  if (refreshes) {
+    int32_t at = 0;
+    for (int i = 0; i < n_br; ++i) {
+      brs[i].page0 = at;
+      const int32_t n = pages_of_rows(brs[i]);
+      std::memcpy(inl.pages + at, bp.slot(slots[i]).table.data() + brs[i].start / kPageTokens, n * sizeof(int32_t));
+      at += n;
+    }
+    Plan table_plan;
+    st = acquire_plan(P, &table_plan, &table_slot);
+    if (st != ST_OK) return poison(P, st);
+    int first = 0;
+    refresh = stage_tables(P, &table_plan, dirty.runs, &first);
+  } else {
+    st = flush_tables(P, s);
+    if (st != ST_OK) return poison(P, st);
+  }
+  if (defers) {
     drop_plan(P, ps);
     *deferred = true;
     return ST_OK;
   }
-  const bool inline_plan = n_br <= kInlineAppendBranches && cows.size() <= (size_t)kInlineCows;
-  InlineAppendPlan inl;
   const AppendBranch* d_br = nullptr;
   const CowCopy* d_cow = nullptr;
   if (inline_plan) {
@@ -491,6 +549,13 @@ st_status do_append_rows(st_pool* P, const int* slots, const int32_t* counts, in
   ap.max_pages = c.max_pages;
   ap.n_rows = (int32_t)n_rows;
   ap.ragged = uniform ? 0 : 1;
+  if (refreshes) {
+    ap.runs = refresh.runs;
+    ap.values = refresh.values;
+    ap.table_out = P->d_tables;
+    ap.chunks_per_run = (int32_t)((refresh.longest + kTableChunk - 1) / kTableChunk);
+    ap.n_table_blocks = refresh.n_runs * ap.chunks_per_run;
+  }
   // algorithmic: the new rows read and written once; the copy-on-write rows
   // are the bookkeeping's own traffic
   const double row_bytes = (double)c.n_layers * c.n_kv_heads * c.head_dim * 2 * 2;
@@ -498,8 +563,15 @@ st_status do_append_rows(st_pool* P, const int* slots, const int32_t* counts, in
   for (auto& e : cows) cow_rows += e.rows;
   st = run_kernel(P, kKAppend, row_bytes * (double)n_rows * 2, 0, s,
                   [&] { return launch_append(ap, inline_plan ? &inl : nullptr, c.head_dim, s); }, 1,
-                  row_bytes * cow_rows * 2);
-  if (st != ST_OK) return poison(P, st);
+                  row_bytes * cow_rows * 2 + (double)refresh.n_values * 8 + refresh.n_runs * 16);
+  if (st != ST_OK) {
+    if (table_slot >= 0) drop_plan(P, table_slot);
+    return poison(P, st);
+  }
+  if (table_slot >= 0) {
+    st = retire_plan(P, table_slot, s);
+    if (st != ST_OK) return poison(P, st);
+  }
   if (!inline_plan) {
     st = retire_plan(P, ps, s);
     if (st != ST_OK) return poison(P, st);
