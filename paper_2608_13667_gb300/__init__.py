@@ -435,7 +435,8 @@ def st_harvest(streams, lens, open_id, close_id, cap=5, stream=None):
     for t, name in ((streams, "streams"), (lens, "lens")):
         if t.dtype != torch.int32 or not t.is_cuda or not t.is_contiguous():
             raise ValueError(f"{name} must be a contiguous int32 CUDA tensor")
-    out_ids, out_src = torch.empty((2, n_br * stride), dtype=torch.int32, device=streams.device)
+    out_ids = torch.empty(n_br * stride, dtype=torch.int32, device=streams.device)
+    out_src = torch.empty_like(out_ids)
     atoms = torch.empty(n_br, dtype=torch.int32, device=streams.device)
     # the kernel writes the count to pinned host memory, so that reading it back
     # is a wait for the stream and no copy
@@ -450,7 +451,7 @@ def st_harvest(streams, lens, open_id, close_id, cap=5, stream=None):
     if not hasattr(stream, "synchronize"):
         stream = torch.cuda.ExternalStream(stream.cuda_stream, device=streams.device)
     stream.synchronize()
-    T = int(count[0])
+    T = count.item()
     return out_ids[:T], out_src[:T], atoms
 
 
