@@ -663,8 +663,11 @@ __global__ void __launch_bounds__(kThreads, 1)
         done[u] = -1;
         if (k < n_own) {
           w[u] = xwt[k * n_src + s];
-          if (w[u] != 0.f)
-            v[u] = ld_cluster_f4(smem_addr(xo + xo_at(src_tile(s, x0 + k), (x0 + k) & (kTileRows - 1), c)), src_cta(s));
+          if (w[u] != 0.f) {
+            const float4* from = xo + xo_at(src_tile(s, x0 + k), (x0 + k) & (kTileRows - 1), c);
+            // (a decode's are its own: 24 branches 329 -> 325 us with plain loads)
+            v[u] = kDecode ? *from : ld_cluster_f4(smem_addr(from), src_cta(s));
+          }
           if (++s == n_src) {
             done[u] = k;
             s = 0;
