@@ -41,10 +41,11 @@
 //               ahead), one 2 KiB TMA copy per (page, 64-wide half of D, K|V)
 //               into a ring of stages, per-stage mbarriers with byte counts;
 //               a stage's copies are issued by the warp's lanes together.
-//               Narrow: one ring of three stages, a stage's K and V slots
-//               freed together after its P V.  Wide: K and V have their own
-//               rings of two slots and barriers; a K slot is freed by the
-//               commit after S_j, a V slot after P_j V_j.
+//               Narrow: one ring of three stages (D = 64: four), a stage's K
+//               and V slots freed together after its P V.  Wide: K and V have
+//               rings and barriers of their own (two and three slots; D = 64:
+//               six and six); a K slot is freed by the commit after S_j, a V
+//               slot after P_j V_j.
 //               A decode step (st_decode_step): the narrow item that holds a
 //               branch's last page first stores the step's new K and V row of
 //               its (layer, KV head) into that page, then a proxy fence makes
@@ -134,8 +135,11 @@ struct TcCfg {
   // stages).
   // As many slots as two CTAs' shared memory takes: what is in flight bounds
   // the rate (D = 64, 8 groups of 5 branches: 171 us with 3 slots, 142 with 4).
+  // Wide: a V slot is held until its P V, a K slot only until its S, so the odd
+  // slot is V's (9 branches, 4 layers: 748 us with 2 + 2, 738 with 2 + 3, 753
+  // with 3 + 2).
   static constexpr int kStages = D == 128 ? (kWide ? 2 : 3) : (kWide ? 6 : 4);  // K slots
-  static constexpr int kVStages = kStages;                                      // V slots
+  static constexpr int kVStages = D == 128 && kWide ? 3 : kStages;              // V slots
   static constexpr bool kSplitKV = kWide;
   // S at M = 64 for <= 64 stacked rows: score rows sit in TMEM lanes 0..15
   // of each warp's 32-lane quarter (row r at lane 32 (r / 16) + r % 16);

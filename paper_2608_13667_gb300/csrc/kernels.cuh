@@ -117,6 +117,7 @@ struct AttnParams {
   int32_t keep_l2;         // decode: the launch's pages fit in L2; load them evict-normal so they stay
   const MergeItem* mitems; // batched merge: cluster x takes mitems[x] (slot, L0, T above unused)
   int32_t kv_split;        // merge: CTAs (a cluster) that share one row tile's keys
+  int32_t layer_base;      // merge: CTA z takes layer layer_base + z
   // decode step (items flagged kItemAppend): the rows the step appends,
   // [L][n_br][Hkv][D], and the pools they go to
   const __nv_bfloat16* app_k;
@@ -227,9 +228,10 @@ cudaError_t launch_decode_tc(const CUtensorMap& kmap, const CUtensorMap& vmap, c
 // Causal merge prefill on tcgen05, two 128-row query tiles per CTA sharing
 // K/V (merge_tc.cu): one sequence (p.slot, p.L0, p.T; p.mitems null) or a
 // batch of n_items work items (p.mitems, and the same items on the host),
-// p.q -> p.out_o, p.out_lse.
+// p.q -> p.out_o, p.out_lse.  *n_launches: the kernels it took (one, or two
+// for some layers each).
 cudaError_t launch_merge_tc(const CUtensorMap& kmap, const CUtensorMap& vmap, const AttnParams& p,
-                            const MergeItem* host_items, int n_items, int D, cudaStream_t s);
+                            const MergeItem* host_items, int n_items, int D, cudaStream_t s, int* n_launches);
 // Decode partials of fork groups of 129 to 256 stacked rows on the same
 // paired tile (one CTA per item x KV head x layer, items from p.item_base on,
 // launched as a programmatic dependent like the other decode kernels).

@@ -132,7 +132,9 @@ struct PairCfg {
   static_assert(kSmemBytes <= 227 * 1024, "shared memory of one CTA");
 };
 
-template <int D, bool kDecode>
+// kRest: the second launch of a merge, layers from p.layer_base on (an argument
+// of the template, since the offset in every launch cost half a per cent).
+template <int D, bool kDecode, bool kRest>
 __global__ void __launch_bounds__(kThreads, 1)
     merge_pair_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant__ CUtensorMap vmap,
                       const AttnParams p, const __grid_constant__ InlineDecodePlan inl) {
@@ -155,7 +157,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   const int warp = threadIdx.x >> 5;
   const int lane = threadIdx.x & 31;
   const int kvh = blockIdx.y;
-  const int layer = blockIdx.z;
+  const int layer = (kRest ? p.layer_base : 0) + blockIdx.z;
   const int G = p.G;
 
   // Launched as a programmatic dependent of the kernel before it in the
@@ -711,12 +713,17 @@ cudaError_t pair_setup(const PairSetup** out) {
   PairSetup& ps = setups[dev];
   std::lock_guard<std::mutex> lock(mu);
   if (!ps.done) {
-    auto* kernel = merge_pair_kernel<D, kDecode>;
+    auto* kernel = merge_pair_kernel<D, kDecode, false>;
     e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmemBytes);
     if (e != cudaSuccess) return e;
     if constexpr (!kDecode) {
-      e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+      auto* rest = merge_pair_kernel<D, false, true>;
+      e = cudaFuncSetAttribute(rest, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmemBytes);
       if (e != cudaSuccess) return e;
+      for (auto* k : {kernel, rest}) {
+        e = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+        if (e != cudaSuccess) return e;
+      }
       for (int n = 1; n <= kMaxMergeSplit; ++n) {
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3(n);
@@ -760,45 +767,77 @@ MergeSplitCost merge_tile_cost(int all_tiles, int n_rows, int split) {
 
 template <int D>
 cudaError_t launch_merge_t(const CUtensorMap& km, const CUtensorMap& vm, AttnParams p, const MergeItem* host_items,
-                           int n_items, cudaStream_t s) {
+                           int n_items, cudaStream_t s, int* n_launches) {
   const PairSetup* ps = nullptr;
   cudaError_t e = pair_setup<D, false>(&ps);
   if (e != cudaSuccess) return e;
-  const int64_t copies = (int64_t)p.Hkv * p.L;  // of every row tile
-  // CTAs per row tile: the size with the least estimated time, which is waves
-  // of CTAs of average length, or the longest CTA if that is more.  Over 19
-  // shapes and 12 sizes the choice was within 6% of the best one measured (10
-  // parts for 24 row tiles, say, need two waves and take 114 us, where 5 take
-  // 93).  With 8 waves and more the last one's loss is small and a split only
-  // adds CTAs: 4 layers of 256 row tiles took 2.01 ms whole, 2.23 in two parts.
-  int split = 1;
-  if (n_items * copies < 8 * (int64_t)ps->resident[1]) {
-    float best = 0.f;
-    for (int n = 1; n <= kMaxMergeSplit; ++n) {
+  // Estimated time of `layers` layers in clusters of n: waves of CTAs of average
+  // length, or the longest CTA if that is more.
+  auto estimate = [&](int n, int layers) {
+    int64_t ctas = 0;
+    float total = 0.f, longest = 0.f;
+    for (int i = 0; i < n_items; ++i) {
+      const int T = host_items ? host_items[i].T : p.T, L0 = host_items ? host_items[i].L0 : p.L0;
+      const int row_base = host_items ? host_items[i].row_base : i * 2 * kTileRows;
+      const int rows = std::min(2 * kTileRows, T * p.G - row_base);
+      const int keys = L0 + (row_base + rows - 1) / p.G + 1;
+      const MergeSplitCost c = merge_tile_cost((keys + kKeys - 1) / kKeys, rows, n);
+      ctas += c.parts;
+      total += c.total;
+      longest = std::max(longest, c.longest);
+    }
+    const int64_t waves = (ctas * p.Hkv * layers + ps->resident[n] - 1) / ps->resident[n];
+    return std::max(longest, waves * total / ctas);
+  };
+  // CTAs per row tile: the size with the least estimate.  Over 19 shapes and 12
+  // sizes the choice was within 6% of the best one measured (10 parts for 24 row
+  // tiles, say, need two waves and take 114 us, where 5 take 93).
+  auto best_split = [&](int layers, float* time) {
+    int split = 1;
+    *time = estimate(1, layers);
+    for (int n = 2; n <= kMaxMergeSplit; ++n) {
       if (ps->resident[n] < 1) continue;
-      int64_t ctas = 0;
-      float total = 0.f, longest = 0.f;
-      for (int i = 0; i < n_items; ++i) {
-        const int T = host_items ? host_items[i].T : p.T, L0 = host_items ? host_items[i].L0 : p.L0;
-        const int row_base = host_items ? host_items[i].row_base : i * 2 * kTileRows;
-        const int rows = std::min(2 * kTileRows, T * p.G - row_base);
-        const int keys = L0 + (row_base + rows - 1) / p.G + 1;
-        const MergeSplitCost c = merge_tile_cost((keys + kKeys - 1) / kKeys, rows, n);
-        ctas += c.parts;
-        total += c.total;
-        longest = std::max(longest, c.longest);
-      }
-      const int64_t waves = (ctas * copies + ps->resident[n] - 1) / ps->resident[n];
-      const float time = std::max(longest, waves * total / ctas);
-      if (n == 1 || time < 0.97f * best) {
-        best = time;
+      const float t = estimate(n, layers);
+      if (t < 0.97f * *time) {
+        *time = t;
         split = n;
       }
     }
+    return split;
+  };
+  // With 8 waves and more the last one's loss is small and a split only adds
+  // CTAs: 4 layers of 256 row tiles took 2.01 ms whole, 2.23 in two parts.
+  int split[2] = {1, 1}, layers[2] = {p.L, 0};
+  const int64_t sms = ps->resident[1], per_layer = (int64_t)n_items * p.Hkv, total = per_layer * p.L;
+  if (total < 8 * sms) {
+    float time;
+    split[0] = best_split(p.L, &time);
+    // A few whole waves and a rest: the layers of the whole waves as they are,
+    // and the rest in a launch behind them, split so that it fills the SMs
+    // (44 rows onto 23040 in 32 layers, 256 row tiles: 755 us in one launch, 712
+    // in two).
+    const int whole = (int)(total / sms * sms / per_layer);
+    if (whole > 0 && whole < p.L) {
+      float rest;
+      const int rest_split = best_split(p.L - whole, &rest);
+      if (estimate(1, whole) + rest < 0.95f * time) {
+        split[0] = 1;
+        split[1] = rest_split;
+        layers[0] = whole;
+        layers[1] = p.L - whole;
+      }
+    }
   }
-  p.kv_split = split;
-  return launch_chained_cluster(merge_pair_kernel<D, false>, dim3(n_items * split, p.Hkv, p.L), dim3(kThreads),
-                                PairCfg<D>::kSmemBytes, s, split, km, vm, p, kNoInline);
+  for (int i = 0; i < 2 && layers[i] > 0; ++i) {
+    p.kv_split = split[i];
+    p.layer_base = i ? layers[0] : 0;
+    e = launch_chained_cluster(i ? merge_pair_kernel<D, false, true> : merge_pair_kernel<D, false, false>,
+                               dim3(n_items * split[i], p.Hkv, layers[i]), dim3(kThreads), PairCfg<D>::kSmemBytes, s,
+                               split[i], km, vm, p, kNoInline);
+    if (e != cudaSuccess) return e;
+    *n_launches = i + 1;
+  }
+  return cudaSuccess;
 }
 
 template <int D>
@@ -807,19 +846,20 @@ cudaError_t launch_decode_pair_t(const CUtensorMap& km, const CUtensorMap& vm, c
   const PairSetup* ps = nullptr;
   cudaError_t e = pair_setup<D, true>(&ps);
   if (e != cudaSuccess) return e;
-  return launch_chained(merge_pair_kernel<D, true>, dim3(n_items, p.Hkv, p.L), dim3(kThreads), PairCfg<D>::kSmemBytes,
+  return launch_chained(merge_pair_kernel<D, true, false>, dim3(n_items, p.Hkv, p.L), dim3(kThreads), PairCfg<D>::kSmemBytes,
                         s, km, vm, p, inl);
 }
 
 }  // namespace
 
 cudaError_t launch_merge_tc(const CUtensorMap& km, const CUtensorMap& vm, const AttnParams& p,
-                            const MergeItem* host_items, int n_items, int D, cudaStream_t s) {
+                            const MergeItem* host_items, int n_items, int D, cudaStream_t s, int* n_launches) {
+  *n_launches = 0;
   // one merge: ceil(T G / 256) row tiles; a batch: its work items
   if (!p.mitems) n_items = (p.T * p.G + 2 * kTileRows - 1) / (2 * kTileRows);
   if (n_items <= 0) return cudaSuccess;
-  if (D == 128) return launch_merge_t<128>(km, vm, p, host_items, n_items, s);
-  if (D == 64) return launch_merge_t<64>(km, vm, p, host_items, n_items, s);
+  if (D == 128) return launch_merge_t<128>(km, vm, p, host_items, n_items, s, n_launches);
+  if (D == 64) return launch_merge_t<64>(km, vm, p, host_items, n_items, s, n_launches);
   return cudaErrorInvalidValue;
 }
 

@@ -1313,8 +1313,10 @@ ST_API st_status st_merge(st_pool* P, st_seq main, int n_tok, const void* q, con
   const double io_bytes = (double)c.n_layers * n_tok * c.n_q_heads * (c.head_dim * 2 + c.head_dim * 4 + 4);
   const double keys = (double)n_tok * L0 + (double)n_tok * (n_tok + 1) / 2;
   const double flops = 4.0 * c.head_dim * keys * c.n_q_heads * c.n_layers;
+  int n_launches = 0;
   st = run_kernel(P, kKMerge, kv_bytes + io_bytes, flops, s,
-                  [&] { return launch_merge_tc(P->kmap, P->vmap, ap, nullptr, 0, c.head_dim, s); });
+                  [&] { return launch_merge_tc(P->kmap, P->vmap, ap, nullptr, 0, c.head_dim, s, &n_launches); }, 0);
+  P->stats[kKMerge].kernels += n_launches;
   return st == ST_OK ? ST_OK : poison(P, st);  // the rows are in, their prefill is not
 }
 
@@ -1412,8 +1414,11 @@ ST_API st_status st_prefill_batch(st_pool* P, const st_seq* seqs, int n_seq, con
   ap.mitems = d_items;
   ap.hold_loads = (c.flags & ST_FLAG_HOLD_LOADS) ? 1 : 0;
   const int n_items = (int)items.size();
-  st = run_kernel(P, kKMerge, kv_bytes + io_bytes, flops, s,
-                  [&] { return launch_merge_tc(P->kmap, P->vmap, ap, items.data(), n_items, c.head_dim, s); });
+  int n_launches = 0;
+  st = run_kernel(P, kKMerge, kv_bytes + io_bytes, flops, s, [&] {
+    return launch_merge_tc(P->kmap, P->vmap, ap, items.data(), n_items, c.head_dim, s, &n_launches);
+  }, 0);
+  P->stats[kKMerge].kernels += n_launches;
   const st_status rs = retire_plan(P, ps, s);
   if (st != ST_OK) return poison(P, st);
   return rs == ST_OK ? ST_OK : poison(P, rs);

@@ -67,3 +67,22 @@ def test_batch_of_short_and_long_tiles_in_one_cluster_size(stlib):
             o_ref, l_ref = A.merge_prefill(q[layer, at:at + n].cpu(), k, v, l0)
             compare(o[layer, at:at + n], lse[layer, at:at + n], o_ref, l_ref, f"seq {r} layer {layer}")
         at += n
+
+
+def test_layers_of_the_last_wave_in_a_launch_of_their_own(stlib):
+    # 256 row tiles: 19 layers fill the SMs once, the other 13 are split
+    L, ctx, T = 32, 26000, 40
+    w = Workload(name="split_layers", n_layers=L, n_q_heads=32, n_kv_heads=8, head_dim=64, n_blocks=(ctx + T) // 16 + 8,
+                 seed=53)
+    run = Run(w, max_seqs=2, max_decode_branches=1, max_splits=2)
+    m = run.create()
+    for i in range(0, ctx, 6500):
+        run.append([m], 6500, ("ctx", i))
+    run.pool.profile_read()
+    q, o, lse, L0 = run.merge(m, T, ("rows",))
+    run.pool.sync()
+    assert run.pool.profile_read()["merge_prefill"]["kernels"] == 2
+    for layer in (0, 18, 19, L - 1):
+        k, v = run.context(m, layer)
+        o_ref, l_ref = A.merge_prefill(q[layer].cpu(), k, v, L0)
+        compare(o[layer], lse[layer], o_ref, l_ref, f"layer {layer}")
