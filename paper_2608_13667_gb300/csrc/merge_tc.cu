@@ -115,6 +115,16 @@ struct MergeSplitCost {
   float total, longest;  // of its CTAs together, of one of them
 };
 
+// 16 bytes from global to shared memory, asynchronously; zeros if !valid.
+__device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, bool valid) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst),
+               "l"(__cvta_generic_to_global(src)), "r"(valid ? 16 : 0)
+               : "memory");
+}
+
+// Waits for every copy of this thread.
+__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
 template <int D>
 struct PairCfg {
   static constexpr int kHalves = D / 64;
@@ -242,6 +252,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   n_pages = min(n_pages - j0 * kPagesPerStage, n_tiles * kPagesPerStage);
   // at most 128 rows: both tiles hold them, tile A takes the even stages and tile B the odd ones
   const bool dual = !kDecode && n_rows <= kTileRows;
+  const bool direct = kDecode || (n_parts == 1 && !dual);  // every row has one source, its thread's
 
 
   // ---- loaders -------------------------------------------------------------------
@@ -453,13 +464,21 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int limit = kDecode ? n_valid_keys : valid ? L0 + qrow + 1 : n_valid_keys;
     const int min_limit = kDecode ? n_valid_keys : L0 + tile_row0 / G + 1;  // the tile's first row sees the fewest keys
     if (!dual || t == 0) {
-      const uint4* src = reinterpret_cast<const uint4*>(p.q + in_row * D);
-      uint8_t* q_s = base + C::kQOff + t * C::kQTileBytes;
-#pragma unroll
-      for (int c = 0; c < D / 8; ++c) {
-        const uint4 v = valid ? src[c] : make_uint4(0u, 0u, 0u, 0u);
-        *reinterpret_cast<uint4*>(q_s + (c >> 3) * C::kQHalfBytes + r * 128 + (((c & 7) ^ (r & 7)) << 4)) = v;
+      // D/8 lanes copy a row's D contiguous values, straight to shared memory:
+      // all 32 rows of the warp are in flight at once (a thread loading its own
+      // row through registers took 4.7 us for the tile, this 1.9)
+      constexpr int kChunks = D / 8, kRows = 32 / kChunks;
+      const uint32_t q_s = smem_addr(base + C::kQOff + t * C::kQTileBytes);
+      const int c = lane % kChunks;
+      const int64_t mine = valid ? in_row : -1;
+#pragma unroll 4
+      for (int i = 0; i < 32 / kRows; ++i) {
+        const int x = i * kRows + lane / kChunks, row = (warp & 3) * 32 + x;
+        const int64_t from = __shfl_sync(0xffffffffu, mine, x);
+        cp_async16(q_s + (c >> 3) * C::kQHalfBytes + row * 128 + (((c & 7) ^ (row & 7)) << 4),
+                   p.q + (from >= 0 ? from * D + c * 8 : 0), from >= 0);
       }
+      cp_async_wait();
       fence_proxy_async_smem();
     }
     mbar_arrive(q_ready);
@@ -581,30 +600,50 @@ __global__ void __launch_bounds__(kThreads, 1)
     if (ok) ok = __all_sync(0xffffffffu, mbar_wait(o_final, 0));
     tc_fence_after_sync();
     if (!ok && lane == 0) atomicCAS(p.status, 0, kDevTimeout);
+    // O out of TMEM, a thread its row; final if this tile has the row's only source
     const bool some = ok && n_it > 0;
     if (some) {
+      const float scale = direct ? 1.f / l : 1.f;
 #pragma unroll 1
       for (int k = 0; k < D / 32; ++k) {
         float o[32];
         tmem_ld32(t_lane + kTmemO + k * 32, o);
 #pragma unroll
         for (int i = 0; i < 8; ++i)
-          xo[xo_at(t, r, k * 8 + i)] = make_float4(o[4 * i], o[4 * i + 1], o[4 * i + 2], o[4 * i + 3]);
+          xo[xo_at(t, r, k * 8 + i)] =
+              make_float4(o[4 * i] * scale, o[4 * i + 1] * scale, o[4 * i + 2] * scale, o[4 * i + 3] * scale);
       }
     }
-    xml[t * kTileRows + r] = make_float2(m_used, some ? l : 0.f);
+    if (!direct) {
+      xml[t * kTileRows + r] = make_float2(m_used, some ? l : 0.f);
+    } else if (some) {
+      // the warp writes its 32 rows, D contiguous values at a time (a thread
+      // writing its own row touches 32 rows per store: 6.3 us from the last P V
+      // to the end; through the exchange below 5.8; this way 3.1)
+      __syncwarp();
+      const int64_t out_row = !valid ? -1 : kDecode ? in_row * p.max_splits + item.split : in_row;
+      constexpr int kRows = 32 / kQuads < 1 ? 1 : 32 / kQuads;
+      const int c = lane % kQuads;
+#pragma unroll 4
+      for (int i = 0; i < 32 / kRows; ++i) {
+        const int x = i * kRows + lane / kQuads;
+        const int64_t to = __shfl_sync(0xffffffffu, out_row, x);
+        if (to >= 0) reinterpret_cast<float4*>(p.out_o + to * D)[c] = xo[xo_at(t, (warp & 3) * 32 + x, c)];
+      }
+      if (valid) p.out_lse[out_row] = (m_used + log2f(l)) * kLn2;
+    }
     tc_fence_before_sync();
     named_barrier_sync(1, kSoftThreads + 32);
   }
 
-  // ---- results ---------------------------------------------------------------------
+  // ---- results of several sources ------------------------------------------------------
+  if (direct) return;
   // A row's sources are the CTAs of its cluster, and in each both tiles when
   // they share their rows: O = sum 2^(m_s - m) O_s / sum 2^(m_s - m) l_s.  The
   // rows are dealt out to the CTAs, and D/4 lanes put together a row: every
   // read of a source's row, through distributed shared memory, and every write
-  // of O are D contiguous values (a thread writing its own row touches 32 rows
-  // per store: 5.6 us for a CTA's 256 rows, against 3 this way).  A source without a key
-  // for the row has l = 0, and its O was perhaps never written.
+  // of O are D contiguous values.  A source without a key for the row has l = 0,
+  // and its O was perhaps never written.
   // This code runs once per CTA, so its time is mostly that of fetching its
   // instructions: loops are kept rolled (a version with 16 loads in flight
   // took 12 us where the same work rolled took 5).
@@ -640,9 +679,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       xwt[i] = (mine.y != 0.f ? ex2(mine.x - m) : 0.f) / l;  // (NaN for a row without any weight)
       if (i == k * n_src) {
         const int gr = row_base + x0 + k;
-        const int row = kDecode ? members[item.member_base + gr / G] : q_row0 + gr / G;
-        int64_t out_row = ((int64_t)layer * p.n_rows_q + row) * p.Hq + kvh * G + gr % G;
-        if constexpr (kDecode) out_row = out_row * p.max_splits + item.split;  // a split-KV partial
+        const int64_t out_row = ((int64_t)layer * p.n_rows_q + q_row0 + gr / G) * p.Hq + kvh * G + gr % G;
         xrow[k] = out_row;
         if (ok) p.out_lse[out_row] = (m + log2f(l)) * kLn2;
       }
@@ -665,11 +702,8 @@ __global__ void __launch_bounds__(kThreads, 1)
         done[u] = -1;
         if (k < n_own) {
           w[u] = xwt[k * n_src + s];
-          if (w[u] != 0.f) {
-            const float4* from = xo + xo_at(src_tile(s, x0 + k), (x0 + k) & (kTileRows - 1), c);
-            // (a decode's are its own: 24 branches 329 -> 325 us with plain loads)
-            v[u] = kDecode ? *from : ld_cluster_f4(smem_addr(from), src_cta(s));
-          }
+          if (w[u] != 0.f)
+            v[u] = ld_cluster_f4(smem_addr(xo + xo_at(src_tile(s, x0 + k), (x0 + k) & (kTileRows - 1), c)), src_cta(s));
           if (++s == n_src) {
             done[u] = k;
             s = 0;
