@@ -21,11 +21,11 @@
 //   - a tile of at most 128 rows leaves tile B without rows: then both tiles
 //     hold the same rows, A takes the even stages and B the odd ones ("dual"),
 //     so the tensor cores do no work for padding and a stage costs half.
-// One layer, 32/8 heads, D 128, a context of 23040: 16 rows 350 -> 38 us, 44
-// rows 353 -> 50, 133 rows 363 -> 93, 512 rows 363 -> 197; 88 rows onto 8192
-// 140 -> 42 us.
+// One layer, 32/8 heads, D 128, a context of 23040: 16 rows 350 -> 37 us, 44
+// rows 353 -> 47, 133 rows 363 -> 88, 512 rows 363 -> 193; 88 rows onto 8192
+// 140 -> 38 us.
 //
-// CTA layout (352 threads, one CTA per SM, all 512 TMEM columns):
+// CTA layout (384 threads, one CTA per SM, all 512 TMEM columns):
 //   warps 0..3  softmax of tile A, warps 4..7 softmax of tile B: thread r of
 //               a tile owns its row r = TMEM lane r (warp w reads lanes
 //               32 (w % 4) ..).  It stages its Q row in shared memory; per
@@ -34,9 +34,9 @@
 //               only when a score exceeds it by more than 2^8 (O in TMEM is
 //               then rescaled in place), and writes P = 2^(s - m) as two bf16
 //               terms (P_hi + P_lo, exact to about 16 bits) into TMEM over its
-//               own scores.  At the end it writes O to shared memory, and the
-//               warps put rows together from there, from every CTA of the
-//               cluster and both tiles where those share the row.
+//               own scores.  At the end it writes O to shared memory, from
+//               where its warp writes the rows out, or, where a cluster's CTAs
+//               or both tiles share them, the warps put them together.
 //   warp 8      K loader, warp 9 V loader: page ids from the block table (32
 //               per read, one batch ahead), one 2 KiB TMA copy per (page,
 //               64-wide half of D) into separate K and V rings.
@@ -47,6 +47,14 @@
 //                 S_t(j) = Q_t K_j^T        (M 128, N 128)
 //               so that the softmax of one tile overlaps the MMAs of the
 //               other.
+//   warp 11     idle: it fills the third warpgroup, for the register split.
+//
+// What bounds it: at N = 128 a tcgen05.mma takes 65 to 78 cycles here with A in
+// tensor memory and some 85 with A in shared memory, against 64; the 48 of a
+// stage take 3360 cycles with a trivial softmax in place of this one, which
+// makes them 3700 to 3800, by its tensor-memory traffic and by the hand-overs
+// (publishing P in quarters, or moving the K and V waits from the MMA warp to
+// a softmax warp, cost 4 to 7%).
 //
 // TMEM columns: tile t (0 = A, 1 = B) has S at 256 t (128 columns; the 16
 // columns of keys [16 k, 16 k + 16) then hold P_hi and P_lo of those keys as
@@ -89,12 +97,53 @@ constexpr int kTileRows = 128;
 constexpr int kKeys = 128;  // keys per stage
 constexpr int kPagesPerStage = kKeys / kPageTokens;
 constexpr int kKLoadWarp = 8, kVLoadWarp = 9, kMmaWarp = 10;
-constexpr int kThreads = 11 * 32;
+constexpr int kThreads = 12 * 32;  // three warpgroups, for the register split
 constexpr int kSoftThreads = 8 * 32;
+// Where the softmax threads hold a row's 128 scores (kHold), the warpgroups'
+// registers are shared out anew, within what the block is launched with (168 a
+// thread): 192 + 192 + 120.
+constexpr int kSoftRegs = 192, kOtherRegs = 120;
+static_assert(kSoftThreads * kSoftRegs + (kThreads - kSoftThreads) * kOtherRegs <= kThreads * 168,
+              "registers of a block");
 constexpr uint32_t kTmemCols = 512;
 constexpr uint32_t kTmemTile = 256, kTmemO = 128;  // per-tile column base, O offset within it
 constexpr float kRescaleThreshold = 8.f;           // log2 units
 constexpr float kLn2 = 0.69314718055994530942f;
+
+// Load 128 consecutive fp32 columns of this thread's TMEM lane with one wait.
+__device__ __forceinline__ void tmem_ld128(uint32_t taddr, float* v) {
+  uint32_t r[128];
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x128.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
+      "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31, "
+      "%32, %33, %34, %35, %36, %37, %38, %39, %40, %41, %42, %43, %44, %45, %46, %47, "
+      "%48, %49, %50, %51, %52, %53, %54, %55, %56, %57, %58, %59, %60, %61, %62, %63, "
+      "%64, %65, %66, %67, %68, %69, %70, %71, %72, %73, %74, %75, %76, %77, %78, %79, "
+      "%80, %81, %82, %83, %84, %85, %86, %87, %88, %89, %90, %91, %92, %93, %94, %95, "
+      "%96, %97, %98, %99, %100, %101, %102, %103, %104, %105, %106, %107, %108, %109, %110, %111, "
+      "%112, %113, %114, %115, %116, %117, %118, %119, %120, %121, %122, %123, %124, %125, %126, %127}, [%128];\n\t"
+      "tcgen05.wait::ld.sync.aligned;"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
+        "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
+        "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31]),
+        "=r"(r[32]), "=r"(r[33]), "=r"(r[34]), "=r"(r[35]), "=r"(r[36]), "=r"(r[37]), "=r"(r[38]), "=r"(r[39]),
+        "=r"(r[40]), "=r"(r[41]), "=r"(r[42]), "=r"(r[43]), "=r"(r[44]), "=r"(r[45]), "=r"(r[46]), "=r"(r[47]),
+        "=r"(r[48]), "=r"(r[49]), "=r"(r[50]), "=r"(r[51]), "=r"(r[52]), "=r"(r[53]), "=r"(r[54]), "=r"(r[55]),
+        "=r"(r[56]), "=r"(r[57]), "=r"(r[58]), "=r"(r[59]), "=r"(r[60]), "=r"(r[61]), "=r"(r[62]), "=r"(r[63]),
+        "=r"(r[64]), "=r"(r[65]), "=r"(r[66]), "=r"(r[67]), "=r"(r[68]), "=r"(r[69]), "=r"(r[70]), "=r"(r[71]),
+        "=r"(r[72]), "=r"(r[73]), "=r"(r[74]), "=r"(r[75]), "=r"(r[76]), "=r"(r[77]), "=r"(r[78]), "=r"(r[79]),
+        "=r"(r[80]), "=r"(r[81]), "=r"(r[82]), "=r"(r[83]), "=r"(r[84]), "=r"(r[85]), "=r"(r[86]), "=r"(r[87]),
+        "=r"(r[88]), "=r"(r[89]), "=r"(r[90]), "=r"(r[91]), "=r"(r[92]), "=r"(r[93]), "=r"(r[94]), "=r"(r[95]),
+        "=r"(r[96]), "=r"(r[97]), "=r"(r[98]), "=r"(r[99]), "=r"(r[100]), "=r"(r[101]), "=r"(r[102]), "=r"(r[103]),
+        "=r"(r[104]), "=r"(r[105]), "=r"(r[106]), "=r"(r[107]), "=r"(r[108]), "=r"(r[109]), "=r"(r[110]), "=r"(r[111]),
+        "=r"(r[112]), "=r"(r[113]), "=r"(r[114]), "=r"(r[115]), "=r"(r[116]), "=r"(r[117]), "=r"(r[118]), "=r"(r[119]),
+        "=r"(r[120]), "=r"(r[121]), "=r"(r[122]), "=r"(r[123]), "=r"(r[124]), "=r"(r[125]), "=r"(r[126]), "=r"(r[127])
+      : "r"(taddr)
+      : "memory");
+#pragma unroll
+  for (int i = 0; i < 128; ++i) v[i] = __uint_as_float(r[i]);
+}
 
 // CTAs of a cluster that share one row tile's keys in a merge, at most (16 is
 // the largest cluster of this part).
@@ -122,6 +171,16 @@ __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, bool v
                : "memory");
 }
 
+// Registers of this warpgroup's threads from here on.
+template <int N>
+__device__ __forceinline__ void regs_inc() {
+  asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(N));
+}
+template <int N>
+__device__ __forceinline__ void regs_dec() {
+  asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(N));
+}
+
 // Waits for every copy of this thread.
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
@@ -142,14 +201,19 @@ struct PairCfg {
   static_assert(kSmemBytes <= 227 * 1024, "shared memory of one CTA");
 };
 
-// kRest: the second launch of a merge, layers from p.layer_base on (an argument
-// of the template, since the offset in every launch cost half a per cent).
-template <int D, bool kDecode, bool kRest>
+// kMapped: a merge's CTAs (clusters) are not its tiles, heads and layers as the
+// grid numbers them.  The layers may start at p.layer_base (a merge's second
+// launch), and a last tile of at most 128 rows, whose stages cost half, comes
+// behind the other tiles of every head and layer, so that the launch ends on
+// the short ones (88 rows onto 8000 in 16 layers: 280 us before, 229).  A form
+// of its own, since the arithmetic in every launch cost half a per cent.
+template <int D, bool kDecode, bool kMapped>
 __global__ void __launch_bounds__(kThreads, 1)
     merge_pair_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant__ CUtensorMap vmap,
                       const AttnParams p, const __grid_constant__ InlineDecodePlan inl) {
   using C = PairCfg<D>;
   constexpr int kKS = C::kKStages, kVS = C::kVStages;
+  constexpr bool kHold = D == 128 && !kDecode;  // the softmax holds its scores (below)
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw = smem_addr(smem_raw);
   uint8_t* base = smem_raw + ((1024u - (raw & 1023u)) & 1023u);
@@ -166,8 +230,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 
   const int warp = threadIdx.x >> 5;
   const int lane = threadIdx.x & 31;
-  const int kvh = blockIdx.y;
-  const int layer = (kRest ? p.layer_base : 0) + blockIdx.z;
+  int kvh = blockIdx.y, layer = blockIdx.z;
   const int G = p.G;
 
   // Launched as a programmatic dependent of the kernel before it in the
@@ -205,7 +268,20 @@ __global__ void __launch_bounds__(kThreads, 1)
   const int cluster = kDecode ? 1 : p.kv_split;  // CTAs that share a row tile
   const int rank = kDecode ? 0 : (int)blockIdx.x % cluster;
   int slot = p.slot, L0 = p.L0, T = p.T, q_row0 = 0;
-  int row_base = ((int)gridDim.x / cluster - 1 - (int)blockIdx.x / cluster) * 2 * kTileRows;
+  int tile = (int)blockIdx.x / cluster;
+  if constexpr (kMapped) {
+    const int n = (int)gridDim.x / cluster;
+    if (!p.mitems && n > 1 && T * G - (n - 1) * 2 * kTileRows <= kTileRows) {  // tile 0, the last rows, is short
+      const int u = tile + n * (int)(blockIdx.y + gridDim.y * blockIdx.z);
+      const int full = (n - 1) * (int)(gridDim.y * gridDim.z);  // the other tiles
+      const int hl = u < full ? u / (n - 1) : u - full;         // head and layer
+      tile = u < full ? 1 + u % (n - 1) : 0;
+      kvh = hl % (int)gridDim.y;
+      layer = hl / (int)gridDim.y;
+    }
+    layer += p.layer_base;
+  }
+  int row_base = ((int)gridDim.x / cluster - 1 - tile) * 2 * kTileRows;
   int page_begin = 0, n_rows, n_pages, n_valid_keys;
   AttnItem item{};
   const int32_t* members = nullptr;
@@ -255,177 +331,186 @@ __global__ void __launch_bounds__(kThreads, 1)
   const bool direct = kDecode || (n_parts == 1 && !dual);  // every row has one source, its thread's
 
 
-  // ---- loaders -------------------------------------------------------------------
-  // (hold_loads, a test hook: nothing arrives, the other roles' waits run out)
-  if ((warp == kKLoadWarp || warp == kVLoadWarp) && !p.hold_loads) {
-    const bool is_k = warp == kKLoadWarp;
-    const CUtensorMap* map = is_k ? &kmap : &vmap;
-    uint64_t* full = is_k ? k_full : v_full;
-    uint64_t* empty = is_k ? k_empty : v_empty;
-    const int n_st = is_k ? kKS : kVS;
-    uint8_t* ring = base + (is_k ? C::kKOff : C::kVOff);
-    if (lane == 0) prefetch_tensormap(map);
-    // merge: every CTA of one (layer, KV head) walks the same pages, keep them
-    // in L2; decode: a page is streamed once, unless a sibling subgroup's CTA
-    // reads it too or the whole launch fits in L2
-    const uint64_t policy = !kDecode ? l2_policy_evict_last()
-                            : (p.keep_l2 || (item.flags & kItemReread)) ? l2_policy_evict_normal()
-                                                                         : l2_policy_evict_first();
-    const int32_t* ids = p.table + (int64_t)slot * p.max_pages + page_begin;
-    int base_id = 0;
-    int cur = lane < n_pages ? ids[lane] : 0;
-    int nxt = 32 + lane < n_pages ? ids[32 + lane] : 0;
-    int j = 0;
-    bool ok = true;
-    for (; j < n_tiles; ++j) {
-      const int s = j % n_st;
-      if (j >= n_st) {
-        int w = 1;
-        if (lane == 0) w = mbar_wait(&empty[s], ((j / n_st) - 1) & 1) ? 1 : 0;
-        w = __shfl_sync(0xffffffffu, w, 0);
-        if (!w) {
-          ok = false;
-          break;
-        }
-      }
-      const int page0 = j * kPagesPerStage;
-      if (page0 >= base_id + 32) {
-        base_id += 32;
-        cur = nxt;
-        nxt = base_id + 32 + lane < n_pages ? ids[base_id + 32 + lane] : 0;
-      }
-      const int np = min(kPagesPerStage, n_pages - page0);
-      uint8_t* dst = ring + s * C::kSlotBytes;
-      if (lane == 0) mbar_arrive_expect_tx(&full[s], (uint32_t)(np * C::kHalves * kPageTokens * 128));
-      __syncwarp();
-      // one copy per lane (lane = D/64 q + h)
-      const int q = lane / C::kHalves, h = lane % C::kHalves;
-      int b = __shfl_sync(0xffffffffu, cur, (page0 - base_id + (q < kPagesPerStage ? q : 0)) & 31);
-      if (lane < C::kHalves * np) {
-        if ((uint64_t)b >= (uint64_t)p.n_blocks) {
-          atomicCAS(p.status, 0, kDevBadIndex);
-          b = 0;
-        }
-        tma_load_4d(dst + h * C::kKVHalfBytes + q * kPageTokens * 128, map, &full[s], 0, h, kvh * kPageTokens,
-                    layer * (int)p.n_blocks + b, policy);
-      }
-    }
-    if (!ok && lane == 0) {
-      atomicCAS(p.status, 0, kDevTimeout);
-      for (int t = max(0, j - n_st); t < j; ++t) mbar_wait(&full[t % n_st], (t / n_st) & 1);
-    }
-  }
-
-  // ---- MMA issuer ----------------------------------------------------------------
-  // One warp issues every MMA (two issuing warps interleaving on the tensor
-  // pipe measured slower): all its lanes run the loop with warp-uniform
-  // operands and an elected lane issues.  The issue rate bounds this kernel
-  // (tens of cycles per tcgen05.mma), so the per-MMA work is a constant add:
-  // a shared-memory descriptor's start field holds address / 16 (below 2^14
-  // here), so the descriptor of an operand shifted by b bytes is the base
-  // descriptor + b / 16.
-  if (warp == kMmaWarp) {
-    {
-      constexpr uint32_t idesc_s = tc_idesc_bf16(kTileRows, kKeys, 0, 0);
-      constexpr uint32_t idesc_o = tc_idesc_bf16(kTileRows, D, 0, 1);
-      const uint64_t q_desc = tc_desc_sw128(smem_addr(base + C::kQOff), 16, 1024);
-      const uint64_t k_desc0 = tc_desc_sw128(smem_addr(base + C::kKOff), 16, 1024);
-      const uint64_t v_desc0 = tc_desc_sw128(smem_addr(base + C::kVOff), C::kKVHalfBytes, 1024);
-      bool ok = __all_sync(0xffffffffu, mbar_wait(q_ready, 0));
-      tc_fence_after_sync();
-      // O_t += P_t(i) V, P_t(i) read from TMEM over S_t(i); each half of P
-      // (64 keys) is published on its own, so the first half's MMAs run while
-      // the softmax finishes the second
-      auto issue_pv = [&](auto tile, int i, uint64_t vd) -> bool {
-        constexpr int t = decltype(tile)::value;
-        const uint32_t acc0 = i > 0 ? 1u : 0u;
-#pragma unroll
-        for (int hf = 0; hf < 2; ++hf) {
-          if (!__all_sync(0xffffffffu, mbar_wait(&p_full[2 * t + hf], i & 1))) return false;
-          tc_fence_after_sync();
-#pragma unroll
-          for (int kq = 0; kq < kKeys / 32; ++kq) {
-            const int ks = hf * (kKeys / 32) + kq;
-            const uint64_t vk = vd + (uint64_t)((ks * 16 * 128) >> 4);
-            tc_mma_bf16_tmem_a_elect(tmem + t * kTmemTile + kTmemO, tmem + t * kTmemTile + ks * 16, vk, idesc_o,
-                               ks > 0 ? 1u : acc0);                                    // P_hi
-            tc_mma_bf16_tmem_a_elect(tmem + t * kTmemTile + kTmemO, tmem + t * kTmemTile + ks * 16 + 8, vk, idesc_o,
-                               1u);                                                     // P_lo
-          }
-        }
-        return true;
-      };
-      // S_t(i) = Q_t K^T
-      auto issue_s = [&](auto tile, uint64_t qd, uint64_t kd) {
-        constexpr int t = decltype(tile)::value;
-#pragma unroll
-        for (int h = 0; h < C::kHalves; ++h)
-#pragma unroll
-          for (int kk = 0; kk < 4; ++kk)
-            tc_mma_bf16_elect(tmem + t * kTmemTile, qd + (uint64_t)((h * C::kQHalfBytes + kk * 32) >> 4),
-                              kd + (uint64_t)((h * C::kKVHalfBytes + kk * 32) >> 4), idesc_s, (h | kk) != 0);
-        tc_commit_elect(&s_full[t]);
-      };
-      const std::integral_constant<int, 0> tile_a;
-      const std::integral_constant<int, 1> tile_b;
-      const uint64_t qd_b = q_desc + (uint64_t)(C::kQTileBytes >> 4);
-      if (!dual) {
-        // iteration i of both tiles is stage i
-        auto pv = [&](auto tile, int i) -> bool {
-          constexpr int t = decltype(tile)::value;
-          const int s = i % kVS;
-          if (t == 0 && !__all_sync(0xffffffffu, mbar_wait(&v_full[s], (i / kVS) & 1))) return false;
-          if (!issue_pv(tile, i, v_desc0 + (uint64_t)((s * C::kSlotBytes) >> 4))) return false;
-          if (t == 1) tc_commit_elect(&v_empty[s]);
-          return true;
-        };
-        for (int i = 0; ok && i < n_tiles; ++i) {
-          const int s = i % kKS;
-          const uint64_t kd = k_desc0 + (uint64_t)((s * C::kSlotBytes) >> 4);
-          ok = (i == 0 || pv(tile_a, i - 1)) && __all_sync(0xffffffffu, mbar_wait(&k_full[s], (i / kKS) & 1));
-          if (!ok) break;
-          tc_fence_after_sync();
-          issue_s(tile_a, q_desc, kd);
-          if (i > 0 && !pv(tile_b, i - 1)) {
+  if (warp >= kKLoadWarp) {
+    if constexpr (kHold) regs_dec<kOtherRegs>();
+    // ---- loaders -----------------------------------------------------------------
+    // (hold_loads, a test hook: nothing arrives, the other roles' waits run out)
+    if ((warp == kKLoadWarp || warp == kVLoadWarp) && !p.hold_loads) {
+      const bool is_k = warp == kKLoadWarp;
+      const CUtensorMap* map = is_k ? &kmap : &vmap;
+      uint64_t* full = is_k ? k_full : v_full;
+      uint64_t* empty = is_k ? k_empty : v_empty;
+      const int n_st = is_k ? kKS : kVS;
+      uint8_t* ring = base + (is_k ? C::kKOff : C::kVOff);
+      if (lane == 0) prefetch_tensormap(map);
+      // merge: every CTA of one (layer, KV head) walks the same pages, keep them
+      // in L2; decode: a page is streamed once, unless a sibling subgroup's CTA
+      // reads it too or the whole launch fits in L2
+      const uint64_t policy = !kDecode ? l2_policy_evict_last()
+                              : (p.keep_l2 || (item.flags & kItemReread)) ? l2_policy_evict_normal()
+                                                                           : l2_policy_evict_first();
+      const int32_t* ids = p.table + (int64_t)slot * p.max_pages + page_begin;
+      int base_id = 0;
+      int cur = lane < n_pages ? ids[lane] : 0;
+      int nxt = 32 + lane < n_pages ? ids[32 + lane] : 0;
+      int j = 0;
+      bool ok = true;
+      for (; j < n_tiles; ++j) {
+        const int s = j % n_st;
+        if (j >= n_st) {
+          int w = 1;
+          if (lane == 0) w = mbar_wait(&empty[s], ((j / n_st) - 1) & 1) ? 1 : 0;
+          w = __shfl_sync(0xffffffffu, w, 0);
+          if (!w) {
             ok = false;
             break;
           }
-          issue_s(tile_b, qd_b, kd);
-          tc_commit_elect(&k_empty[s]);
         }
-        if (ok && n_tiles > 0) ok = pv(tile_a, n_tiles - 1) && pv(tile_b, n_tiles - 1);
-      } else {
-        // iteration i of tile t is stage 2 i + t, its own K and V slot; of an
-        // odd number of stages B has one fewer
-        auto pv = [&](auto tile, int i) -> bool {
-          const int j = 2 * i + decltype(tile)::value, s = j % kVS;
-          if (!__all_sync(0xffffffffu, mbar_wait(&v_full[s], (j / kVS) & 1))) return false;
-          if (!issue_pv(tile, i, v_desc0 + (uint64_t)((s * C::kSlotBytes) >> 4))) return false;
-          tc_commit_elect(&v_empty[s]);
-          return true;
-        };
-        auto qk = [&](auto tile, int i) -> bool {
-          const int j = 2 * i + decltype(tile)::value, s = j % kKS;
-          if (!__all_sync(0xffffffffu, mbar_wait(&k_full[s], (j / kKS) & 1))) return false;
-          tc_fence_after_sync();
-          issue_s(tile, q_desc, k_desc0 + (uint64_t)((s * C::kSlotBytes) >> 4));
-          tc_commit_elect(&k_empty[s]);
-          return true;
-        };
-        const int n_a = (n_tiles + 1) / 2, n_b = n_tiles / 2;
-        for (int i = 0; ok && i < n_a; ++i)
-          ok = (i == 0 || pv(tile_a, i - 1)) && qk(tile_a, i) && (i == 0 || pv(tile_b, i - 1)) &&
-               (i >= n_b || qk(tile_b, i));
-        if (ok && n_a > 0) ok = pv(tile_a, n_a - 1) && (n_b < n_a || pv(tile_b, n_b - 1));
+        const int page0 = j * kPagesPerStage;
+        if (page0 >= base_id + 32) {
+          base_id += 32;
+          cur = nxt;
+          nxt = base_id + 32 + lane < n_pages ? ids[base_id + 32 + lane] : 0;
+        }
+        const int np = min(kPagesPerStage, n_pages - page0);
+        uint8_t* dst = ring + s * C::kSlotBytes;
+        if (lane == 0) mbar_arrive_expect_tx(&full[s], (uint32_t)(np * C::kHalves * kPageTokens * 128));
+        __syncwarp();
+        // one copy per lane (lane = D/64 q + h)
+        const int q = lane / C::kHalves, h = lane % C::kHalves;
+        int b = __shfl_sync(0xffffffffu, cur, (page0 - base_id + (q < kPagesPerStage ? q : 0)) & 31);
+        if (lane < C::kHalves * np) {
+          if ((uint64_t)b >= (uint64_t)p.n_blocks) {
+            atomicCAS(p.status, 0, kDevBadIndex);
+            b = 0;
+          }
+          tma_load_4d(dst + h * C::kKVHalfBytes + q * kPageTokens * 128, map, &full[s], 0, h, kvh * kPageTokens,
+                      layer * (int)p.n_blocks + b, policy);
+        }
       }
-      tc_commit_elect(o_final);
-      if (!ok && lane == 0) atomicCAS(p.status, 0, kDevTimeout);
+      if (!ok && lane == 0) {
+        atomicCAS(p.status, 0, kDevTimeout);
+        for (int t = max(0, j - n_st); t < j; ++t) mbar_wait(&full[t % n_st], (t / n_st) & 1);
+      }
     }
-    __syncwarp();
-    named_barrier_sync(1, kSoftThreads + 32);
-    tc_fence_after_sync();
-    tmem_dealloc(tmem, kTmemCols);
+
+    // ---- MMA issuer ----------------------------------------------------------------
+    // One warp issues every MMA (two issuing warps interleaving on the tensor
+    // pipe measured slower): all its lanes run the loop with warp-uniform
+    // operands and an elected lane issues.  The issue rate bounds this kernel
+    // (tens of cycles per tcgen05.mma), so the per-MMA work is a constant add:
+    // a shared-memory descriptor's start field holds address / 16 (below 2^14
+    // here), so the descriptor of an operand shifted by b bytes is the base
+    // descriptor + b / 16.
+    if (warp == kMmaWarp) {
+      {
+        constexpr uint32_t idesc_s = tc_idesc_bf16(kTileRows, kKeys, 0, 0);
+        constexpr uint32_t idesc_o = tc_idesc_bf16(kTileRows, D, 0, 1);
+        const uint64_t q_desc = tc_desc_sw128(smem_addr(base + C::kQOff), 16, 1024);
+        const uint64_t k_desc0 = tc_desc_sw128(smem_addr(base + C::kKOff), 16, 1024);
+        const uint64_t v_desc0 = tc_desc_sw128(smem_addr(base + C::kVOff), C::kKVHalfBytes, 1024);
+        bool ok = __all_sync(0xffffffffu, mbar_wait(q_ready, 0));
+        tc_fence_after_sync();
+        // O_t += P_t(i) V, P_t(i) read from TMEM over S_t(i); each half of P
+        // (64 keys) is published on its own, so the first half's MMAs run while
+        // the softmax finishes the second
+        auto issue_pv = [&](auto tile, int i, uint64_t vd) -> bool {
+          constexpr int t = decltype(tile)::value;
+          const uint32_t acc0 = i > 0 ? 1u : 0u;
+#pragma unroll
+          for (int hf = 0; hf < 2; ++hf) {
+            if (!__all_sync(0xffffffffu, mbar_wait(&p_full[2 * t + hf], i & 1))) return false;
+            tc_fence_after_sync();
+#pragma unroll
+            for (int kq = 0; kq < kKeys / 32; ++kq) {
+              const int ks = hf * (kKeys / 32) + kq;
+              const uint64_t vk = vd + (uint64_t)((ks * 16 * 128) >> 4);
+              tc_mma_bf16_tmem_a_elect(tmem + t * kTmemTile + kTmemO, tmem + t * kTmemTile + ks * 16, vk, idesc_o,
+                                 ks > 0 ? 1u : acc0);                                    // P_hi
+              tc_mma_bf16_tmem_a_elect(tmem + t * kTmemTile + kTmemO, tmem + t * kTmemTile + ks * 16 + 8, vk, idesc_o,
+                                 1u);                                                     // P_lo
+            }
+          }
+          return true;
+        };
+        // S_t(i) = Q_t K^T
+        auto issue_s = [&](auto tile, uint64_t qd, uint64_t kd) {
+          constexpr int t = decltype(tile)::value;
+#pragma unroll
+          for (int h = 0; h < C::kHalves; ++h)
+#pragma unroll
+            for (int kk = 0; kk < 4; ++kk)
+              tc_mma_bf16_elect(tmem + t * kTmemTile, qd + (uint64_t)((h * C::kQHalfBytes + kk * 32) >> 4),
+                                kd + (uint64_t)((h * C::kKVHalfBytes + kk * 32) >> 4), idesc_s, (h | kk) != 0);
+          tc_commit_elect(&s_full[t]);
+        };
+        const std::integral_constant<int, 0> tile_a;
+        const std::integral_constant<int, 1> tile_b;
+        const uint64_t qd_b = q_desc + (uint64_t)(C::kQTileBytes >> 4);
+        if (!dual) {
+          // iteration i of both tiles is stage i
+          auto pv = [&](auto tile, int i) -> bool {
+            constexpr int t = decltype(tile)::value;
+            const int s = i % kVS;
+            if (t == 0 && !__all_sync(0xffffffffu, mbar_wait(&v_full[s], (i / kVS) & 1))) return false;
+            if (!issue_pv(tile, i, v_desc0 + (uint64_t)((s * C::kSlotBytes) >> 4))) return false;
+            if (t == 1) tc_commit_elect(&v_empty[s]);
+            return true;
+          };
+          for (int i = 0; ok && i < n_tiles; ++i) {
+            const int s = i % kKS;
+            const uint64_t kd = k_desc0 + (uint64_t)((s * C::kSlotBytes) >> 4);
+            ok = (i == 0 || pv(tile_a, i - 1)) && __all_sync(0xffffffffu, mbar_wait(&k_full[s], (i / kKS) & 1));
+            if (!ok) break;
+            tc_fence_after_sync();
+            issue_s(tile_a, q_desc, kd);
+            if (i > 0 && !pv(tile_b, i - 1)) {
+              ok = false;
+              break;
+            }
+            issue_s(tile_b, qd_b, kd);
+            tc_commit_elect(&k_empty[s]);
+          }
+          if (ok && n_tiles > 0) ok = pv(tile_a, n_tiles - 1) && pv(tile_b, n_tiles - 1);
+        } else {
+          // iteration i of tile t is stage 2 i + t, its own K and V slot; of an
+          // odd number of stages B has one fewer
+          auto pv = [&](auto tile, int i) -> bool {
+            const int j = 2 * i + decltype(tile)::value, s = j % kVS;
+            if (!__all_sync(0xffffffffu, mbar_wait(&v_full[s], (j / kVS) & 1))) return false;
+            if (!issue_pv(tile, i, v_desc0 + (uint64_t)((s * C::kSlotBytes) >> 4))) return false;
+            tc_commit_elect(&v_empty[s]);
+            return true;
+          };
+          auto qk = [&](auto tile, int i) -> bool {
+            const int j = 2 * i + decltype(tile)::value, s = j % kKS;
+            if (!__all_sync(0xffffffffu, mbar_wait(&k_full[s], (j / kKS) & 1))) return false;
+            tc_fence_after_sync();
+            issue_s(tile, q_desc, k_desc0 + (uint64_t)((s * C::kSlotBytes) >> 4));
+            tc_commit_elect(&k_empty[s]);
+            return true;
+          };
+          const int n_a = (n_tiles + 1) / 2, n_b = n_tiles / 2;
+          for (int i = 0; ok && i < n_a; ++i)
+            ok = (i == 0 || pv(tile_a, i - 1)) && qk(tile_a, i) && (i == 0 || pv(tile_b, i - 1)) &&
+                 (i >= n_b || qk(tile_b, i));
+          if (ok && n_a > 0) ok = pv(tile_a, n_a - 1) && (n_b < n_a || pv(tile_b, n_b - 1));
+        }
+        tc_commit_elect(o_final);
+        if (!ok && lane == 0) atomicCAS(p.status, 0, kDevTimeout);
+      }
+      __syncwarp();
+      named_barrier_sync(1, kSoftThreads + 32);
+      tc_fence_after_sync();
+      tmem_dealloc(tmem, kTmemCols);
+    }
+    if (n_parts > 1) {  // the softmax warps' exchange
+      cluster_sync();
+      cluster_sync();
+    }
+    return;
   }
+  if constexpr (kHold) regs_inc<kSoftRegs>();
 
   // ---- softmax warps ---------------------------------------------------------------
   const int t = warp >> 2;               // tile (of a softmax warp)
@@ -507,9 +592,30 @@ __global__ void __launch_bounds__(kThreads, 1)
             if (c >= n_seen - hf * 64) sc[c] = -INFINITY;
         }
       };
-      // row max over both halves: independent chains of three-input max
+      // With kHold the row's scores stay in registers from the maximum to the
+      // probabilities: reading them twice takes tensor-memory bandwidth from
+      // the MMAs (4 layers of 2048 rows: 1980 us reading twice, 1942 holding;
+      // D = 64, whose MMAs leave the softmax the longer chain, and the decode
+      // are faster with the shorter code that reads twice).
+      float held[kHold ? kKeys : 1];
       float mx;
-      {
+      if constexpr (kHold) {
+        tmem_ld128(t_lane, held);
+        if (edge) {
+#pragma unroll
+          for (int c = 0; c < kKeys; ++c)
+            if (c >= n_seen) held[c] = -INFINITY;
+        }
+        float mx8[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) mx8[i] = fmaxf(held[i], held[8 + i]);
+#pragma unroll
+        for (int c = 16; c < kKeys; c += 16)
+#pragma unroll
+          for (int i = 0; i < 8; ++i) mx8[i] = fmax3(mx8[i], held[c + i], held[c + 8 + i]);
+        mx = fmax3(fmax3(mx8[0], mx8[1], mx8[2]), fmax3(mx8[3], mx8[4], mx8[5]), fmaxf(mx8[6], mx8[7]));
+      } else {
+        // row max over both halves: independent chains of three-input max
         float mx8[8];
 #pragma unroll
         for (int i = 0; i < 8; ++i) mx8[i] = -INFINITY;
@@ -571,27 +677,31 @@ __global__ void __launch_bounds__(kThreads, 1)
       {
         const float2 scale2 = make_float2(sl2, sl2), neg_m2 = make_float2(-m_used, -m_used);
         float2 rs[4] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
-#pragma unroll 1
-        for (int hf = 0; hf < 2; ++hf) {
-          float sc[64];
-          load_half(hf, sc);
+        // one half's P from its scores, published
+        auto publish = [&](int hf, const float* sc) {
 #pragma unroll
           for (int kq = 0; kq < 4; ++kq) {  // 16 keys per step
             uint32_t pk[16];
 #pragma unroll
-            for (int c = 0; c < 16; c += 2) {
-              const float2 x = __ffma2_rn(make_float2(sc[kq * 16 + c], sc[kq * 16 + c + 1]), scale2, neg_m2);
-              const float a = ex2(x.x), b = ex2(x.y);
-              rs[(c >> 1) & 3] = __fadd2_rn(rs[(c >> 1) & 3], make_float2(a, b));
-              const uint32_t hi = pack_bf16(a, b);
-              pk[c / 2] = hi;
-              pk[8 + c / 2] = pack_bf16(a - __uint_as_float(hi << 16), b - __uint_as_float(hi & 0xffff0000u));
-            }
+            for (int c = 0; c < 16; c += 2)
+              prob_pair(sc[kq * 16 + c], sc[kq * 16 + c + 1], scale2, neg_m2, &rs[(c >> 1) & 3], &pk[c / 2],
+                        &pk[8 + c / 2]);
             tmem_st16u_nowait(t_lane + (hf * 4 + kq) * 16, pk);
           }
           tmem_wait_st();
           tc_fence_before_sync();
           mbar_arrive(&p_full[2 * t + hf]);
+        };
+        if constexpr (kHold) {
+          publish(0, held);
+          publish(1, held + 64);
+        } else {
+#pragma unroll 1
+          for (int hf = 0; hf < 2; ++hf) {
+            float sc[64];
+            load_half(hf, sc);
+            publish(hf, sc);
+          }
         }
         const float2 s = __fadd2_rn(__fadd2_rn(rs[0], rs[1]), __fadd2_rn(rs[2], rs[3]));
         l += s.x + s.y;
@@ -650,7 +760,8 @@ __global__ void __launch_bounds__(kThreads, 1)
   if (n_parts > 1) cluster_sync();  // (one part: the barrier above has ordered the exchange)
   if (warp < kKLoadWarp) {
     const int per_cta = dual ? 2 : 1, n_src = n_parts * per_cta;
-    const int x0 = rank * n_rows / n_parts, n_own = (rank + 1) * n_rows / n_parts - x0;  // this CTA's rows: x0 + [0, n_own)
+    // this CTA's rows: x0 + [0, n_own)
+    const int x0 = rank * n_rows / n_parts, n_own = (rank + 1) * n_rows / n_parts - x0;
     // source s of row x: CTA s (tile x / 128), or tile s & 1 of CTA s >> 1
     auto src_cta = [&](int s) { return (uint32_t)(dual ? s >> 1 : s); };
     auto src_tile = [&](int s, int x) { return dual ? s & 1 : x >> 7; };
@@ -862,12 +973,13 @@ cudaError_t launch_merge_t(const CUtensorMap& km, const CUtensorMap& vm, AttnPar
       }
     }
   }
+  const bool short_last = !host_items && n_items > 1 && p.T * p.G - (n_items - 1) * 2 * kTileRows <= kTileRows;
   for (int i = 0; i < 2 && layers[i] > 0; ++i) {
     p.kv_split = split[i];
     p.layer_base = i ? layers[0] : 0;
-    e = launch_chained_cluster(i ? merge_pair_kernel<D, false, true> : merge_pair_kernel<D, false, false>,
-                               dim3(n_items * split[i], p.Hkv, layers[i]), dim3(kThreads), PairCfg<D>::kSmemBytes, s,
-                               split[i], km, vm, p, kNoInline);
+    auto* kernel = i > 0 || short_last ? merge_pair_kernel<D, false, true> : merge_pair_kernel<D, false, false>;
+    e = launch_chained_cluster(kernel, dim3(n_items * split[i], p.Hkv, layers[i]), dim3(kThreads),
+                               PairCfg<D>::kSmemBytes, s, split[i], km, vm, p, kNoInline);
     if (e != cudaSuccess) return e;
     *n_launches = i + 1;
   }
@@ -880,8 +992,8 @@ cudaError_t launch_decode_pair_t(const CUtensorMap& km, const CUtensorMap& vm, c
   const PairSetup* ps = nullptr;
   cudaError_t e = pair_setup<D, true>(&ps);
   if (e != cudaSuccess) return e;
-  return launch_chained(merge_pair_kernel<D, true, false>, dim3(n_items, p.Hkv, p.L), dim3(kThreads), PairCfg<D>::kSmemBytes,
-                        s, km, vm, p, inl);
+  return launch_chained(merge_pair_kernel<D, true, false>, dim3(n_items, p.Hkv, p.L), dim3(kThreads),
+                        PairCfg<D>::kSmemBytes, s, km, vm, p, inl);
 }
 
 }  // namespace

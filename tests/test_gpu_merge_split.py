@@ -86,3 +86,10 @@ def test_layers_of_the_last_wave_in_a_launch_of_their_own(stlib):
         k, v = run.context(m, layer)
         o_ref, l_ref = A.merge_prefill(q[layer].cpu(), k, v, L0)
         compare(o[layer], lse[layer], o_ref, l_ref, f"layer {layer}")
+
+
+@pytest.mark.parametrize("D,ctx,T", [(128, 300, 70), (64, 300, 70), (128, 40, 130), (128, 5000, 85), (64, 5000, 85)])
+def test_short_last_tile_behind_the_others(stlib, D, ctx, T):
+    # 280, 520 and 340 stacked rows in 3 layers of 8 heads: the last tile of 24, 8
+    # and 84 rows comes behind the others of every head and layer, whole or split
+    _merge(D, 32, 8, ctx, T, L=3)
