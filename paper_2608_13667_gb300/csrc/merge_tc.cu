@@ -164,6 +164,32 @@ struct MergeSplitCost {
   float total, longest;  // of its CTAs together, of one of them
 };
 
+// A decode's run of pages of a fork group, for one KV head of one layer.
+struct PairWork {
+  AttnItem item;
+  int32_t kvh, layer;
+  int32_t valid;  // 0: no further one
+};
+
+// 16 rows x 64 columns of fp32 from tensor memory (taddr: the first of the 16
+// lanes): v[4 i ..] are columns 8 i + 2 (lane % 4) and the next of row lane / 4,
+// then the same of row lane / 4 + 8.
+__device__ __forceinline__ void tmem_ld_16x64(uint32_t taddr, float* v) {
+  uint32_t r[32];
+  asm volatile(
+      "tcgen05.ld.sync.aligned.16x256b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
+      "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];\n\t"
+      "tcgen05.wait::ld.sync.aligned;"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
+        "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
+        "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+      : "r"(taddr)
+      : "memory");
+#pragma unroll
+  for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
+}
+
 // 16 bytes from global to shared memory, asynchronously; zeros if !valid.
 __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, bool valid) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst),
@@ -197,7 +223,7 @@ struct PairCfg {
   static constexpr int kKOff = kQOff + 2 * kQTileBytes;
   static constexpr int kVOff = kKOff + kKStages * kSlotBytes;
   static constexpr int kBarOff = kVOff + kVStages * kSlotBytes;
-  static constexpr int kSmemBytes = 1024 + kBarOff + 256;
+  static constexpr int kSmemBytes = 1024 + kBarOff + 512;
   static_assert(kSmemBytes <= 227 * 1024, "shared memory of one CTA");
 };
 
@@ -207,12 +233,24 @@ struct PairCfg {
 // behind the other tiles of every head and layer, so that the launch ends on
 // the short ones (88 rows onto 8000 in 16 layers: 280 us before, 229).  A form
 // of its own, since the arithmetic in every launch cost half a per cent.
-template <int D, bool kDecode, bool kMapped>
+//
+// kPersist: a decode of more than one wave.  A run of pages is some 30 us here,
+// and a CTA of its own for each left its SM idle for 6 more, from the last P V
+// to the first of the next one.  So a CTA that is about to load its run's last
+// stage asks for a CTA of the grid that has not started (cluster launch
+// control) and goes on with its item: the next run's K and V land, its Q goes in
+// and its first S is computed while the results come out.  Stage and barrier
+// counts run on over a CTA's items; the K loader passes the items on through
+// two slots, which every role reads in order.  Two layers of 2 groups of 24
+// branches over 65536 tokens 316 -> 300 us, 17 branches in 4 layers 284 -> 263,
+// 41 in 4 layers 482 -> 424, D = 64 162 -> 145.
+template <int D, bool kDecode, bool kForm>
 __global__ void __launch_bounds__(kThreads, 1)
     merge_pair_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant__ CUtensorMap vmap,
                       const AttnParams p, const __grid_constant__ InlineDecodePlan inl) {
   using C = PairCfg<D>;
   constexpr int kKS = C::kKStages, kVS = C::kVStages;
+  constexpr bool kMapped = !kDecode && kForm, kPersist = kDecode && kForm;
   constexpr bool kHold = D == 128 && !kDecode;  // the softmax holds its scores (below)
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw = smem_addr(smem_raw);
@@ -226,7 +264,13 @@ __global__ void __launch_bounds__(kThreads, 1)
   uint64_t* p_full = s_full + 2;     // [2 tiles][2 key halves]
   uint64_t* o_final = p_full + 4;
   uint64_t* q_ready = o_final + 1;
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(q_ready + 1);
+  uint64_t* work_full = q_ready + 1;     // [2] kPersist: an item taken over is in its slot
+  uint64_t* work_empty = work_full + 2;  // [2] every role has read it
+  uint64_t* clc_bar = work_empty + 2;    // the answer to a request for one has landed
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(clc_bar + 1);
+  uint8_t* clc_resp = base + C::kBarOff + 320;  // 16 bytes
+  PairWork* work_slots = reinterpret_cast<PairWork*>(base + C::kBarOff + 336);  // [2]
+  static_assert(8 * (2 * kKS + 2 * kVS + 14) <= 320 && 336 + 2 * sizeof(PairWork) <= 512, "barrier area");
 
   const int warp = threadIdx.x >> 5;
   const int lane = threadIdx.x & 31;
@@ -253,6 +297,13 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
     mbar_init(o_final, 1);
     mbar_init(q_ready, kSoftThreads);
+    if constexpr (kPersist) {
+      for (int b = 0; b < 2; ++b) {
+        mbar_init(&work_full[b], 1);
+        mbar_init(&work_empty[b], 10);  // the V loader, the MMA warp and the softmax warps
+      }
+      mbar_init(clc_bar, 1);
+    }
     fence_mbar_init();
   }
   tc_fence_before_sync();
@@ -285,15 +336,21 @@ __global__ void __launch_bounds__(kThreads, 1)
   int page_begin = 0, n_rows, n_pages, n_valid_keys;
   AttnItem item{};
   const int32_t* members = nullptr;
-  if constexpr (kDecode) {
-    members = p.members ? p.members : inl.members;
-    item = p.items ? p.items[p.item_base + blockIdx.x] : inl.items[p.item_base + blockIdx.x];
+  auto item_at = [&](int x) -> const AttnItem& {
+    return p.items ? p.items[p.item_base + x] : inl.items[p.item_base + x];
+  };
+  auto take_item = [&](const AttnItem& it) {  // a decode's work of this thread's role
+    item = it;
     slot = item.slot;
     page_begin = item.page_begin;
     row_base = 0;
     n_rows = min(2 * kTileRows, item.n_members * G);
     n_pages = item.n_pages;
     n_valid_keys = item.n_tokens;
+  };
+  if constexpr (kDecode) {
+    members = p.members ? p.members : inl.members;
+    take_item(item_at(blockIdx.x));
   } else {
     if (p.mitems) {
       const MergeItem mi = p.mitems[blockIdx.x / cluster];
@@ -322,7 +379,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   // (the longer parts first: the last one has the stages at the causal limit,
   // whose masks cost it another microsecond or two)
   const int j0 = (rank * all_tiles + n_parts - 1) / n_parts, j1 = ((rank + 1) * all_tiles + n_parts - 1) / n_parts;
-  const int n_tiles = j1 - j0;
+  int n_tiles = j1 - j0;
   const int key_base = j0 * kKeys;
   page_begin += j0 * kPagesPerStage;
   n_pages = min(n_pages - j0 * kPagesPerStage, n_tiles * kPagesPerStage);
@@ -330,6 +387,23 @@ __global__ void __launch_bounds__(kThreads, 1)
   const bool dual = !kDecode && n_rows <= kTileRows;
   const bool direct = kDecode || (n_parts == 1 && !dual);  // every row has one source, its thread's
 
+  auto next_item = [&](const PairWork& w) {
+    take_item(w.item);
+    kvh = w.kvh;
+    layer = w.layer;
+    n_tiles = (n_pages + kPagesPerStage - 1) / kPagesPerStage;
+  };
+  // kPersist: the item after a role's n-th, which the K loader writes to slot n % 2.
+  // False when there is none (or the wait ran out: *ok).
+  auto next_work = [&](int n, PairWork* w, bool* ok) -> bool {
+    const int b = n & 1;
+    *ok = __all_sync(0xffffffffu, mbar_wait(&work_full[b], (n >> 1) & 1));
+    if (!*ok) return false;
+    *w = work_slots[b];
+    __syncwarp();
+    if (lane == 0) mbar_arrive(&work_empty[b]);
+    return w->valid != 0;
+  };
 
   if (warp >= kKLoadWarp) {
     if constexpr (kHold) regs_dec<kOtherRegs>();
@@ -343,54 +417,94 @@ __global__ void __launch_bounds__(kThreads, 1)
       const int n_st = is_k ? kKS : kVS;
       uint8_t* ring = base + (is_k ? C::kKOff : C::kVOff);
       if (lane == 0) prefetch_tensormap(map);
-      // merge: every CTA of one (layer, KV head) walks the same pages, keep them
-      // in L2; decode: a page is streamed once, unless a sibling subgroup's CTA
-      // reads it too or the whole launch fits in L2
-      const uint64_t policy = !kDecode ? l2_policy_evict_last()
-                              : (p.keep_l2 || (item.flags & kItemReread)) ? l2_policy_evict_normal()
-                                                                           : l2_policy_evict_first();
-      const int32_t* ids = p.table + (int64_t)slot * p.max_pages + page_begin;
-      int base_id = 0;
-      int cur = lane < n_pages ? ids[lane] : 0;
-      int nxt = 32 + lane < n_pages ? ids[32 + lane] : 0;
-      int j = 0;
+      int g = 0;  // stages whose copies have been issued, over all items
       bool ok = true;
-      for (; j < n_tiles; ++j) {
-        const int s = j % n_st;
-        if (j >= n_st) {
-          int w = 1;
-          if (lane == 0) w = mbar_wait(&empty[s], ((j / n_st) - 1) & 1) ? 1 : 0;
-          w = __shfl_sync(0xffffffffu, w, 0);
-          if (!w) {
-            ok = false;
+      for (int n = 0;; ++n) {  // the CTA's items
+        // merge: every CTA of one (layer, KV head) walks the same pages, keep them
+        // in L2; decode: a page is streamed once, unless a sibling subgroup's CTA
+        // reads it too or the whole launch fits in L2
+        const uint64_t policy = !kDecode ? l2_policy_evict_last()
+                                : (p.keep_l2 || (item.flags & kItemReread)) ? l2_policy_evict_normal()
+                                                                             : l2_policy_evict_first();
+        const int32_t* ids = p.table + (int64_t)slot * p.max_pages + page_begin;
+        int base_id = 0;
+        int cur = lane < n_pages ? ids[lane] : 0;
+        int nxt = 32 + lane < n_pages ? ids[32 + lane] : 0;
+        bool asked = false;
+        for (int j = 0; j < n_tiles; ++j, ++g) {
+          // ask for the next item no earlier than needed: one taken over sooner
+          // waits here while another SM may have run dry
+          if (kPersist && is_k && j == n_tiles - 1) {
+            asked = true;
+            if (lane == 0) {
+              mbar_arrive_expect_tx(clc_bar, 16);
+              clc_try_cancel(clc_resp, clc_bar);
+            }
+          }
+          const int s = g % n_st;
+          if (g >= n_st) {
+            int w = 1;
+            if (lane == 0) w = mbar_wait(&empty[s], ((g / n_st) - 1) & 1) ? 1 : 0;
+            w = __shfl_sync(0xffffffffu, w, 0);
+            if (!w) {
+              ok = false;
+              break;
+            }
+          }
+          const int page0 = j * kPagesPerStage;
+          if (page0 >= base_id + 32) {
+            base_id += 32;
+            cur = nxt;
+            nxt = base_id + 32 + lane < n_pages ? ids[base_id + 32 + lane] : 0;
+          }
+          const int np = min(kPagesPerStage, n_pages - page0);
+          uint8_t* dst = ring + s * C::kSlotBytes;
+          if (lane == 0) mbar_arrive_expect_tx(&full[s], (uint32_t)(np * C::kHalves * kPageTokens * 128));
+          __syncwarp();
+          // one copy per lane (lane = D/64 q + h)
+          const int q = lane / C::kHalves, h = lane % C::kHalves;
+          int b = __shfl_sync(0xffffffffu, cur, (page0 - base_id + (q < kPagesPerStage ? q : 0)) & 31);
+          if (lane < C::kHalves * np) {
+            if ((uint64_t)b >= (uint64_t)p.n_blocks) {
+              atomicCAS(p.status, 0, kDevBadIndex);
+              b = 0;
+            }
+            tma_load_4d(dst + h * C::kKVHalfBytes + q * kPageTokens * 128, map, &full[s], 0, h, kvh * kPageTokens,
+                        layer * (int)p.n_blocks + b, policy);
+          }
+        }
+        if constexpr (!kPersist) {
+          break;
+        } else {
+          PairWork w{};
+          if (is_k) {
+            uint32_t x = 0, y = 0, z = 0;
+            const bool answered = asked && __all_sync(0xffffffffu, mbar_wait(clc_bar, n & 1));
+            const bool more = answered && clc_answer(clc_resp, &x, &y, &z);
+            fence_proxy_async_smem();  // every lane has read the answer before the next one lands
+            __syncwarp();
+            if (more) w = PairWork{item_at(x), (int)y, (int)z, 1};
+            if (ok && answered && n >= 2) {  // the slot's last item has been read by every role
+              int e = 1;
+              if (lane == 0) e = mbar_wait(&work_empty[n & 1], ((n >> 1) - 1) & 1) ? 1 : 0;
+              ok = __shfl_sync(0xffffffffu, e, 0) != 0;
+            }
+            ok = ok && answered;
+            if (!ok) break;
+            if (lane == 0) {
+              work_slots[n & 1] = w;
+              mbar_arrive(&work_full[n & 1]);
+            }
+          } else if (!ok || !next_work(n, &w, &ok)) {
             break;
           }
-        }
-        const int page0 = j * kPagesPerStage;
-        if (page0 >= base_id + 32) {
-          base_id += 32;
-          cur = nxt;
-          nxt = base_id + 32 + lane < n_pages ? ids[base_id + 32 + lane] : 0;
-        }
-        const int np = min(kPagesPerStage, n_pages - page0);
-        uint8_t* dst = ring + s * C::kSlotBytes;
-        if (lane == 0) mbar_arrive_expect_tx(&full[s], (uint32_t)(np * C::kHalves * kPageTokens * 128));
-        __syncwarp();
-        // one copy per lane (lane = D/64 q + h)
-        const int q = lane / C::kHalves, h = lane % C::kHalves;
-        int b = __shfl_sync(0xffffffffu, cur, (page0 - base_id + (q < kPagesPerStage ? q : 0)) & 31);
-        if (lane < C::kHalves * np) {
-          if ((uint64_t)b >= (uint64_t)p.n_blocks) {
-            atomicCAS(p.status, 0, kDevBadIndex);
-            b = 0;
-          }
-          tma_load_4d(dst + h * C::kKVHalfBytes + q * kPageTokens * 128, map, &full[s], 0, h, kvh * kPageTokens,
-                      layer * (int)p.n_blocks + b, policy);
+          if (!w.valid) break;
+          next_item(w);
         }
       }
       if (!ok && lane == 0) {
         atomicCAS(p.status, 0, kDevTimeout);
-        for (int t = max(0, j - n_st); t < j; ++t) mbar_wait(&full[t % n_st], (t / n_st) & 1);
+        for (int t = max(0, g - n_st); t < g; ++t) mbar_wait(&full[t % n_st], (t / n_st) & 1);
       }
     }
 
@@ -409,8 +523,8 @@ __global__ void __launch_bounds__(kThreads, 1)
         const uint64_t q_desc = tc_desc_sw128(smem_addr(base + C::kQOff), 16, 1024);
         const uint64_t k_desc0 = tc_desc_sw128(smem_addr(base + C::kKOff), 16, 1024);
         const uint64_t v_desc0 = tc_desc_sw128(smem_addr(base + C::kVOff), C::kKVHalfBytes, 1024);
-        bool ok = __all_sync(0xffffffffu, mbar_wait(q_ready, 0));
-        tc_fence_after_sync();
+        bool ok = true;
+        int g0 = 0;  // the item's first stage among the CTA's
         // O_t += P_t(i) V, P_t(i) read from TMEM over S_t(i); each half of P
         // (64 keys) is published on its own, so the first half's MMAs run while
         // the softmax finishes the second
@@ -419,7 +533,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           const uint32_t acc0 = i > 0 ? 1u : 0u;
 #pragma unroll
           for (int hf = 0; hf < 2; ++hf) {
-            if (!__all_sync(0xffffffffu, mbar_wait(&p_full[2 * t + hf], i & 1))) return false;
+            if (!__all_sync(0xffffffffu, mbar_wait(&p_full[2 * t + hf], (g0 + i) & 1))) return false;
             tc_fence_after_sync();
 #pragma unroll
             for (int kq = 0; kq < kKeys / 32; ++kq) {
@@ -447,56 +561,68 @@ __global__ void __launch_bounds__(kThreads, 1)
         const std::integral_constant<int, 0> tile_a;
         const std::integral_constant<int, 1> tile_b;
         const uint64_t qd_b = q_desc + (uint64_t)(C::kQTileBytes >> 4);
-        if (!dual) {
-          // iteration i of both tiles is stage i
-          auto pv = [&](auto tile, int i) -> bool {
-            constexpr int t = decltype(tile)::value;
-            const int s = i % kVS;
-            if (t == 0 && !__all_sync(0xffffffffu, mbar_wait(&v_full[s], (i / kVS) & 1))) return false;
-            if (!issue_pv(tile, i, v_desc0 + (uint64_t)((s * C::kSlotBytes) >> 4))) return false;
-            if (t == 1) tc_commit_elect(&v_empty[s]);
-            return true;
-          };
-          for (int i = 0; ok && i < n_tiles; ++i) {
-            const int s = i % kKS;
-            const uint64_t kd = k_desc0 + (uint64_t)((s * C::kSlotBytes) >> 4);
-            ok = (i == 0 || pv(tile_a, i - 1)) && __all_sync(0xffffffffu, mbar_wait(&k_full[s], (i / kKS) & 1));
-            if (!ok) break;
-            tc_fence_after_sync();
-            issue_s(tile_a, q_desc, kd);
-            if (i > 0 && !pv(tile_b, i - 1)) {
-              ok = false;
-              break;
+        for (int n = 0;; ++n) {  // the CTA's items
+          ok = __all_sync(0xffffffffu, mbar_wait(q_ready, n & 1));
+          tc_fence_after_sync();
+          if (!dual) {
+            // iteration i of both tiles is stage i
+            auto pv = [&](auto tile, int i) -> bool {
+              constexpr int t = decltype(tile)::value;
+              const int g = g0 + i, s = g % kVS;
+              if (t == 0 && !__all_sync(0xffffffffu, mbar_wait(&v_full[s], (g / kVS) & 1))) return false;
+              if (!issue_pv(tile, i, v_desc0 + (uint64_t)((s * C::kSlotBytes) >> 4))) return false;
+              if (t == 1) tc_commit_elect(&v_empty[s]);
+              return true;
+            };
+            for (int i = 0; ok && i < n_tiles; ++i) {
+              const int g = g0 + i, s = g % kKS;
+              const uint64_t kd = k_desc0 + (uint64_t)((s * C::kSlotBytes) >> 4);
+              ok = (i == 0 || pv(tile_a, i - 1)) && __all_sync(0xffffffffu, mbar_wait(&k_full[s], (g / kKS) & 1));
+              if (!ok) break;
+              tc_fence_after_sync();
+              issue_s(tile_a, q_desc, kd);
+              if (i > 0 && !pv(tile_b, i - 1)) {
+                ok = false;
+                break;
+              }
+              issue_s(tile_b, qd_b, kd);
+              tc_commit_elect(&k_empty[s]);
             }
-            issue_s(tile_b, qd_b, kd);
-            tc_commit_elect(&k_empty[s]);
+            if (ok && n_tiles > 0) ok = pv(tile_a, n_tiles - 1) && pv(tile_b, n_tiles - 1);
+          } else {
+            // iteration i of tile t is stage 2 i + t, its own K and V slot; of an
+            // odd number of stages B has one fewer
+            auto pv = [&](auto tile, int i) -> bool {
+              const int j = 2 * i + decltype(tile)::value, s = j % kVS;
+              if (!__all_sync(0xffffffffu, mbar_wait(&v_full[s], (j / kVS) & 1))) return false;
+              if (!issue_pv(tile, i, v_desc0 + (uint64_t)((s * C::kSlotBytes) >> 4))) return false;
+              tc_commit_elect(&v_empty[s]);
+              return true;
+            };
+            auto qk = [&](auto tile, int i) -> bool {
+              const int j = 2 * i + decltype(tile)::value, s = j % kKS;
+              if (!__all_sync(0xffffffffu, mbar_wait(&k_full[s], (j / kKS) & 1))) return false;
+              tc_fence_after_sync();
+              issue_s(tile, q_desc, k_desc0 + (uint64_t)((s * C::kSlotBytes) >> 4));
+              tc_commit_elect(&k_empty[s]);
+              return true;
+            };
+            const int n_a = (n_tiles + 1) / 2, n_b = n_tiles / 2;
+            for (int i = 0; ok && i < n_a; ++i)
+              ok = (i == 0 || pv(tile_a, i - 1)) && qk(tile_a, i) && (i == 0 || pv(tile_b, i - 1)) &&
+                   (i >= n_b || qk(tile_b, i));
+            if (ok && n_a > 0) ok = pv(tile_a, n_a - 1) && (n_b < n_a || pv(tile_b, n_b - 1));
           }
-          if (ok && n_tiles > 0) ok = pv(tile_a, n_tiles - 1) && pv(tile_b, n_tiles - 1);
-        } else {
-          // iteration i of tile t is stage 2 i + t, its own K and V slot; of an
-          // odd number of stages B has one fewer
-          auto pv = [&](auto tile, int i) -> bool {
-            const int j = 2 * i + decltype(tile)::value, s = j % kVS;
-            if (!__all_sync(0xffffffffu, mbar_wait(&v_full[s], (j / kVS) & 1))) return false;
-            if (!issue_pv(tile, i, v_desc0 + (uint64_t)((s * C::kSlotBytes) >> 4))) return false;
-            tc_commit_elect(&v_empty[s]);
-            return true;
-          };
-          auto qk = [&](auto tile, int i) -> bool {
-            const int j = 2 * i + decltype(tile)::value, s = j % kKS;
-            if (!__all_sync(0xffffffffu, mbar_wait(&k_full[s], (j / kKS) & 1))) return false;
-            tc_fence_after_sync();
-            issue_s(tile, q_desc, k_desc0 + (uint64_t)((s * C::kSlotBytes) >> 4));
-            tc_commit_elect(&k_empty[s]);
-            return true;
-          };
-          const int n_a = (n_tiles + 1) / 2, n_b = n_tiles / 2;
-          for (int i = 0; ok && i < n_a; ++i)
-            ok = (i == 0 || pv(tile_a, i - 1)) && qk(tile_a, i) && (i == 0 || pv(tile_b, i - 1)) &&
-                 (i >= n_b || qk(tile_b, i));
-          if (ok && n_a > 0) ok = pv(tile_a, n_a - 1) && (n_b < n_a || pv(tile_b, n_b - 1));
+          tc_commit_elect(o_final);
+          if constexpr (!kPersist) {
+            break;
+          } else {
+            g0 += n_tiles;
+            PairWork w;
+            if (!ok || !next_work(n, &w, &ok)) break;
+            next_item(w);
+          }
         }
-        tc_commit_elect(o_final);
         if (!ok && lane == 0) atomicCAS(p.status, 0, kDevTimeout);
       }
       __syncwarp();
@@ -516,14 +642,21 @@ __global__ void __launch_bounds__(kThreads, 1)
   const int t = warp >> 2;               // tile (of a softmax warp)
   const int r = (warp & 3) * 32 + lane;  // row within the tile = TMEM lane
   const int tile_row0 = row_base + (dual ? 0 : t * kTileRows);
-  const bool valid = warp < kKLoadWarp && tile_row0 - row_base + r < n_rows;
-  int qrow = 0, head = 0;
-  if (valid) {
-    const int gr = tile_row0 + r;
-    qrow = kDecode ? members[item.member_base + gr / G] : gr / G;
-    head = kvh * G + gr % G;
-  }
-  const int64_t io_row = (int64_t)layer * p.n_rows_q + q_row0 + qrow;  // this row in Q / O / LSE
+  bool valid;
+  int qrow;
+  int64_t in_row;  // this row in Q / O / LSE
+  auto find_row = [&]() {
+    int head = 0;
+    valid = tile_row0 - row_base + r < n_rows;
+    qrow = 0;
+    if (valid) {
+      const int gr = tile_row0 + r;
+      qrow = kDecode ? members[item.member_base + gr / G] : gr / G;
+      head = kvh * G + gr % G;
+    }
+    in_row = ((int64_t)layer * p.n_rows_q + q_row0 + qrow) * p.Hq + head;
+  };
+  find_row();
   // Results on their way out, over the K, V and Q buffers once every MMA has
   // completed: xo [2 tiles][128 rows][D/4] float4 of the unnormalised O (xo_at:
   // columns swizzled by the row, so that a warp reads or writes a column of 32
@@ -538,17 +671,13 @@ __global__ void __launch_bounds__(kThreads, 1)
   float* xwt = reinterpret_cast<float*>(xw + 4 * kTileRows);
   int64_t* xrow = reinterpret_cast<int64_t*>(xw + 8 * kTileRows);
   auto xo_at = [&](int tile, int row, int c) { return (tile * kTileRows + row) * kQuads + (c ^ (row & (kQuads - 1))); };
-  const int64_t in_row = io_row * p.Hq + head;
   static_assert(2 * kTileRows * D * 4 <= C::kBarOff - C::kKOff, "the exchange fits the K and V rings");
 
   bool ok = true;
-  if (warp < kKLoadWarp) {
+  {
     const int tid = threadIdx.x & (kTileRows - 1);
     const uint32_t t_lane = tmem + ((uint32_t)((warp & 3) * 32) << 16) + t * kTmemTile;
-    // causal limit of this row (a decode row sees the whole run)
-    const int limit = kDecode ? n_valid_keys : valid ? L0 + qrow + 1 : n_valid_keys;
-    const int min_limit = kDecode ? n_valid_keys : L0 + tile_row0 / G + 1;  // the tile's first row sees the fewest keys
-    if (!dual || t == 0) {
+    auto load_q = [&]() {
       // D/8 lanes copy a row's D contiguous values, straight to shared memory:
       // all 32 rows of the warp are in flight at once (a thread loading its own
       // row through registers took 4.7 us for the tile, this 1.9)
@@ -565,147 +694,213 @@ __global__ void __launch_bounds__(kThreads, 1)
       }
       cp_async_wait();
       fence_proxy_async_smem();
-    }
+    };
+    if (!dual || t == 0) load_q();
     mbar_arrive(q_ready);
 
     const float sl2 = p.scale_log2;
-    float m_used = -1e30f, l = 0.f;
-    const int n_it = dual ? (n_tiles + 1 - t) / 2 : n_tiles;
-    for (int it = 0; it < n_it; ++it) {
-      const int j = dual ? 2 * it + t : it;  // the stage
-      if (!__all_sync(0xffffffffu, mbar_wait(&s_full[t], it & 1))) {
-        ok = false;
-        break;
-      }
-      tc_fence_after_sync();
-      const int key0 = key_base + j * kKeys;
-      const int loaded = min(kPagesPerStage, n_pages - j * kPagesPerStage) * kPageTokens;
-      const bool edge = key0 + kKeys > min_limit || loaded < kKeys;
-      const int n_seen = min(loaded, limit - key0);  // this row's keys of the stage
-      // scores of keys [hf * 64, hf * 64 + 64), masked past the stage's pages and
-      // past this row's causal limit
-      auto load_half = [&](int hf, float* sc) {
-        tmem_ld64(t_lane + hf * 64, sc);
-        if (edge) {
-#pragma unroll
-          for (int c = 0; c < 64; ++c)
-            if (c >= n_seen - hf * 64) sc[c] = -INFINITY;
-        }
-      };
-      // With kHold the row's scores stay in registers from the maximum to the
-      // probabilities: reading them twice takes tensor-memory bandwidth from
-      // the MMAs (4 layers of 2048 rows: 1980 us reading twice, 1942 holding;
-      // D = 64, whose MMAs leave the softmax the longer chain, and the decode
-      // are faster with the shorter code that reads twice).
-      float held[kHold ? kKeys : 1];
-      float mx;
-      if constexpr (kHold) {
-        tmem_ld128(t_lane, held);
-        if (edge) {
-#pragma unroll
-          for (int c = 0; c < kKeys; ++c)
-            if (c >= n_seen) held[c] = -INFINITY;
-        }
-        float mx8[8];
-#pragma unroll
-        for (int i = 0; i < 8; ++i) mx8[i] = fmaxf(held[i], held[8 + i]);
-#pragma unroll
-        for (int c = 16; c < kKeys; c += 16)
-#pragma unroll
-          for (int i = 0; i < 8; ++i) mx8[i] = fmax3(mx8[i], held[c + i], held[c + 8 + i]);
-        mx = fmax3(fmax3(mx8[0], mx8[1], mx8[2]), fmax3(mx8[3], mx8[4], mx8[5]), fmaxf(mx8[6], mx8[7]));
-      } else {
-        // row max over both halves: independent chains of three-input max
-        float mx8[8];
-#pragma unroll
-        for (int i = 0; i < 8; ++i) mx8[i] = -INFINITY;
-#pragma unroll 1  // one half's scores live at a time
-        for (int hf = 0; hf < 2; ++hf) {
-          float sc[64];
-          load_half(hf, sc);
-#pragma unroll
-          for (int c = 0; c < 64; c += 16)
-#pragma unroll
-            for (int i = 0; i < 8; ++i) mx8[i] = fmax3(mx8[i], sc[c + i], sc[c + 8 + i]);
-        }
-        mx = fmax3(fmax3(mx8[0], mx8[1], mx8[2]), fmax3(mx8[3], mx8[4], mx8[5]), fmaxf(mx8[6], mx8[7]));
-      }
-      const float m_new = fmaxf(m_used, mx * sl2);  // sl2 > 0: max commutes with the scale
-      const bool need = valid && m_new > m_used + kRescaleThreshold;
-      if (__any_sync(0xffffffffu, need)) {
-        const float alpha = need ? ex2(m_used - m_new) : 1.f;
-        if (it > 0) {
-          // the O_t += P_t V before has completed (covered by the commit of this S_t)
-#pragma unroll 1
-          for (int k = 0; k < D / 32; ++k) {
-            float o[32];
-            tmem_ld32(t_lane + kTmemO + k * 32, o);
-#pragma unroll
-            for (int i = 0; i < 32; ++i) o[i] *= alpha;
-            tmem_st32(t_lane + kTmemO + k * 32, o);
-          }
-        }
-        l *= alpha;
-        if (need) m_used = m_new;
-      }
-      if ((t == 0 || dual) && (key0 + kKeys > n_valid_keys || loaded < kKeys)) {
-        // zero the V rows of keys that are not valid once the stage's copies
-        // have landed; the P V that read the stage are issued after this tile's
-        // first P half
-        const int s = j % kVS;
-        if (!__all_sync(0xffffffffu, mbar_wait(&v_full[s], (j / kVS) & 1))) {
+    float m_used, l;
+    int n_it, g0 = 0;  // the item's stages of this tile, the first one's number among the CTA's
+    for (int n = 0;; ++n) {  // the CTA's items
+      // causal limit of this row (a decode row sees the whole run)
+      const int limit = kDecode ? n_valid_keys : valid ? L0 + qrow + 1 : n_valid_keys;
+      const int min_limit = kDecode ? n_valid_keys : L0 + tile_row0 / G + 1;  // the tile's first row sees the fewest keys
+      m_used = -1e30f;
+      l = 0.f;
+      n_it = dual ? (n_tiles + 1 - t) / 2 : n_tiles;
+      for (int it = 0; it < n_it; ++it) {
+        const int j = dual ? 2 * it + t : it;  // the stage
+        if (!__all_sync(0xffffffffu, mbar_wait(&s_full[t], (g0 + it) & 1))) {
           ok = false;
           break;
         }
-        uint8_t* vslot = base + C::kVOff + s * C::kSlotBytes;
-        for (int x = tid; x < kKeys * C::kHalves; x += kTileRows) {
-          const int c = x % kKeys, h = x / kKeys;
-          if (c >= loaded || key0 + c >= n_valid_keys) {
+        tc_fence_after_sync();
+        const int key0 = key_base + j * kKeys;
+        const int loaded = min(kPagesPerStage, n_pages - j * kPagesPerStage) * kPageTokens;
+        const bool edge = key0 + kKeys > min_limit || loaded < kKeys;
+        const int n_seen = min(loaded, limit - key0);  // this row's keys of the stage
+        // scores of keys [hf * 64, hf * 64 + 64), masked past the stage's pages and
+        // past this row's causal limit
+        auto load_half = [&](int hf, float* sc) {
+          tmem_ld64(t_lane + hf * 64, sc);
+          if (edge) {
 #pragma unroll
-            for (int y = 0; y < 8; ++y)
-              *reinterpret_cast<uint4*>(vslot + h * C::kKVHalfBytes + c * 128 + y * 16) = make_uint4(0u, 0u, 0u, 0u);
+            for (int c = 0; c < 64; ++c)
+              if (c >= n_seen - hf * 64) sc[c] = -INFINITY;
           }
-        }
-        fence_proxy_async_smem();
-      }
-      // P = 2^(s sl2 - m) (two keys per packed f32x2 FMA / add) as two bf16
-      // terms, P_hi = bf16(P) and P_lo = bf16(P - P_hi), so that P V is exact to
-      // about 16 bits whatever the spread of the scores.  The 16 score columns
-      // of keys [16 ks, 16 ks + 16) take P_hi of those keys (8 columns of bf16
-      // pairs) and then P_lo (8 columns): each store overwrites only scores
-      // already read.
-      {
-        const float2 scale2 = make_float2(sl2, sl2), neg_m2 = make_float2(-m_used, -m_used);
-        float2 rs[4] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
-        // one half's P from its scores, published
-        auto publish = [&](int hf, const float* sc) {
-#pragma unroll
-          for (int kq = 0; kq < 4; ++kq) {  // 16 keys per step
-            uint32_t pk[16];
-#pragma unroll
-            for (int c = 0; c < 16; c += 2)
-              prob_pair(sc[kq * 16 + c], sc[kq * 16 + c + 1], scale2, neg_m2, &rs[(c >> 1) & 3], &pk[c / 2],
-                        &pk[8 + c / 2]);
-            tmem_st16u_nowait(t_lane + (hf * 4 + kq) * 16, pk);
-          }
-          tmem_wait_st();
-          tc_fence_before_sync();
-          mbar_arrive(&p_full[2 * t + hf]);
         };
+        // With kHold the row's scores stay in registers from the maximum to the
+        // probabilities: reading them twice takes tensor-memory bandwidth from
+        // the MMAs (4 layers of 2048 rows: 1980 us reading twice, 1942 holding;
+        // D = 64, whose MMAs leave the softmax the longer chain, and the decode
+        // are faster with the shorter code that reads twice).
+        float held[kHold ? kKeys : 1];
+        float mx;
         if constexpr (kHold) {
-          publish(0, held);
-          publish(1, held + 64);
+          tmem_ld128(t_lane, held);
+          if (edge) {
+#pragma unroll
+            for (int c = 0; c < kKeys; ++c)
+              if (c >= n_seen) held[c] = -INFINITY;
+          }
+          float mx8[8];
+#pragma unroll
+          for (int i = 0; i < 8; ++i) mx8[i] = fmaxf(held[i], held[8 + i]);
+#pragma unroll
+          for (int c = 16; c < kKeys; c += 16)
+#pragma unroll
+            for (int i = 0; i < 8; ++i) mx8[i] = fmax3(mx8[i], held[c + i], held[c + 8 + i]);
+          mx = fmax3(fmax3(mx8[0], mx8[1], mx8[2]), fmax3(mx8[3], mx8[4], mx8[5]), fmaxf(mx8[6], mx8[7]));
         } else {
-#pragma unroll 1
+          // row max over both halves: independent chains of three-input max
+          float mx8[8];
+#pragma unroll
+          for (int i = 0; i < 8; ++i) mx8[i] = -INFINITY;
+#pragma unroll 1  // one half's scores live at a time
           for (int hf = 0; hf < 2; ++hf) {
             float sc[64];
             load_half(hf, sc);
-            publish(hf, sc);
+#pragma unroll
+            for (int c = 0; c < 64; c += 16)
+#pragma unroll
+              for (int i = 0; i < 8; ++i) mx8[i] = fmax3(mx8[i], sc[c + i], sc[c + 8 + i]);
+          }
+          mx = fmax3(fmax3(mx8[0], mx8[1], mx8[2]), fmax3(mx8[3], mx8[4], mx8[5]), fmaxf(mx8[6], mx8[7]));
+        }
+        const float m_new = fmaxf(m_used, mx * sl2);  // sl2 > 0: max commutes with the scale
+        const bool need = valid && m_new > m_used + kRescaleThreshold;
+        if (__any_sync(0xffffffffu, need)) {
+          const float alpha = need ? ex2(m_used - m_new) : 1.f;
+          if (it > 0) {
+            // the O_t += P_t V before has completed (covered by the commit of this S_t)
+#pragma unroll 1
+            for (int k = 0; k < D / 32; ++k) {
+              float o[32];
+              tmem_ld32(t_lane + kTmemO + k * 32, o);
+#pragma unroll
+              for (int i = 0; i < 32; ++i) o[i] *= alpha;
+              tmem_st32(t_lane + kTmemO + k * 32, o);
+            }
+          }
+          l *= alpha;
+          if (need) m_used = m_new;
+        }
+        if ((t == 0 || dual) && (key0 + kKeys > n_valid_keys || loaded < kKeys)) {
+          // zero the V rows of keys that are not valid once the stage's copies
+          // have landed; the P V that read the stage are issued after this tile's
+          // first P half
+          const int g = g0 + j, s = g % kVS;
+          if (!__all_sync(0xffffffffu, mbar_wait(&v_full[s], (g / kVS) & 1))) {
+            ok = false;
+            break;
+          }
+          uint8_t* vslot = base + C::kVOff + s * C::kSlotBytes;
+          for (int x = tid; x < kKeys * C::kHalves; x += kTileRows) {
+            const int c = x % kKeys, h = x / kKeys;
+            if (c >= loaded || key0 + c >= n_valid_keys) {
+#pragma unroll
+              for (int y = 0; y < 8; ++y)
+                *reinterpret_cast<uint4*>(vslot + h * C::kKVHalfBytes + c * 128 + y * 16) = make_uint4(0u, 0u, 0u, 0u);
+            }
+          }
+          fence_proxy_async_smem();
+        }
+        // P = 2^(s sl2 - m) (two keys per packed f32x2 FMA / add) as two bf16
+        // terms, P_hi = bf16(P) and P_lo = bf16(P - P_hi), so that P V is exact to
+        // about 16 bits whatever the spread of the scores.  The 16 score columns
+        // of keys [16 ks, 16 ks + 16) take P_hi of those keys (8 columns of bf16
+        // pairs) and then P_lo (8 columns): each store overwrites only scores
+        // already read.
+        {
+          const float2 scale2 = make_float2(sl2, sl2), neg_m2 = make_float2(-m_used, -m_used);
+          float2 rs[4] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+          // one half's P from its scores, published
+          auto publish = [&](int hf, const float* sc) {
+#pragma unroll
+            for (int kq = 0; kq < 4; ++kq) {  // 16 keys per step
+              uint32_t pk[16];
+#pragma unroll
+              for (int c = 0; c < 16; c += 2)
+                prob_pair(sc[kq * 16 + c], sc[kq * 16 + c + 1], scale2, neg_m2, &rs[(c >> 1) & 3], &pk[c / 2],
+                          &pk[8 + c / 2]);
+              tmem_st16u_nowait(t_lane + (hf * 4 + kq) * 16, pk);
+            }
+            tmem_wait_st();
+            tc_fence_before_sync();
+            mbar_arrive(&p_full[2 * t + hf]);
+          };
+          if constexpr (kHold) {
+            publish(0, held);
+            publish(1, held + 64);
+          } else {
+#pragma unroll 1
+            for (int hf = 0; hf < 2; ++hf) {
+              float sc[64];
+              load_half(hf, sc);
+              publish(hf, sc);
+            }
+          }
+          const float2 s = __fadd2_rn(__fadd2_rn(rs[0], rs[1]), __fadd2_rn(rs[2], rs[3]));
+          l += s.x + s.y;
+        }
+      }
+      if constexpr (!kPersist) {
+        break;
+      } else {
+        if (!ok) break;
+        // the next item's Q goes in before this one's results come out: its S
+        // (every S of this tile has been computed) runs meanwhile.  Its first P V
+        // waits for this thread's P, behind the results.
+        const int64_t out_row = valid ? in_row * p.max_splits + item.split : -1;
+        PairWork next;
+        const bool more = next_work(n, &next, &ok);
+        if (!ok) break;
+        if (more) {
+          g0 += n_tiles;
+          next_item(next);
+          find_row();
+          load_q();
+          mbar_arrive(q_ready);
+        }
+        if (!__all_sync(0xffffffffu, mbar_wait(o_final, n & 1))) {
+          ok = false;
+          break;
+        }
+        tc_fence_after_sync();
+        // straight from tensor memory, whole 32-byte sectors: four lanes have 8
+        // columns of a row (the next item's stages are landing in the buffers
+        // through which a single item's results leave)
+        const float inv = 1.f / l;
+#pragma unroll 1
+        for (int hf = 0; hf < 2; ++hf) {
+          const int ra = 16 * hf + lane / 4;  // of the warp's 32 rows; the other one is ra + 8
+          const float inv_a = __shfl_sync(0xffffffffu, inv, ra), inv_b = __shfl_sync(0xffffffffu, inv, ra + 8);
+          const int64_t to_a = __shfl_sync(0xffffffffu, out_row, ra), to_b = __shfl_sync(0xffffffffu, out_row, ra + 8);
+#pragma unroll 1
+          for (int k = 0; k < D / 64; ++k) {
+            float o[32];
+            tmem_ld_16x64(t_lane + ((uint32_t)(16 * hf) << 16) + kTmemO + 64 * k, o);
+            const int c = 64 * k + 2 * (lane % 4);
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+              if (to_a >= 0)
+                *reinterpret_cast<float2*>(p.out_o + to_a * D + c + 8 * i) =
+                    make_float2(o[4 * i] * inv_a, o[4 * i + 1] * inv_a);
+              if (to_b >= 0)
+                *reinterpret_cast<float2*>(p.out_o + to_b * D + c + 8 * i) =
+                    make_float2(o[4 * i + 2] * inv_b, o[4 * i + 3] * inv_b);
+            }
           }
         }
-        const float2 s = __fadd2_rn(__fadd2_rn(rs[0], rs[1]), __fadd2_rn(rs[2], rs[3]));
-        l += s.x + s.y;
+        if (out_row >= 0) p.out_lse[out_row] = (m_used + log2f(l)) * kLn2;
+        if (!more) break;
       }
+    }
+    if constexpr (kPersist) {
+      if (!ok && lane == 0) atomicCAS(p.status, 0, kDevTimeout);
+      tc_fence_before_sync();
+      named_barrier_sync(1, kSoftThreads + 32);
+      return;
     }
     if (ok) ok = __all_sync(0xffffffffu, mbar_wait(o_final, 0));
     tc_fence_after_sync();
@@ -758,7 +953,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   // instructions: loops are kept rolled (a version with 16 loads in flight
   // took 12 us where the same work rolled took 5).
   if (n_parts > 1) cluster_sync();  // (one part: the barrier above has ordered the exchange)
-  if (warp < kKLoadWarp) {
+  {
     const int per_cta = dual ? 2 : 1, n_src = n_parts * per_cta;
     // this CTA's rows: x0 + [0, n_own)
     const int x0 = rank * n_rows / n_parts, n_own = (rank + 1) * n_rows / n_parts - x0;
@@ -843,6 +1038,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 // leaves over stay idle; 0: the size is not available).
 struct PairSetup {
   bool done = false;
+  int sms = 0;
   int resident[kMaxMergeSplit + 1] = {};
 };
 
@@ -858,14 +1054,16 @@ cudaError_t pair_setup(const PairSetup** out) {
   PairSetup& ps = setups[dev];
   std::lock_guard<std::mutex> lock(mu);
   if (!ps.done) {
-    auto* kernel = merge_pair_kernel<D, kDecode, false>;
-    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmemBytes);
+    e = cudaDeviceGetAttribute(&ps.sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
-    if constexpr (!kDecode) {
-      auto* rest = merge_pair_kernel<D, false, true>;
-      e = cudaFuncSetAttribute(rest, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmemBytes);
+    auto* kernel = merge_pair_kernel<D, kDecode, false>;
+    auto* other = merge_pair_kernel<D, kDecode, true>;
+    for (auto* k : {kernel, other}) {
+      e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmemBytes);
       if (e != cudaSuccess) return e;
-      for (auto* k : {kernel, rest}) {
+    }
+    if constexpr (!kDecode) {
+      for (auto* k : {kernel, other}) {
         e = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
         if (e != cudaSuccess) return e;
       }
@@ -992,7 +1190,11 @@ cudaError_t launch_decode_pair_t(const CUtensorMap& km, const CUtensorMap& vm, c
   const PairSetup* ps = nullptr;
   cudaError_t e = pair_setup<D, true>(&ps);
   if (e != cudaSuccess) return e;
-  return launch_chained(merge_pair_kernel<D, true, false>, dim3(n_items, p.Hkv, p.L), dim3(kThreads),
+  // CTAs that take over further items where there is more than one wave of
+  // them, one CTA per SM; within one wave there is nothing to take over
+  auto* kernel = (int64_t)n_items * p.Hkv * p.L > ps->sms ? merge_pair_kernel<D, true, true>
+                                                          : merge_pair_kernel<D, true, false>;
+  return launch_chained(kernel, dim3(n_items, p.Hkv, p.L), dim3(kThreads),
                         PairCfg<D>::kSmemBytes, s, km, vm, p, inl);
 }
 

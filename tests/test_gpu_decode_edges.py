@@ -102,3 +102,29 @@ def test_many_short_items_beside_a_wide_tile(stlib):
         for layer in (0, L - 1):
             o_ref, l_ref = run.oracle_decode(rids, q, layer)
             compare(o[layer], lse[layer], o_ref, l_ref, f"step {step} layer {layer}")
+
+
+@pytest.mark.parametrize("D", [64, 128])
+def test_paired_items_taken_over(stlib, D):
+    """More than one wave of CTAs on the paired tile, so that each takes over
+    further items: runs of one page to many, short last stages, one row to all
+    128 in the second tile, and a group split into two."""
+    L = 12
+    w = Workload(name=f"paired_taken_{D}", n_layers=L, n_q_heads=64, n_kv_heads=8, head_dim=D, n_blocks=2048, seed=64)
+    run = Run(w, max_seqs=192, max_decode_branches=160, max_splits=16)
+    rids = []
+    for g, (prefix, n_aux) in enumerate(((2000, 16), (16, 31), (6016, 23), (130 * 16, 40), (144, 20))):
+        m = run.create()
+        run.append([m], prefix, ("prefix", g))
+        family = [m] + run.fork(m, n_aux)
+        run.append(family[::2], 3 + g, ("suffix", g))
+        rids += family
+    items, _, _ = run.pool.decode_plan([run.handle[r] for r in rids])
+    paired = [it for it in items if it["n_members"] * 8 > 128]
+    assert len(paired) * 8 * L > 2 * 152 and len({it["n_pages"] for it in paired}) > 2
+    for step in range(2):     # the rings and the slots start anew with every launch
+        q, o, lse = run.decode(rids, ("q", step))
+        run.pool.sync()
+        for layer in (0, L - 1):
+            o_ref, l_ref = run.oracle_decode(rids, q, layer)
+            compare(o[layer], lse[layer], o_ref, l_ref, f"step {step} layer {layer}")
