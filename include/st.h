@@ -286,8 +286,9 @@ typedef struct {
   double total_ms;     /* summed event time (0 when timing was off) */
   double bytes;        /* algorithmic bytes the launches had to move */
   double flops;        /* algorithmic floating-point operations */
-  int64_t kernels;     /* device kernels launched (a decode call with both tile
-                          shapes launches two per call) */
+  int64_t kernels;     /* device kernels launched (a decode call with several tile
+                          shapes launches one for each; a merge whose last
+                          layers are split among more CTAs launches two) */
   double overhead_bytes; /* bytes moved beyond the algorithmic ones: split-KV
                             partials (written by the decode, read by the
                             combine), second reads of a split fork family's

@@ -3,8 +3,8 @@
 // The host side is authoritative: the block pool (block_pool.cpp) decides
 // every allocation, and each call turns its decision into a small plan that
 // the kernels of that call consume -- inside their parameter block when it is
-// small (the common decode step), else copied to the device through a pinned
-// staging ring.  Planning for st_decode_attn groups the branches of a
+// small (the common decode step), else in a pinned staging ring, from which a
+// kernel brings it to the device or reads it in place.  Planning for st_decode_attn groups the branches of a
 // call by fork family and finds the pages they share, so the kernels read a
 // shared prefix page once per group (Section 3.3 of the paper).
 #include <cudaTypedefs.h>
