@@ -750,49 +750,42 @@ __global__ void __launch_bounds__(kThreads, 2)
       }
       tc_fence_after_sync();
       if constexpr (kPair) l += __shfl_xor_sync(0xffffffffu, l, 16);  // the row's full sum
+      // Four lanes have 8 columns of a row: every store fills whole 32-byte
+      // sectors of 8 rows (a thread writing its own row touches 32 rows per
+      // store, half a sector each).  Narrow: O = O_hi + O_lo, from a row's two
+      // lanes in the same places of two loads.  One layer of 9 branches over 16384
+      // tokens 25.0 -> 23.5 us, 20 branches, D 64, 312 -> 299, 16 branches 452 ->
+      // 443, 5 branches over 8192 tokens 14.2 -> 13.8.
       const float inv = 1.f / l;
-      float* dst = nullptr;
-      float* dst_lse = nullptr;
-      if (valid) {
-        const int64_t idx = row * p.max_splits + work.item.split;
-        dst = p.out_o + idx * D;
-        if (half == 0) dst_lse = p.out_lse + idx;
-      }
-      if constexpr (kPair) {
-        // O = O_hi + O_lo: thread t writes columns [0, D/2) of the row, thread
-        // t + 16 columns [D/2, D); one shuffle per column pair swaps the halves
-        // each needs from the other's lane
+      const int64_t to = valid ? row * p.max_splits + work.item.split : -1;
+#pragma unroll 1
+      for (int hf = 0; hf < (kPair ? 1 : 2); ++hf) {
+        const int ra = 16 * hf + lane / 4;  // of the warp's rows; the other one is ra + 8
+        const float inv_a = __shfl_sync(0xffffffffu, inv, ra), inv_b = __shfl_sync(0xffffffffu, inv, ra + 8);
+        const int64_t to_a = __shfl_sync(0xffffffffu, to, ra), to_b = __shfl_sync(0xffffffffu, to, ra + 8);
 #pragma unroll 1
         for (int k = 0; k < D / 64; ++k) {
-          float a[32], b[32];
-          o_load(k, a);           // columns [32 k, 32 k + 32)
-          o_load(k + D / 64, b);  // columns [D/2 + 32 k, D/2 + 32 k + 32)
-#pragma unroll
-          for (int i = 0; i < 32; ++i) {
-            const float other = __shfl_xor_sync(0xffffffffu, half ? a[i] : b[i], 16);
-            a[i] = (half ? b[i] : a[i]) + other;
-          }
-          if (dst) {
-            float* d = dst + half * (D / 2) + k * 32;
-#pragma unroll
-            for (int i = 0; i < 32; i += 4)
-              *reinterpret_cast<float4*>(d + i) = make_float4(a[i] * inv, a[i + 1] * inv, a[i + 2] * inv, a[i + 3] * inv);
-          }
-        }
-      } else {
-#pragma unroll 1
-        for (int k = 0; k < D / 32; ++k) {
           float o[32];
-          o_load(k, o);
-          if (dst) {
+          tmem_ld_16x64(t_lane + ((uint32_t)(16 * hf) << 16) + kTmemO + 64 * k, o);
+          if constexpr (kPair) {
+            float lo[32];
+            tmem_ld_16x64(t_lane + (16u << 16) + kTmemO + 64 * k, lo);
 #pragma unroll
-            for (int i = 0; i < 32; i += 4)
-              *reinterpret_cast<float4*>(dst + k * 32 + i) =
-                  make_float4(o[i] * inv, o[i + 1] * inv, o[i + 2] * inv, o[i + 3] * inv);
+            for (int i = 0; i < 32; ++i) o[i] += lo[i];
+          }
+          const int c = 64 * k + 2 * (lane % 4);
+#pragma unroll
+          for (int i = 0; i < 8; ++i) {
+            if (to_a >= 0)
+              *reinterpret_cast<float2*>(p.out_o + to_a * D + c + 8 * i) =
+                  make_float2(o[4 * i] * inv_a, o[4 * i + 1] * inv_a);
+            if (to_b >= 0)
+              *reinterpret_cast<float2*>(p.out_o + to_b * D + c + 8 * i) =
+                  make_float2(o[4 * i + 2] * inv_b, o[4 * i + 3] * inv_b);
           }
         }
       }
-      if (dst_lse) *dst_lse = (m_used + log2f(l)) * kLn2;
+      if (valid && half == 0) p.out_lse[to] = (m_used + log2f(l)) * kLn2;
     }
     if (!more) break;
     work = next;
