@@ -11,6 +11,7 @@ st_decode_attn, st_merge, st_release, ...) take a Pool as first argument;
 Pool's methods do the same work.
 """
 import ctypes
+import functools
 import os
 
 from ._build import LIB, build  # noqa: F401
@@ -173,10 +174,14 @@ class Pool:
         self._lib = L
         self._layers, self._q_heads, self._kv_heads, self._dim = n_layers, n_q_heads, n_kv_heads, head_dim
         if self.device is not None:
-            self._torch = torch
             self._raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
 
     # -- plumbing ---------------------------------------------------------
+    @functools.cached_property
+    def _torch(self):  # (a metadata-only pool needs it for its checks alone)
+        import torch
+        return torch
+
     def _check(self, st, what):
         if st != ST_OK:
             L = lib()

@@ -216,3 +216,19 @@ def test_fork_at_rejects_points_past_the_end(stlib):
         assert e.value.status == stlib.ST_ERR_INVALID
     (c,) = lp.fork_at(a, 0, 1)
     assert lp.block_table(c) == ([], 0)
+
+
+def test_metadata_pool_refuses_tensors_by_their_checks(stlib):
+    """The binding's checks answer on a metadata-only pool too: not a tensor,
+    or one that is not on the pool's device."""
+    import torch
+    lp = _meta(stlib, 16, 0)
+    a = lp.seq_create()
+    lp.append_kv([a], 3, None)
+    q, k = (torch.zeros(1, 1, h, 64, dtype=torch.bfloat16) for h in (4, 2))
+    for call in (lambda x, y: lp.decode_attn([a], x), lambda x, y: lp.decode_step([a], y, y, x)):
+        with pytest.raises(TypeError):
+            call(None, None)
+        with pytest.raises(ValueError):
+            call(q, k)
+    assert lp.block_table(a)[1] == 3
