@@ -112,7 +112,7 @@ __global__ void __launch_bounds__(kTableThreads) append_kernel(const AppendParam
       }
       const AppendBranch br = branches[b];
       const int pos = br.start + (row - br.row0);
-      const int32_t blk = p.n_table_blocks ? inl.pages[br.page0 + pos / kPageTokens - br.start / kPageTokens]
+      const int32_t blk = p.n_table_blocks ? inl.pages[inl.page0[b] + pos / kPageTokens - br.start / kPageTokens]
                                            : p.table[(int64_t)br.slot * p.max_pages + pos / kPageTokens];
       if ((uint64_t)blk >= (uint64_t)p.n_blocks) {
         atomicCAS(p.status, 0, kDevBadIndex);

@@ -40,7 +40,6 @@ struct AppendBranch {
   int32_t start;  // sequence length before this call
   int32_t row0;   // first of this branch's rows in the call's input
   int32_t n;      // rows appended to this branch
-  int32_t page0;  // with an inline page list: where the page of row `start` is in it
 };
 
 struct AppendParams {
@@ -157,6 +156,7 @@ struct InlineAppendPlan {
   AppendBranch branches[kInlineAppendBranches];
   CowCopy cows[kInlineCows];
   int32_t pages[kInlinePages];  // the pages of each branch's new rows
+  int32_t page0[kInlineAppendBranches];  // where the page of a branch's row `start` is in them
 };
 // Entries of one run that a block of a table refresh writes.
 constexpr int kTableThreads = 256;

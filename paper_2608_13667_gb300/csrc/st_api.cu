@@ -466,7 +466,7 @@ st_status do_append_rows(st_pool* P, const int* slots, const int32_t* counts, in
   brs.resize(n_br);
   int32_t row0 = 0;
   for (int i = 0; i < n_br; ++i) {
-    brs[i] = AppendBranch{slots[i], (int32_t)bp.slot(slots[i]).len, row0, counts[i], 0};
+    brs[i] = AppendBranch{slots[i], (int32_t)bp.slot(slots[i]).len, row0, counts[i]};
     row0 += counts[i];
   }
   std::vector<CowEvent>& cows = P->app_cows;
@@ -494,7 +494,7 @@ st_status do_append_rows(st_pool* P, const int* slots, const int32_t* counts, in
   if (refreshes) {
     int32_t at = 0;
     for (int i = 0; i < n_br; ++i) {
-      brs[i].page0 = at;
+      inl.page0[i] = at;
       const int32_t n = pages_of_rows(brs[i]);
       std::memcpy(inl.pages + at, bp.slot(slots[i]).table.data() + brs[i].start / kPageTokens, n * sizeof(int32_t));
       at += n;

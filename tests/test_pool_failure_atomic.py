@@ -98,3 +98,17 @@ def test_decode_calls_on_a_metadata_pool_change_nothing(stlib):
     assert L.st_decode_step(lp._h, arr, 1, None, None, None, None, None, None) == stlib.ST_ERR_STATE
     assert L.st_decode_attn(lp._h, arr, 1, None, None, None, None) == stlib.ST_ERR_STATE
     assert _state(lp, [a]) == before
+
+
+def test_append_plan_that_fills_a_slot(stlib):
+    # two sequences fewer than in the refused call above: 65536 records of
+    # 16 bytes and as many copies are a slot exactly
+    n = 65536
+    lp = _meta(stlib, n_blocks=70000, max_seqs=n)
+    main = lp.seq_create()
+    lp.append_kv([main], 5, None)
+    handles = [main] + lp.fork(main, n - 1)
+    lp.append_kv(handles, 1, None)
+    tables = [lp.block_table(h) for h in handles[:100] + handles[-100:]]
+    assert all(length == 6 and len(table) == 1 for table, length in tables)
+    assert len({table[0] for table, _ in tables}) == 200
