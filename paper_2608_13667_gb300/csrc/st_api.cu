@@ -390,12 +390,10 @@ TableRefresh stage_tables(st_pool* P, Plan* plan, int n_dirty, int* slot) {
   return t;
 }
 
-// Refresh the device copy of every block-table range the host changed.
-st_status flush_tables(st_pool* P, cudaStream_t s) {
+// Refresh the device copy of every block-table range the host changed (d).
+st_status flush_tables(st_pool* P, DirtyTables d, cudaStream_t s) {
   int slot = 0;
-  while (slot < P->pool->max_seqs()) {
-    const DirtyTables d = dirty_tables(*P->pool, slot);
-    if (d.runs == 0) return ST_OK;
+  while (d.runs > 0) {
     Plan plan;
     int ps;
     st_status st = acquire_plan(P, &plan, &ps);
@@ -407,6 +405,8 @@ st_status flush_tables(st_pool* P, cudaStream_t s) {
     if (st != ST_OK) return st;
     st = retire_plan(P, ps, s);
     if (st != ST_OK) return st;
+    if (t.n_values == d.values) break;
+    d = dirty_tables(*P->pool, slot);
   }
   return ST_OK;
 }
@@ -505,7 +505,7 @@ st_status do_append_rows(st_pool* P, const int* slots, const int32_t* counts, in
     int first = 0;
     refresh = stage_tables(P, &table_plan, dirty.runs, &first);
   } else {
-    st = flush_tables(P, s);
+    st = flush_tables(P, dirty, s);
     if (st != ST_OK) return poison(P, st);
   }
   if (defers) {
@@ -1090,7 +1090,7 @@ st_status decode_impl(st_pool* P, const std::vector<int>& slots, const void* q, 
                                   n_br * sizeof(int32_t)}) > kStageSlotBytes)
     return fail(P, ST_ERR_INVALID, "decode plan of %d items does not fit one plan slot", (int)items.size());
   // device tables that missed an upload would disagree with the host's
-  st_status st = flush_tables(P, s);
+  st_status st = flush_tables(P, dirty_tables(*P->pool), s);
   if (st != ST_OK) return poison(P, st);
 
   InlineDecodePlan inl;
