@@ -82,11 +82,18 @@
 //
 // A call with large groups launches their tiles first and the narrow items,
 // most of them the branches' own pages, right behind as their programmatic
-// dependents (beside_prev).  Those do not depend on the large tiles' results,
-// and by the time they start, every CTA of the large tiles has passed its own
-// wait: whatever was before both is complete.  So they skip the wait and run on
-// the SMs that the large tiles' last wave leaves idle; only the grid's last CTA
-// waits, at its end, so that what follows (the combine) sees both complete.
+// dependents (beside_prev).  Those do not depend on the large tiles' results
+// and run on the SMs that the large tiles' last wave leaves idle.  They start
+// once every CTA of the large tiles has passed its own wait, so whatever was
+// before both is complete; but only the wait makes a grid see what earlier
+// grids wrote, and theirs would be for the large tiles too.  So the first CTA of
+// the large tiles publishes a tag behind its wait, a release at device scope,
+// and every thread of a narrow CTA acquires it: what the first saw is then
+// visible to the second (the copies' proxy by a fence).  A CTA that finds
+// another value executes the wait.  The tag is another one in every call, and
+// the word is moved on when the narrow launch is through, so that a replayed
+// graph cannot find its own earlier tag.  The grid's last CTA waits at its end,
+// so that what follows (the combine) sees both complete.
 // 12 branches per group, 2 groups, 4 layers: 449 -> 420 us for the two launches;
 // 24 branches, 2 layers: 340 -> 315; one layer, 4 groups of 20: 118 -> 94.
 //
@@ -223,7 +230,11 @@ __global__ void __launch_bounds__(kThreads, 2)
   // allocation, and all of the set-up when the item is in the parameters.
   if (warp == kMmaWarp) tmem_alloc(tmem_slot, kTmemCols);
   const bool beside = !kWide && p.beside_prev;
-  if (p.items && !beside) griddep_wait();
+  auto wait_for_prev = [&] {
+    if constexpr (kWide) griddep_wait();
+    else narrow_wait(p);
+  };
+  if (p.items) wait_for_prev();
 
   // ---- what this CTA reads and for whom ------------------------------------------
   const int32_t* members = p.members ? p.members : inl.members;
@@ -264,7 +275,8 @@ __global__ void __launch_bounds__(kThreads, 2)
   __syncthreads();
   tc_fence_after_sync();
   const uint32_t tmem = *tmem_slot;
-  if (!p.items && !beside) griddep_wait();
+  if (!p.items) wait_for_prev();
+  if constexpr (kWide) publish_large_launch(p);
   griddep_launch_dependents();
 
   // The item after a role's n-th: written to slot n % 2 by the loader.  False
@@ -317,6 +329,9 @@ __global__ void __launch_bounds__(kThreads, 2)
       prefetch_tensormap(&kmap);
       prefetch_tensormap(&vmap);
     }
+    // the pages were written by ordinary stores; past a griddep_wait() that is
+    // settled, past an acquire alone the copies need the proxy fence
+    if (beside) fence_proxy_async_global();
     // lane 0 waits, for the warp
     auto wait0 = [&](uint64_t* bar, uint32_t parity) -> bool {
       int w = 1;
@@ -551,8 +566,12 @@ __global__ void __launch_bounds__(kThreads, 2)
     // kPersist the last CTA may be taken over before it starts: all wait, when
     // there is nothing left to run)
     if (beside && (kPersist || (blockIdx.x == gridDim.x - 1 && blockIdx.y == gridDim.y - 1 &&
-                                blockIdx.z == gridDim.z - 1)))
+                                blockIdx.z == gridDim.z - 1))) {
       griddep_wait();
+      // The word has served.  A replay of a captured call carries the same tag,
+      // which must not be found before the large launch of that replay publishes it.
+      if (lane == 0) st_release_gpu(p.large_word, p.large_tag + 1);
+    }
     return;
   }
   if (warp >= n_part) return;

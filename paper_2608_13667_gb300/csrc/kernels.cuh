@@ -112,7 +112,11 @@ struct AttnParams {
   int32_t slot, L0, T;     // merge only: main's slot, length before the append, thought rows
   int32_t hold_loads;      // test hook (ST_FLAG_HOLD_LOADS): the loader issues nothing
   int32_t item_base;       // decode: CTA x reads item item_base + x
-  int32_t beside_prev;     // decode: runs beside the kernel before it in the stream (attend_tc.cu)
+  int32_t beside_prev;     // decode: runs beside the large launch before it in the stream (attend_tc.cu)
+  // decode, a call with both: the large launches publish `tag` in *large_word
+  // once they are past their own wait, the narrow one looks for it (null: alone)
+  uint32_t* large_word;
+  uint32_t large_tag;
   int32_t keep_l2;         // decode: the launch's pages fit in L2; load them evict-normal so they stay
   const MergeItem* mitems; // batched merge: cluster x takes mitems[x] (slot, L0, T above unused)
   int32_t kv_split;        // merge: CTAs (a cluster) that share one row tile's keys
@@ -173,9 +177,43 @@ constexpr int kTableChunk = 4 * kTableThreads;
 // A dependent grid is launched only after every CTA of its predecessor has
 // signalled (or exited), so a waiting grid never keeps its predecessor's
 // CTAs off the SMs.
+//
+// One launch may run without that wait: the narrow decode items beside the
+// large tiles of the same call (AttnParams::beside_prev; attend_tc.cu).  It
+// reads and writes nothing that the large launches write, but all that came
+// before them, and the wait is what makes earlier grids' writes visible.  So
+// the large launches publish a word after their own wait
+// (publish_large_launch), and a narrow CTA that acquires it is synchronised
+// with everything before the large launches; one that does not see it executes
+// the wait (narrow_wait).  Nothing spins on the word.
 __device__ __forceinline__ void griddep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void griddep_launch_dependents() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+// Synchronisation through a word of global memory, between grids of one device:
+// what was visible to the releasing thread is visible to one that acquires the
+// value.
+__device__ __forceinline__ void st_release_gpu(uint32_t* p, uint32_t v) {
+  asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(__cvta_generic_to_global(p)), "r"(v) : "memory");
+}
+
+__device__ __forceinline__ uint32_t ld_acquire_gpu(const uint32_t* p) {
+  uint32_t v;
+  asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(__cvta_generic_to_global(p)) : "memory");
+  return v;
+}
+
+// Of a large decode launch, by every thread between its griddep_wait() and its
+// griddep_launch_dependents().
+__device__ __forceinline__ void publish_large_launch(const AttnParams& p) {
+  if (p.large_word && threadIdx.x == 0 && (blockIdx.x | blockIdx.y | blockIdx.z) == 0)
+    st_release_gpu(p.large_word, p.large_tag);
+}
+
+// Of the narrow decode launch, by every thread in place of griddep_wait().
+__device__ __forceinline__ void narrow_wait(const AttnParams& p) {
+  if (!p.beside_prev || ld_acquire_gpu(p.large_word) != p.large_tag) griddep_wait();
 }
 
 template <typename... KArgs, typename... Args>

@@ -292,6 +292,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   tc_fence_after_sync();
   const uint32_t tmem = *tmem_slot;
   griddep_wait();
+  if constexpr (kDecode) publish_large_launch(p);
   griddep_launch_dependents();
   // one merge: its row tiles, the last ones (most keys) first; a batch: one
   // work item per cluster (the host orders those longest first); a decode: one

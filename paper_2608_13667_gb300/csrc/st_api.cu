@@ -45,7 +45,7 @@ const char* const kKernelNames[kNumKernels] = {"table_update", "append_kv", "dec
 size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
 struct WorkspaceLayout {
-  size_t status = 0, tables = 0, staging = 0, part_o = 0, part_lse = 0, total = 0;
+  size_t status = 0, large_word = 0, tables = 0, staging = 0, part_o = 0, part_lse = 0, total = 0;
 };
 
 bool config_valid(const st_config* c, std::string* why) {
@@ -75,7 +75,8 @@ WorkspaceLayout layout_for(const st_config* c) {
   WorkspaceLayout w;
   size_t off = 0;
   w.status = off;
-  off = align_up(off + 64, 256);
+  w.large_word = off + 128;  // a sector of its own
+  off = align_up(off + 192, 256);
   w.tables = off;
   off = align_up(off + (size_t)c->max_seqs * c->max_pages * sizeof(int32_t), 256);
   w.staging = off;
@@ -151,6 +152,8 @@ struct st_pool {
   uint8_t* ws = nullptr;
   WorkspaceLayout lay;
   int32_t* d_status = nullptr;
+  uint32_t* d_large_word = nullptr;  // AttnParams::large_word
+  uint32_t large_tag = 0;            // the last call's: even, its own + 1 marks the launch as through
   int32_t* d_tables = nullptr;
   float* d_part_o = nullptr;
   float* d_part_lse = nullptr;
@@ -672,6 +675,7 @@ ST_API st_status st_pool_create(const st_config* cfg, void* k_pool, void* v_pool
   P->ws = static_cast<uint8_t*>(workspace);
   P->lay = layout_for(cfg);
   P->d_status = reinterpret_cast<int32_t*>(P->ws + P->lay.status);
+  P->d_large_word = reinterpret_cast<uint32_t*>(P->ws + P->lay.large_word);
   P->d_tables = reinterpret_cast<int32_t*>(P->ws + P->lay.tables);
   P->d_part_o = reinterpret_cast<float*>(P->ws + P->lay.part_o);
   P->d_part_lse = reinterpret_cast<float*>(P->ws + P->lay.part_lse);
@@ -1151,8 +1155,14 @@ st_status decode_impl(st_pool* P, const std::vector<int>& slots, const void* q, 
   const int n_pair = n_items - n_narrow - n_wide;
   st = run_kernel(P, kKDecode, bytes, flops, s, [&] {
     const InlineDecodePlan* ip = inline_plan ? &inl : nullptr;
-    // the large tiles first, the narrow items beside their last wave
+    // the large tiles first, the narrow items beside their last wave: these rely
+    // on the large launches to publish the tag after their own dependent wait
     AttnParams aw = ap;
+    aw.beside_prev = 0;
+    if (n_narrow > 0 && n_wide + n_pair > 0) {
+      aw.large_word = P->d_large_word;
+      aw.large_tag = P->large_tag += 2;
+    }
     aw.item_base = n_narrow;
     cudaError_t e = launch_decode_tc(P->kmap, P->vmap, aw, ip, n_wide, c.head_dim, true, s);
     if (e != cudaSuccess) return e;
@@ -1160,7 +1170,7 @@ st_status decode_impl(st_pool* P, const std::vector<int>& slots, const void* q, 
     e = launch_decode_pair(P->kmap, P->vmap, aw, ip, n_pair, c.head_dim, s);
     if (e != cudaSuccess) return e;
     aw.item_base = 0;
-    aw.beside_prev = n_wide > 0 || n_pair > 0 ? 1 : 0;
+    aw.beside_prev = n_wide + n_pair > 0 ? 1 : 0;
     return launch_decode_tc(P->kmap, P->vmap, aw, ip, n_narrow, c.head_dim, false, s);
   }, (n_narrow > 0 ? 1 : 0) + (n_wide > 0 ? 1 : 0) + (n_pair > 0 ? 1 : 0),
                   dp.reread_bytes + part_bytes);
