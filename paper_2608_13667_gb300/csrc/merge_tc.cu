@@ -101,10 +101,17 @@ constexpr int kThreads = 12 * 32;  // three warpgroups, for the register split
 constexpr int kSoftThreads = 8 * 32;
 // Where the softmax threads hold a row's 128 scores (kHold), the warpgroups'
 // registers are shared out anew, within what the block is launched with (168 a
-// thread): 192 + 192 + 120.
+// thread): 192 + 192 + 120.  setmaxnreg.inc waits without a limit for registers
+// that the block does not have, and the launch bounds only cap what the compiler
+// assigns, so pair_setup refuses a build with fewer before any launch.
 constexpr int kSoftRegs = 192, kOtherRegs = 120;
-static_assert(kSoftThreads * kSoftRegs + (kThreads - kSoftThreads) * kOtherRegs <= kThreads * 168,
-              "registers of a block");
+constexpr bool regs_suffice(int launch_regs) {  // registers a thread at launch
+  return launch_regs >= kOtherRegs &&
+         kSoftThreads * kSoftRegs + (kThreads - kSoftThreads) * kOtherRegs <= kThreads * launch_regs;
+}
+template <int D, bool kDecode>
+constexpr bool kSharesRegs = D == 128 && !kDecode;
+static_assert(regs_suffice(168) && !regs_suffice(167), "registers of a block");
 constexpr uint32_t kTmemCols = 512;
 constexpr uint32_t kTmemTile = 256, kTmemO = 128;  // per-tile column base, O offset within it
 constexpr float kRescaleThreshold = 8.f;           // log2 units
@@ -232,7 +239,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   using C = PairCfg<D>;
   constexpr int kKS = C::kKStages, kVS = C::kVStages;
   constexpr bool kMapped = !kDecode && kForm, kPersist = kDecode && kForm;
-  constexpr bool kHold = D == 128 && !kDecode;  // the softmax holds its scores (below)
+  constexpr bool kHold = kSharesRegs<D, kDecode>;  // the softmax holds its scores (below)
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw = smem_addr(smem_raw);
   uint8_t* base = smem_raw + ((1024u - (raw & 1023u)) & 1023u);
@@ -1043,6 +1050,12 @@ cudaError_t pair_setup(const PairSetup** out) {
     for (auto* k : {kernel, other}) {
       e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmemBytes);
       if (e != cudaSuccess) return e;
+      if (kSharesRegs<D, kDecode>) {
+        cudaFuncAttributes fa;
+        e = cudaFuncGetAttributes(&fa, k);
+        if (e != cudaSuccess) return e;
+        if (!regs_suffice(fa.numRegs)) return cudaErrorInvalidKernelImage;
+      }
     }
     if constexpr (!kDecode) {
       for (auto* k : {kernel, other}) {
