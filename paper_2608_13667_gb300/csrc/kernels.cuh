@@ -24,7 +24,7 @@ constexpr int32_t kDevTimeout = 5;
 
 struct TableRun {
   int64_t dst;    // slot * max_pages + first entry
-  int32_t count;  // entries
+  int32_t count;  // entries, at most kTableChunk
   int32_t src;    // offset into the values array
 };
 
@@ -60,7 +60,7 @@ struct AppendParams {
   const TableRun* runs;
   const int32_t* values;
   int32_t* table_out;
-  int32_t n_table_blocks, chunks_per_run;
+  int32_t n_table_blocks;  // one per run
 };
 
 // One unit of decode work: a run of pages of one block table, read for a set
@@ -162,7 +162,7 @@ struct InlineAppendPlan {
   int32_t pages[kInlinePages];  // the pages of each branch's new rows
   int32_t page0[kInlineAppendBranches];  // where the page of a branch's row `start` is in them
 };
-// Entries of one run that a block of a table refresh writes.
+// Entries that a run has at most; a block of a table refresh writes one run.
 constexpr int kTableThreads = 256;
 constexpr int kTableChunk = 4 * kTableThreads;
 
@@ -252,9 +252,9 @@ cudaError_t launch_chained_cluster(void (*kernel)(KArgs...), dim3 grid, dim3 blo
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<Args&&>(args)...);
 }
 
-// runs, values: readable by the device, here in pinned host memory; max_count: the longest run's.
+// runs, values: readable by the device, here in pinned host memory.
 cudaError_t launch_table_update(int32_t* table, const TableRun* runs, const int32_t* values, int n_runs,
-                                int max_count, cudaStream_t s);
+                                cudaStream_t s);
 // bytes rounded up to 16 from pinned host memory to the device; both 16-byte aligned.
 cudaError_t launch_plan_copy(void* dst, const void* src, size_t bytes, cudaStream_t s);
 cudaError_t launch_append(const AppendParams& p, const InlineAppendPlan* inl, int D, cudaStream_t s);

@@ -339,7 +339,7 @@ size_t plan_bytes(std::initializer_list<size_t> parts) {
 
 // Block-table ranges the host has changed and the device has not seen.
 struct DirtyTables {
-  int runs = 0;
+  int64_t runs = 0;  // of at most kTableChunk entries
   size_t values = 0;
 };
 
@@ -348,7 +348,7 @@ DirtyTables dirty_tables(const BlockPool& bp, int first_slot = 0) {
   for (int i = first_slot; i < bp.max_seqs(); ++i) {
     const SeqSlot& ss = bp.slot(i);
     if (!ss.live || ss.dirty_hi <= ss.dirty_lo) continue;
-    ++d.runs;
+    d.runs += (ss.dirty_hi - ss.dirty_lo + kTableChunk - 1) / kTableChunk;
     d.values += (size_t)(ss.dirty_hi - ss.dirty_lo);
   }
   return d;
@@ -359,13 +359,13 @@ struct TableRefresh {
   const TableRun* runs = nullptr;  // device addresses
   const int32_t* values = nullptr;
   int n_runs = 0;
-  size_t n_values = 0, longest = 0;
+  size_t n_values = 0;
 };
 
-TableRefresh stage_tables(st_pool* P, Plan* plan, int n_dirty, int* slot) {
+TableRefresh stage_tables(st_pool* P, Plan* plan, int64_t n_dirty, int* slot) {
   BlockPool& bp = *P->pool;
   // runs first (bounded count), then values
-  const int max_runs = std::min(n_dirty, 4096);
+  const int max_runs = (int)std::min<int64_t>(n_dirty, 4096);
   const TableRun* unused_runs;
   TableRun* runs = plan->alloc<TableRun>(max_runs, &unused_runs);
   const size_t vals_cap = (plan->cap - plan->off - 64) / sizeof(int32_t);
@@ -374,20 +374,19 @@ TableRefresh stage_tables(st_pool* P, Plan* plan, int n_dirty, int* slot) {
   TableRefresh t;
   t.runs = on_device(P, runs);
   t.values = on_device(P, vals);
-  for (; *slot < bp.max_seqs() && t.n_runs < max_runs; ++*slot) {
+  for (; *slot < bp.max_seqs(); ++*slot) {
     SeqSlot& ss = bp.slot_mut(*slot);
     if (!ss.live || ss.dirty_hi <= ss.dirty_lo) continue;
-    const size_t cnt = (size_t)(ss.dirty_hi - ss.dirty_lo);
-    const size_t room = vals_cap - t.n_values;
-    if (room == 0) break;
-    const size_t take = std::min(cnt, room);
-    runs[t.n_runs] = TableRun{(int64_t)*slot * bp.max_pages() + ss.dirty_lo, (int32_t)take, (int32_t)t.n_values};
+    const size_t take = std::min({(size_t)(ss.dirty_hi - ss.dirty_lo), (size_t)(max_runs - t.n_runs) * kTableChunk,
+                                  vals_cap - t.n_values});
     std::memcpy(vals + t.n_values, ss.table.data() + ss.dirty_lo, take * sizeof(int32_t));
+    const int64_t dst = (int64_t)*slot * bp.max_pages() + ss.dirty_lo;
+    for (size_t i = 0; i < take; i += kTableChunk)
+      runs[t.n_runs++] = TableRun{dst + (int64_t)i, (int32_t)std::min<size_t>(kTableChunk, take - i),
+                                  (int32_t)(t.n_values + i)};
     t.n_values += take;
-    t.longest = std::max(t.longest, take);
-    ++t.n_runs;
     ss.dirty_lo += (int32_t)take;
-    if (ss.dirty_lo < ss.dirty_hi) break;  // slot only partly uploaded: continue it next round
+    if (ss.dirty_lo < ss.dirty_hi) break;  // full: the rest of this slot's range goes with the next staging slot
     ss.dirty_lo = ss.dirty_hi = 0;
   }
   return t;
@@ -403,7 +402,7 @@ st_status flush_tables(st_pool* P, DirtyTables d, cudaStream_t s) {
     if (st != ST_OK) return st;
     const TableRefresh t = stage_tables(P, &plan, d.runs, &slot);
     st = run_kernel(P, kKTable, (double)t.n_values * 8 + t.n_runs * 16, 0, s, [&] {
-      return launch_table_update(P->d_tables, t.runs, t.values, t.n_runs, (int)t.longest, s);
+      return launch_table_update(P->d_tables, t.runs, t.values, t.n_runs, s);
     });
     if (st != ST_OK) return st;
     st = retire_plan(P, ps, s);
@@ -556,8 +555,7 @@ st_status do_append_rows(st_pool* P, const int* slots, const int32_t* counts, in
     ap.runs = refresh.runs;
     ap.values = refresh.values;
     ap.table_out = P->d_tables;
-    ap.chunks_per_run = (int32_t)((refresh.longest + kTableChunk - 1) / kTableChunk);
-    ap.n_table_blocks = refresh.n_runs * ap.chunks_per_run;
+    ap.n_table_blocks = refresh.n_runs;
   }
   // algorithmic: the new rows read and written once; the copy-on-write rows
   // are the bookkeeping's own traffic

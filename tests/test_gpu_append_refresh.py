@@ -61,3 +61,34 @@ def test_forks_not_appended_to_are_refreshed_too(stlib):
     aux = run.fork(m, 4)                    # their tables go up with the append below
     run.append([other], 30, ("rows",))
     _check(run, [other] + aux)
+
+
+@pytest.mark.parametrize("pages,n_long,n_short,rows", [
+    (1023, 1, 3, 1), (1024, 1, 3, 1), (1025, 1, 3, 1), (2050, 2, 40, 1),   # runs of 1024 entries at most
+    (1025, 1, 3, 0), (5000, 1, 300, 0),                                    # the refresh as a launch of its own
+    (1030, 520, 30, 0), (1030, 520, 30, 1),                                # more entries than a staging slot holds
+    (4, 4200, 0, 1),                                                       # more runs than a staging slot's list
+])
+def test_device_tables_of_long_and_short_ranges(stlib, pages, n_long, n_short, rows):
+    """Every live table on the device, entry by entry: ranges longer than a run
+    beside short ones, refreshed by an append (rows > 0) or ahead of a decode."""
+    import torch
+    n = n_long + n_short + 8
+    w = Workload(name="ranges", n_layers=1, n_q_heads=1, n_kv_heads=1, head_dim=64, n_blocks=pages + 64, seed=74)
+    run = Run(w, max_seqs=n, max_decode_branches=2, max_splits=4, max_pages=pages + 8)
+    long, short, x = run.create(), run.create(), run.create()
+    run.append([long], 16 * pages - 3, ("long",))
+    run.append([short], 20, ("short",))
+    run.append([x], 5, ("x",))
+    run.decode([x], ("q",))                               # every table so far is on the device
+    live = [long, short, x] + run.fork(short, n_short // 2) + run.fork(long, n_long) + run.fork(short, n_short - n_short // 2)
+    if rows:
+        run.append([x], rows, ("rows",))
+    else:
+        run.decode([x], ("q",))
+    run.pool.sync()
+    tables = run.pool.workspace[256:256 + 4 * n * (pages + 8)].view(torch.int32).view(n, pages + 8).cpu()
+    for r in live:
+        h = run.handle[r]
+        table, _ = run.pool.block_table(h)
+        assert tables[h & 0xffffffff, :len(table)].tolist() == table, r
