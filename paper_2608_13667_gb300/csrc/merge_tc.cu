@@ -85,6 +85,7 @@
 #include <algorithm>
 #include <mutex>
 #include <type_traits>
+#include <vector>
 
 #include "kernels.cuh"
 #include "ptx.cuh"
@@ -169,6 +170,11 @@ __host__ __device__ constexpr int merge_parts(int all_tiles, int cluster) {
 struct MergeSplitCost {
   int parts;
   float total, longest;  // of its CTAs together, of one of them
+};
+
+// Row tiles of a launch that cost the same.
+struct MergeTileKind {
+  int all_tiles, rows, n;
 };
 
 // A decode's run of pages of a fork group, for one KV head of one layer.
@@ -1109,19 +1115,31 @@ cudaError_t launch_merge_t(const CUtensorMap& km, const CUtensorMap& vm, AttnPar
   const PairSetup* ps = nullptr;
   cudaError_t e = pair_setup<D, false>(&ps);
   if (e != cudaSuccess) return e;
-  // Estimated time of `layers` layers in clusters of n: waves of CTAs of average
-  // length, or the longest CTA if that is more.
-  auto estimate = [&](int n, int layers) {
-    int64_t ctas = 0;
-    float total = 0.f, longest = 0.f;
+  // The launch's row tiles, neighbours of equal cost counted together: a batch's
+  // come in the order of their keys, and the estimates below go over them up to
+  // 32 times (one by one, the call of 600 sequences of a row each took 33 us more, that of
+  // 32 of 150 rows 5 of 99).
+  std::vector<MergeTileKind> kinds;
+  auto list_kinds = [&] {
     for (int i = 0; i < n_items; ++i) {
       const int T = host_items ? host_items[i].T : p.T, L0 = host_items ? host_items[i].L0 : p.L0;
       const int row_base = host_items ? host_items[i].row_base : i * 2 * kTileRows;
       const int rows = std::min(2 * kTileRows, T * p.G - row_base);
       const int keys = L0 + (row_base + rows - 1) / p.G + 1;
-      const MergeSplitCost c = merge_tile_cost((keys + kKeys - 1) / kKeys, rows, n);
-      ctas += c.parts;
-      total += c.total;
+      const MergeTileKind k{(keys + kKeys - 1) / kKeys, rows <= kTileRows ? kTileRows : 2 * kTileRows, 1};
+      if (!kinds.empty() && kinds.back().all_tiles == k.all_tiles && kinds.back().rows == k.rows) ++kinds.back().n;
+      else kinds.push_back(k);
+    }
+  };
+  // Estimated time of `layers` layers in clusters of n: waves of CTAs of average
+  // length, or the longest CTA if that is more.
+  auto estimate = [&](int n, int layers) {
+    int64_t ctas = 0;
+    float total = 0.f, longest = 0.f;
+    for (const MergeTileKind& k : kinds) {
+      const MergeSplitCost c = merge_tile_cost(k.all_tiles, k.rows, n);
+      ctas += (int64_t)c.parts * k.n;
+      total += c.total * k.n;
       longest = std::max(longest, c.longest);
     }
     const int64_t waves = (ctas * p.Hkv * layers + ps->resident[n] - 1) / ps->resident[n];
@@ -1148,6 +1166,7 @@ cudaError_t launch_merge_t(const CUtensorMap& km, const CUtensorMap& vm, AttnPar
   int split[2] = {1, 1}, layers[2] = {p.L, 0};
   const int64_t sms = ps->resident[1], per_layer = (int64_t)n_items * p.Hkv, total = per_layer * p.L;
   if (total < 8 * sms) {
+    list_kinds();
     float time;
     split[0] = best_split(p.L, &time);
     // A few whole waves and a rest: the layers of the whole waves as they are,
