@@ -11,7 +11,6 @@ st_decode_attn, st_merge, st_release, ...) take a Pool as first argument;
 Pool's methods do the same work.
 """
 import ctypes
-import functools
 import os
 
 from ._build import LIB, build  # noqa: F401
@@ -126,6 +125,17 @@ class _SeqArrays:
         return self._val
 
 
+class _LazyTorch:
+    """torch for a metadata-only pool, whose checks alone need it: imported when
+    they do.  (A cached_property for it writes to the instance's __dict__, which
+    makes every attribute access of that pool slower: 600 releases 256 us with a
+    plain attribute, 291 so, 600 forks 1050 and 1085.)"""
+
+    def __getattr__(self, name):
+        import torch
+        return getattr(torch, name)
+
+
 class Pool:
     """A KV block pool on one GPU (or metadata-only with device=None).
 
@@ -175,13 +185,11 @@ class Pool:
         self._layers, self._q_heads, self._kv_heads, self._dim = n_layers, n_q_heads, n_kv_heads, head_dim
         if self.device is not None:
             self._raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+            self._torch = torch
+        else:
+            self._torch = _LazyTorch()
 
     # -- plumbing ---------------------------------------------------------
-    @functools.cached_property
-    def _torch(self):  # (a metadata-only pool needs it for its checks alone)
-        import torch
-        return torch
-
     def _check(self, st, what):
         if st != ST_OK:
             L = lib()
