@@ -63,8 +63,10 @@
 // commit that announces S_t(j) also covers O_t += P_t(j-1) V_{j-1}, so the
 // softmax may rescale O_t as soon as it sees S_t(j).
 //
-// Synchronisation (every wait bounded; a wait that runs out sets the status
-// word and the CTA winds down):
+// Synchronisation (every wait on these is bounded; one that runs out sets the
+// status word and the CTA winds down.  A cluster's CTAs meet at two cluster
+// barriers, whose wait has no limit: it ends because every thread of every CTA
+// gets there, whatever ran out before):
 //   k_full / k_empty, v_full / v_empty   ring slots (TMA bytes / MMA commit)
 //   s_full[t]      S_t of the stage is complete                 (MMA commit)
 //   p_full[t][h]   P_t of keys [64 h, 64 h + 64) is in TMEM     (128 arrivals)
