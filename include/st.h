@@ -222,7 +222,10 @@ ST_API st_status st_merge(st_pool* pool, st_seq main, int n_tok, const void* q, 
  * rules as st_append_kv; the pages are taken as if the sequences were
  * appended one after another) and run through the causal prefill of
  * st_merge: row r of sequence i attends over its rows [0, L0_i + r], L0_i =
- * its length before the call.  One launch covers every sequence.
+ * its length before the call.  One launch covers every sequence.  How a
+ * sequence's keys are split among CTAs depends on the whole launch, so the
+ * same rows in another batch, or in st_merge, may differ in their last bits;
+ * the same call over the same lengths gives the same bits.
  * n_tok:  host int32 [n_seq], each >= 0 (0: the sequence is left unchanged)
  * rows are packed in sequence order, R = sum of n_tok:
  * q: bf16 [n_layers][R][n_q_heads][head_dim];

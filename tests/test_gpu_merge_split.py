@@ -3,10 +3,11 @@ most 128 rows, whose two halves of the tensor memory take the stages in turn:
 against the float64 oracle at the sizes where a part, a stage or a tile begins
 or ends.  A stage is 128 keys and a part at least 4 stages."""
 import pytest
+import torch
 
 from fg_harness import Run, compare
 from oracle import attention as A
-from workloads import Workload
+from workloads import Workload, kv_rows, queries
 
 pytestmark = pytest.mark.gpu
 
@@ -93,3 +94,37 @@ def test_short_last_tile_behind_the_others(stlib, D, ctx, T):
     # 280, 520 and 340 stacked rows in 3 layers of 8 heads: the last tile of 24, 8
     # and 84 rows comes behind the others of every head and layer, whole or split
     _merge(D, 32, 8, ctx, T, L=3)
+
+
+def test_rows_merged_alone_and_among_others(stlib):
+    """How a row tile's keys are split depends on what else is in the launch, so
+    the same rows merged alone and in a batch may differ in their last bits, each
+    within the tolerance.  The same call gives the same bits."""
+    n, ctx, T = 16, 9000, 20
+    w = Workload(name="split_among", n_layers=1, n_q_heads=32, n_kv_heads=8, head_dim=128,
+                 n_blocks=n * ((ctx + T) // 16 + 2), seed=54)
+    outs = []
+    for batch, seed in ((True, 1), (True, 2), (False, 1)):
+        run = Run(w, max_seqs=n, max_decode_branches=1, max_splits=2, pool_seed=seed)
+        rids = [run.create() for _ in range(n)]
+        for i, r in enumerate(rids):
+            run.append([r], ctx, ("ctx", i))
+        if batch:
+            q, o, lse, L0 = run.prefill_batch(rids, [T] * n, ("rows",))
+        else:                               # the last sequence's rows of the batch by themselves
+            k, v = kv_rows(w, ("rows",), n * T, device="cuda")
+            q = queries(w, ("prefill_q", "rows"), n * T, device="cuda")
+            rows = slice((n - 1) * T, n * T)
+            o, lse = run.pool.merge(run.handle[rids[-1]], q[:, rows].contiguous(), k[:, rows].contiguous(),
+                                    v[:, rows].contiguous())
+        run.pool.sync()
+        outs.append((o.cpu(), lse.cpu()))
+        if len(outs) == 1:
+            ctx_k, ctx_v = run.context(rids[-1], 0)
+            o_ref, l_ref = A.merge_prefill(q[0, (n - 1) * T:].cpu(), ctx_k, ctx_v, ctx)
+        run.pool.close()
+    (o1, l1), (o2, l2), (o3, l3) = outs
+    assert torch.equal(o1, o2) and torch.equal(l1, l2)
+    assert not torch.equal(o1[:, (n - 1) * T:], o3)      # other parts, another order of the sums
+    compare(o1[0, (n - 1) * T:], l1[0, (n - 1) * T:], o_ref, l_ref, "among others")
+    compare(o3[0], l3[0], o_ref, l_ref, "alone")
