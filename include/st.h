@@ -252,7 +252,8 @@ ST_API st_status st_prefill_batch(st_pool* pool, const st_seq* seqs, int n_seq, 
  * out_src:  device int32 [n_br * stride] or NULL: b * stride + position of
  *           each harvested token in its branch's stream
  * out_atoms: device int32 [n_br] or NULL: atoms kept per branch
- * out_count: device int32 [1]
+ * out_count: int32 [1] that the device can write: device memory, or pinned host
+ *           memory, which can be read once the stream has passed the call
  * n_br <= 32, 0 <= cap <= 64, open_id != close_id.  Runs on `stream`; no pool
  * is needed. */
 ST_API st_status st_harvest(const int32_t* streams, int stride, const int32_t* lens, int n_br,
@@ -282,7 +283,11 @@ ST_API st_status st_sync(st_pool* pool, void* stream);
 /* Kernel accounting.  Launch counts are always kept; with timing enabled
  * (st_profile_enable(pool, 1)) each launch is bracketed by CUDA events on
  * its stream.  st_profile_read synchronises, fills up to cap records and
- * resets the counters. */
+ * resets the counters.  Kinds: table_update (block-table refreshes in a launch
+ * of their own, and the copies of plans too large for a kernel's parameters
+ * from the staging ring to the device, read and written bytes each), append_kv
+ * (a small append refreshes the tables itself, as overhead_bytes),
+ * decode_partial, lse_combine, merge_prefill. */
 typedef struct {
   char name[32];
   int64_t launches;
@@ -295,7 +300,8 @@ typedef struct {
   double overhead_bytes; /* bytes moved beyond the algorithmic ones: split-KV
                             partials (written by the decode, read by the
                             combine), second reads of a split fork family's
-                            shared pages, copy-on-write rows */
+                            shared pages, copy-on-write rows, table entries
+                            that an append refreshes */
 } st_kernel_stat;
 ST_API st_status st_profile_enable(st_pool* pool, int enable);
 ST_API st_status st_profile_read(st_pool* pool, st_kernel_stat* out, int cap, int* n);

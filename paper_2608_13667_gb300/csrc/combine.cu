@@ -25,7 +25,7 @@ namespace {
 // 160 rows: from the wait for the decode to the last write 3.1 us with one warp
 // and 16 loads in flight, 1.3 with four).  All index arithmetic comes ahead of that wait, in 32 bits.
 constexpr int kBatch = 8;
-constexpr int kFewRows = 152 * 16;  // rows of a small launch
+constexpr int kFewRows = 152 * 16;  // rows of a small launch: one block each on the 152 SMs of this part
 
 template <int D, int kWarps>
 __global__ void __launch_bounds__(128) combine_kernel(const CombineParams p, const __grid_constant__ InlineSplits inl) {

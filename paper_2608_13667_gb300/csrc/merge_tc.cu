@@ -1100,10 +1100,17 @@ const InlineDecodePlan kNoInline{};
 
 // Cost of a row tile's CTAs in a launch of clusters of `split`.
 MergeSplitCost merge_tile_cost(int all_tiles, int n_rows, int split) {
-  // microseconds, measured: a stage of 128 keys for 256 rows and for up to 128
-  // (the tiles taking the stages in turn), a CTA's start and end, the exchange
-  // (a merge of 183 stages took 352, 187, 105, 62 and 50 us in 1, 2, 4, 8 and
-  // 12 parts)
+  // microseconds: a stage of 128 keys for 256 rows and for up to 128 (the tiles
+  // taking the stages in turn), a CTA's start and end, the exchange.  The stages
+  // and the exchange are as measured at D = 128 (a merge of 183 stages: 344, 182,
+  // 99, 58 and 47 us in 1, 2, 4, 8 and 12 parts).  A CTA's start and end take about
+  // half of kCta since Q comes in by asynchronous copies and rows with one source
+  // leave through their warp; the value stays, because with the measured 5 (and 11
+  // for the exchange) the model left tiles of a few stages whole that two parts do
+  // faster (9 stages: 31.2 us in the one part it chose, 26.6 in two).  D = 64 has no constants of its own:
+  // of 17 shapes the choice was within 7% of the best of 16 sizes in 16, never
+  // behind one part, and 15% behind two parts in one (200 rows onto 9000 in 8
+  // layers: 262 and 228 us).
   constexpr float kStage = 1.9f, kDualStage = 1.15f, kCta = 10.f, kExchange = 6.f;
   const int parts = merge_parts(all_tiles, split);
   const float stage = n_rows <= kTileRows ? kDualStage : kStage;
@@ -1147,9 +1154,9 @@ cudaError_t launch_merge_t(const CUtensorMap& km, const CUtensorMap& vm, AttnPar
     const int64_t waves = (ctas * p.Hkv * layers + ps->resident[n] - 1) / ps->resident[n];
     return std::max(longest, waves * total / ctas);
   };
-  // CTAs per row tile: the size with the least estimate.  Over 19 shapes and 12
-  // sizes the choice was within 6% of the best one measured (10 parts for 24 row
-  // tiles, say, need two waves and take 114 us, where 5 take 93).
+  // CTAs per row tile: the size with the least estimate.  At D = 128 the choice was
+  // within 6% of the best of 16 sizes on every shape measured (10 parts for 24 row
+  // tiles, say, need two waves and take 105 us, where 5 take 87); D = 64: above.
   auto best_split = [&](int layers, float* time) {
     int split = 1;
     *time = estimate(1, layers);
