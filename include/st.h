@@ -296,7 +296,8 @@ typedef struct {
   double flops;        /* algorithmic floating-point operations */
   int64_t kernels;     /* device kernels launched (a decode call with several tile
                           shapes launches one for each; a merge whose last
-                          layers are split among more CTAs launches two) */
+                          layers are split among more CTAs launches two; so
+                          does an append that writes over rows it copies) */
   double overhead_bytes; /* bytes moved beyond the algorithmic ones: split-KV
                             partials (written by the decode, read by the
                             combine), second reads of a split fork family's

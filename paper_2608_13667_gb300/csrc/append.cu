@@ -56,7 +56,10 @@ __global__ void __launch_bounds__(256) plan_copy_kernel(uint4* __restrict__ dst,
 // One thread moves 16 bytes (8 bf16).  Index space: copy-on-write chunks
 // first (n_cow x L x Hkv x 16 rows x D/8, rows past the copy length idle),
 // then the appended rows in the input's own order [L][n_rows][Hkv][D/8];
-// row r belongs to the branch whose [row0, row0 + n) holds it.  A small append
+// row r belongs to the branch whose [row0, row0 + n) holds it.  Copies and rows of
+// a launch touch different rows of the pool; where a call's would not (the last
+// holder of a page, forked from inside it, writes in place over rows that others
+// copy), the host launches the copies first and the rows behind them.  A small append
 // that also changes the tables (new pages, or a fork's whole table) refreshes
 // them in its first blocks and takes its rows' pages from the parameters, one
 // launch and one hand-over less in the chain to the attention kernel (a merge

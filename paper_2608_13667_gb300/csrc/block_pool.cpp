@@ -79,6 +79,7 @@ bool BlockPool::fork_at(int parent, int64_t length, int n_aux, int* out) {
   if (found < n_aux) return false;
   const SeqSlot& src = slots_[parent];
   const size_t n_pages = (size_t)((length + page_ - 1) / page_);
+  if (length % page_ != 0 && length < src.len && n_aux > 0) cut_forks_ = true;
   for (int a = 0; a < n_aux; ++a) {
     SeqSlot& s = slots_[out[a]];
     s.live = true;

@@ -58,6 +58,10 @@ class BlockPool {
   // Fork from the parent's first `length` rows (0 <= length <= parent length):
   // the children take the first ceil(length / page) table entries.
   bool fork_at(int parent, int64_t length, int n_aux, int* out);
+  // Whether a child was ever forked from inside a page that its parent has more
+  // rows in: holders of a shared page may then differ in how many of its rows
+  // are theirs.
+  bool cut_forks() const { return cut_forks_; }
   // Pages an append of n_tok rows to `slot` takes from the free list.
   int64_t pages_needed(int slot, int64_t n_tok) const;
   // Would the table outgrow max_pages?
@@ -86,6 +90,7 @@ class BlockPool {
   int64_t head_ = 0, free_count_ = 0;
   std::vector<SeqSlot> slots_;
   int32_t next_family_ = 0;
+  bool cut_forks_ = false;
 };
 
 }  // namespace st

@@ -420,6 +420,31 @@ int32_t pages_of_rows(const AppendBranch& b) {
   return b.n > 0 ? (b.start + b.n - 1) / kPageTokens - b.start / kPageTokens + 1 : 0;
 }
 
+// Whether a call (its tables changed already) writes rows into a page that it
+// also copies these rows from.  The last holder of a shared page writes in place,
+// after the others' copies in the order of the call; where it was forked from
+// inside the page it starts below the end of what they copy.
+bool writes_copied_rows(const BlockPool& bp, const int* slots, const std::vector<AppendBranch>& brs,
+                        const std::vector<CowEvent>& cows) {
+  if (cows.empty() || !bp.cut_forks()) return false;
+  std::vector<std::pair<int32_t, int32_t>> sources;  // page and rows copied from it
+  for (const CowEvent& c : cows) sources.emplace_back(c.src_block, c.rows);
+  std::sort(sources.begin(), sources.end());
+  size_t copied = 0;  // copies come in the order of their branches
+  for (size_t i = 0; i < brs.size(); ++i) {
+    const int32_t off = brs[i].start % kPageTokens;
+    if (brs[i].n == 0 || off == 0) continue;
+    const int32_t page = bp.slot(slots[i]).table[brs[i].start / kPageTokens];
+    if (copied < cows.size() && cows[copied].dst_block == page) {
+      ++copied;
+      continue;
+    }
+    const auto more = std::upper_bound(sources.begin(), sources.end(), std::make_pair(page, off));
+    if (more != sources.end() && more->first == page) return true;
+  }
+  return false;
+}
+
 // Validates and performs an append (shared by st_append_kv, st_merge and
 // st_prefill_batch).  Appends counts[i] rows to slots[i], in order (the same
 // page allocation as appending to each sequence in turn); k, v: [L][sum of
@@ -562,8 +587,20 @@ st_status do_append_rows(st_pool* P, const int* slots, const int32_t* counts, in
   const double row_bytes = (double)c.n_layers * c.n_kv_heads * c.head_dim * 2 * 2;
   double cow_rows = 0;
   for (auto& e : cows) cow_rows += e.rows;
-  st = run_kernel(P, kKAppend, row_bytes * (double)n_rows * 2, 0, s,
-                  [&] { return launch_append(ap, inline_plan ? &inl : nullptr, c.head_dim, s); }, 1,
+  // one launch copies and writes; two where the rows would go over what is copied
+  const bool copies_first = writes_copied_rows(bp, slots, brs, cows);
+  st = run_kernel(P, kKAppend, row_bytes * (double)n_rows * 2, 0, s, [&] {
+    const InlineAppendPlan* ip = inline_plan ? &inl : nullptr;
+    if (copies_first) {
+      AppendParams copies = ap;
+      copies.n_rows = 0;
+      const cudaError_t e = launch_append(copies, ip, c.head_dim, s);
+      if (e != cudaSuccess) return e;
+      ap.n_cow = 0;
+      ap.n_table_blocks = 0;  // refreshed by the first
+    }
+    return launch_append(ap, ip, c.head_dim, s);
+  }, copies_first ? 2 : 1,
                   row_bytes * cow_rows * 2 + (double)refresh.n_values * 8 + refresh.n_runs * 16);
   if (st != ST_OK) {
     if (table_slot >= 0) drop_plan(P, table_slot);
