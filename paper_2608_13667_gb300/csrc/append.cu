@@ -1,11 +1,12 @@
 // Block-table refresh and the KV append (scatter + copy-on-write).
 //
 // The host owns the allocator; the device keeps a copy of every live block
-// table.  An append call first refreshes the table entries the host changed
-// (table_update), then one launch of append_kv performs the call's
-// copy-on-write page copies and writes its new rows.  The two parts of
-// append_kv never touch the same row: a copy fills rows [0, off) of a fresh
-// page and the appended rows start at row off, so they need no ordering.
+// table.  An append call refreshes the table entries the host changed (in its
+// own launch where it is small, else by table_update ahead of it), performs the
+// call's copy-on-write page copies and writes its new rows.  A copy fills rows
+// [0, off) of a fresh page whose own rows start at row off, so the two need no
+// ordering in one launch, except where rows go in place over what is copied
+// (below).
 #include "kernels.cuh"
 
 namespace st {
